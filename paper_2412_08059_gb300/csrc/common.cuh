@@ -247,15 +247,20 @@ __device__ __forceinline__ bool mbar_try_wait(unsigned long long* bar, uint32_t 
   return done != 0;
 }
 // Bounded wait for the completion of the phase with the given parity.
-// Returns false on timeout (status set) or when *stop becomes non-zero.
+// Returns false on timeout (status set) or when *stop becomes non-zero.  A
+// try_wait that finds the phase open suspends the thread for microseconds
+// before it gives up, so *stop is read after every one: read after every
+// 64th, the producer left its kernel 0.25 ms after the consumers (measured
+// at every size: 0.25 ms between the end of the iterations and the end of
+// the call; 64 x 64 grid, fixed eps1: 2.96 ms a solve before, 2.45 ms after).
 __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, uint32_t parity, Ctl* ctl,
                                           const volatile int* stop) {
   if (mbar_try_wait(bar, parity)) return true;
   const unsigned long long t0 = globaltimer();
   unsigned spins = 0;
   while (!mbar_try_wait(bar, parity)) {
+    if (stop && *stop) return false;
     if ((++spins & 63u) == 0) {
-      if (stop && *stop) return false;
       if (globaltimer() - t0 > (unsigned long long)ctl->timeout_ns) {
         set_status(ctl, MPCG_ERR_TIMEOUT);
         return false;
