@@ -36,7 +36,9 @@ struct BlockBfs {
   int32_t* qs[4];    // shared queue heads: A even, A odd, B even, B odd (cap entries)
   int32_t* qg[4];    // global queues of n entries (entries at index >= cap)
   int cap;
-  int* cnt;          // shared: A sizes [0..2] and B sizes [3..5] by level mod 3, [6] scratch
+  int* cnt;          // shared: A sizes [0..2] and B sizes [3..5] by level mod 3, [6] scratch,
+                     // [7] set when the search is to end
+  Ctl* poll;         // when set: the search ends on an error or the caller's cancel word
 };
 
 // Partition of a block's shared buffer (bytes, 16-aligned base) for n
@@ -49,6 +51,7 @@ static __device__ BlockBfs block_bfs_layout(const int32_t* rp, const int32_t* co
   b.rp = rp;
   b.col = col;
   b.n = n;
+  b.poll = nullptr;
   const int words = (n + 31) >> 5;
   b.cnt = reinterpret_cast<int*>(smem);
   unsigned char* p = smem + 64;
@@ -119,7 +122,7 @@ static __device__ BlockBfsOut block_bfs2(const BlockBfs& b, int srcA, int srcB) 
     b.vis[0][i] = 0u;
     b.vis[1][i] = 0u;
   }
-  if (tid < 7) b.cnt[tid] = 0;
+  if (tid < 8) b.cnt[tid] = 0;
   __syncthreads();
   if (tid == 0) {
     b.vis[0][srcA >> 5] |= 1u << (srcA & 31);
@@ -148,6 +151,14 @@ static __device__ BlockBfsOut block_bfs2(const BlockBfs& b, int srcA, int srcB) 
       }
     }
     if (sa == 0 && sb == 0) break;
+    if (b.poll && (level & 255) == 255) {
+      if (tid == 0 && (volatile_status(b.poll) != 0 || poll_cancel(b.poll))) b.cnt[7] = 1;
+      __syncthreads();
+      if (*reinterpret_cast<volatile int*>(&b.cnt[7])) {
+        o.reached = -1;
+        break;
+      }
+    }
     o.reached += sa;
     if (sa) {
       o.la = level;
@@ -236,7 +247,7 @@ static __device__ BlockBfsOut block_bfs2(const BlockBfs& b, int srcA, int srcB) 
     }
     __syncthreads();
   }
-  return o;  // the loop ends only after A has ended, so o.t is set
+  return o;  // unless stopped, the loop ends only after A has ended, so o.t is set
 }
 
 // 2BFS of a connected graph in one block.  Returns false (in every thread)
@@ -251,6 +262,7 @@ static __device__ bool block_pseudo_diameter(const BlockBfs& b, int* pdiam, int*
     *pdiam = o.lb;
   } else {
     const BlockBfsOut o2 = block_bfs2(b, o.t, -1);
+    if (o2.reached != b.n) return false;  // stopped
     *pdiam = o2.la;
   }
   return true;

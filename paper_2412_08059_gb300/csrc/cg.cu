@@ -1288,26 +1288,6 @@ struct Stage1Args {
   int bfs_slot;
 };
 
-// Thread 0: wait (bounded) until the feature warp has published the label.
-// Returns t >= 0, or -1 on failure (status set).
-__device__ __forceinline__ int wait_label(Ctl* ctl) {
-  const volatile int* p = &ctl->eps1_ready;
-  const unsigned long long t0 = globaltimer();
-  unsigned spins = 0;
-  while (true) {
-    const int label = *p;
-    if (label > 0) return label - 1;
-    if (label < 0) return -1;
-    if ((++spins & 255u) == 0) {
-      if (volatile_status(ctl) != 0 || poll_cancel(ctl)) return -1;
-      if (globaltimer() - t0 > (unsigned long long)ctl->timeout_ns) {
-        set_status(ctl, MPCG_ERR_TIMEOUT);
-        return -1;
-      }
-    }
-  }
-}
-
 // The feature warp's 2BFS (out of line: its registers are its own).  The
 // block's consumers join its levels once stage 1 waits for nothing but the
 // label (help_begin); the release ends their part on every path.

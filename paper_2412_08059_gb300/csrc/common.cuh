@@ -59,6 +59,7 @@ struct Ctl {
   alignas(128) int cls;
   int eps1_ready;  // fused stage 1: 0 pending, t + 1 when the kNN chose t, -1 on failure
   int x32_src;     // stage-1 result: -1 = x32, s >= 0 = snapshot slot s
+  int feat_sides;  // cluster kernel: sides of the features (l~, v) that are complete
   // device clock marks (ns)
   unsigned long long t_start, t_prep, t_features, t_fp32, t_fp64, t_end;
   unsigned long long t_s2;  // team kernels: start of the double-precision stage (0: not marked)
@@ -167,6 +168,26 @@ __device__ __forceinline__ bool poll_cancel(Ctl* c) {
   if (cancel_word(c) == 0) return false;
   set_status(c, MPCG_ERR_CANCELLED);
   return true;
+}
+
+// Thread 0: wait (bounded) until the label has been published.
+// Returns t >= 0, or -1 on failure (status set).
+__device__ __forceinline__ int wait_label(Ctl* ctl) {
+  const volatile int* p = &ctl->eps1_ready;
+  const unsigned long long t0 = globaltimer();
+  unsigned spins = 0;
+  while (true) {
+    const int label = *p;
+    if (label > 0) return label - 1;
+    if (label < 0) return -1;
+    if ((++spins & 255u) == 0) {
+      if (volatile_status(ctl) != 0 || poll_cancel(ctl)) return -1;
+      if (globaltimer() - t0 > (unsigned long long)ctl->timeout_ns) {
+        set_status(ctl, MPCG_ERR_TIMEOUT);
+        return -1;
+      }
+    }
+  }
 }
 
 // Streaming (read-once-per-sweep) loads for the matrix: evict-first in L1/L2.

@@ -1,0 +1,96 @@
+"""The cluster kernel (small systems) against the grid-wide kernels.
+
+An explicit grid size keeps the grid-wide kernels, so the same call runs both
+ways.  Sizes at the edges: one row, a ragged last slice, fewer slices than
+blocks, one slice more than fills a block's 16 warps, every instance (rows
+per thread), the largest size, and one past it (both calls then take the
+grid).  The two ways sum the inner products in another order, so counts may
+differ by 2 % (at least 1), x within the parity bar of 1e-6; l~, the class
+and the status are equal."""
+import numpy as np
+import pytest
+
+import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def mp():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2412_08059_gb300 import build, mpcg
+    build.build()
+    mpcg.load()
+    return mpcg
+
+
+def _grid(n):
+    """A 2-D grid of n = nx * ny rows with the most square nx that divides n."""
+    nx = next(k for k in range(int(n ** 0.5), 0, -1) if n % k == 0)
+    return synth.laplacian_2d(n // nx, nx, sigma=1e-2)
+
+
+def _two(n):
+    """Two components (the per-component 2BFS)."""
+    A, B = _grid(n), _grid(n // 2)
+    return synth.CSR(np.concatenate([A.row_ptr, A.nnz + B.row_ptr[1:]]).astype(np.int32),
+                     np.concatenate([A.col, A.n + B.col]).astype(np.int32),
+                     np.concatenate([A.val, B.val]))
+
+
+CASES = {f"grid{n}": (lambda n=n: _grid(n)) for n in
+         (1, 31, 33, 480, 512, 513, 8192, 8224, 16384, 16400, 32768, 39990, 40200)}
+CASES.update({
+    "star_1001": lambda: synth.star(1001, 1.1),          # one row past the width cap
+    "rtree_5000": lambda: synth.random_tree_plus(5000, 0.5, 1.1, seed=3),
+    "rreg_20000": lambda: synth.random_regular_laplacian(20000, 8, 1e-3, seed=4),  # columns far away
+    "band_9000_b29": lambda: synth.banded(9000, 29, 0.6, 1.1, seed=7),
+    "two_3000": lambda: _two(2000),
+})
+MODES = {"eps1": dict(eps1=1e-5), "auto": dict(), "fp64": dict(fp64_only=1)}
+
+
+@pytest.mark.parametrize("mode", sorted(MODES))
+@pytest.mark.parametrize("name", sorted(CASES))
+def test_cluster_against_grid(mp, name, mode):
+    A = CASES[name]()
+    _, b = synth.rhs(A, seed=5)
+    feat, cls = synth.random_sample(300, seed=2)
+    S = mp.DeviceSample(feat, cls) if mode == "auto" else None
+    dA, db = mp.DeviceCSR.from_host(A), torch.from_numpy(b).cuda()
+    xc, rc = mp.solve(dA, db, S, **MODES[mode])
+    xg, rg = mp.solve(dA, db, S, grid_blocks=4096, **MODES[mode])
+    assert (rc["status"], rc["pdiam"], rc["cls"]) == (rg["status"], rg["pdiam"], rg["cls"]), (rc, rg)
+    for k in ("n1", "n2"):
+        assert abs(rc[k] - rg[k]) <= max(1, 0.02 * rg[k]), (k, rc[k], rg[k])
+    assert rc["true_rel_resid"] <= 1e-10
+    assert abs(rc["v"] - rg["v"]) <= 1e-9
+    assert torch.linalg.vector_norm(xc - xg) <= 1e-6 * torch.linalg.vector_norm(xg)
+    x2, r2 = mp.solve(dA, db, S, **MODES[mode])
+    assert torch.equal(xc, x2)  # the sums have a fixed order
+
+
+def test_cluster_statuses(mp):
+    """b = 0, NaN in b, an indefinite matrix, a cap, a cancel word set, a broken CSR."""
+    A = _grid(3000)
+    _, b = synth.rhs(A, seed=5)
+    dA, db = mp.DeviceCSR.from_host(A), torch.from_numpy(b).cuda()
+    x, r = mp.solve(dA, torch.zeros_like(db), eps1=1e-4)
+    assert r["status"] == mp.OK and not x.any()
+    bad = db.clone()
+    bad[1234] = float("nan")
+    for kw in (dict(eps1=1e-4), dict(fp64_only=1)):
+        assert mp.solve(dA, bad, **kw)[1]["status"] == mp.ERR_NAN
+        neg = mp.DeviceCSR(dA.row_ptr, dA.col, -dA.val)
+        assert mp.solve(neg, db, **kw)[1]["status"] == mp.ERR_BREAKDOWN
+        r = mp.solve(dA, db, max_it_fp64=3, max_it_fp32=2, **kw)[1]
+        g = mp.solve(dA, db, max_it_fp64=3, max_it_fp32=2, grid_blocks=4096, **kw)[1]
+        assert r["status"] == g["status"] == mp.ERR_NOT_CONVERGED and r["n2"] == g["n2"] == 3
+        assert abs(r["true_rel_resid"] - g["true_rel_resid"]) <= 1e-6 * g["true_rel_resid"]
+        word = torch.ones(1, dtype=torch.int32, pin_memory=True)
+        assert mp.solve(dA, db, cancel=word.data_ptr(), **kw)[1]["status"] == mp.ERR_CANCELLED
+    col = dA.col.clone()
+    col[0] = A.n
+    assert mp.solve(mp.DeviceCSR(dA.row_ptr, col, dA.val), db, eps1=1e-4)[1]["status"] == mp.ERR_INVALID_ARG
