@@ -109,14 +109,15 @@ __device__ __forceinline__ void cbar() {
   asm volatile("bar.sync 1, %0;" ::"r"(NC * 32) : "memory");
 }
 
-// Shared scratch of the consumer group: per-thread partials and the values
+// Shared scratch of the consumer group: partial sums and the values
 // that thread 0 broadcasts after each reduction.  Scalars of the iteration
 // (alpha, beta, the stop test) are computed once per block by thread 0 (they
 // are the same in every block: same totals, same operations), which keeps
 // the slow FP64 units free of redundant work.
 template <int NC>
 struct CShared {
-  double part[NC * 32];
+  double part[NC * 16];
+  double wsum[4];
   float ffp[2 * NC];
   double rr, val;
   float alpha, beta;
@@ -145,20 +146,30 @@ __device__ __forceinline__ double block_ff(FF v, CShared<NC>& S, bool f32) {
   return r;
 }
 
-// Block partial of per-thread doubles, valid in thread 0 (one warp adds them
-// in a fixed order).
+// Block partial of per-thread doubles, valid in warp 0.  A dependent FP64 add
+// takes 64 clocks, and one warp cannot issue them faster; so the threads'
+// values are folded in half in each warp, then summed by four warps (one per
+// sub-partition of the SM, which issue side by side): about 1,000 clocks
+// against 1,460 with one warp adding 15 values a lane.  Half a warp's values
+// a warp also keep the block's static shared memory under 3 KB, so that the
+// FP64 ring and it fit the 196 KB carve-out and the L1 cache keeps 60 KB
+// instead of 28 for the gathers.
 template <int NC>
 __device__ __forceinline__ double block_d(double p, CShared<NC>& S) {
-  const int lane = threadIdx.x & 31;
-  S.part[threadIdx.x] = p;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  p += __shfl_xor_sync(0xffffffffu, p, 16);
+  if (lane < 16) S.part[16 * warp + lane] = p;
+  cbar<NC>();
+  constexpr int N = 16 * NC;  // values; thread t < 128 sums t and t + 128
+  if (warp < 4) {
+    const int t = threadIdx.x;
+    double s = S.part[t] + (t + 128 < N ? S.part[t + 128] : 0.0);
+    s = warp_sum(s);
+    if (lane == 0) S.wsum[warp] = s;
+  }
   cbar<NC>();
   double r = 0.0;
-  if (threadIdx.x < 32) {
-    double s = 0.0;
-#pragma unroll
-    for (int j = 0; j < NC; ++j) s += S.part[lane + 32 * j];
-    r = warp_sum(s);
-  }
+  if (warp == 0) r = (S.wsum[0] + S.wsum[1]) + (S.wsum[2] + S.wsum[3]);
   return r;
 }
 
@@ -321,12 +332,6 @@ __device__ __forceinline__ bool ring_acquire(Ring<T>& R, Cursor& C, unsigned g_l
   return true;
 }
 
-// Chunk range [lo, hi] of a slice's k-rows (w > 0) relative to the pass.
-__device__ __forceinline__ void slice_chunks(int r0, int w, unsigned& lo, unsigned& hi) {
-  lo = (unsigned)r0 >> kLogCH;
-  hi = (unsigned)(r0 + kSlice * (w - 1)) >> kLogCH;
-}
-
 // Load the (column, value) pairs of one slice row from the ring.  A slice
 // spans at most two chunks: the stage of its first chunk and the next one.
 // C16: the ring holds int16 offsets from the row index i.
@@ -373,102 +378,186 @@ __device__ __forceinline__ void ring_load(const Ring<T>& R, const Cursor& C, int
   else ring_load_t<T, false>(R, C, r0, w, lane, i, c, v);
 }
 
-// Row sum of one slice row, generic width, from the ring (plus the tail of an
-// overflowing row from the caller's CSR).
-template <typename T, class Gather>
-__device__ __forceinline__ T ring_row_generic(const CgArgs& a, const Ring<T>& R, const Cursor& C,
-                                              int r0, uint32_t wf, int i, int lane, Gather G) {
-  const int w = (int)(wf & ~kOverflowBit);
-  T acc = (T)0;
-  for (int k = 0; k < w; ++k) {
-    const int rr = r0 + kSlice * k + lane;
-    const int st = (int)((C.pass_base + ((unsigned)rr >> kLogCH)) % Ring<T>::S);
-    const int off = rr & (kCH - 1);
-    const int cc = R.c16 ? i + (int)R.cols16(st)[off] : R.cols(st)[off];
-    acc = fma(R.vals(st)[off], G(cc), acc);
+__device__ __forceinline__ bool fast_w(uint32_t wf) {
+  return !(wf & kOverflowBit) && (int)wf <= kFastW;
+}
+
+// Sums over W entries a row, from entry k0 of the rows on, of one slice or of
+// two adjacent ones (kRows; the second slice's entries start `stride` columns
+// of 32 after the first's): all gathers first, then the chains of fused
+// multiply-adds.  Nothing is predicated: a predicated-off FP64 instruction
+// takes its turn of the FP64 pipe all the same (measured: 16 warps x 1 FMA
+// take 304 clocks of an SM with the predicate on or off), so a form for any
+// width up to 8 paid 8 FMAs a row for the 5 of a 2-D and the 7 of a 3-D
+// stencil.  kCross: the entries may cross into the ring's next stage.
+template <typename T, bool C16, int W, int kRows, bool kCross, class Gather>
+__device__ __forceinline__ void row_sums(const Ring<T>& R, const Cursor& C, int r0, int stride, int lane,
+                                         int i0, Gather G, T& acc0, T& acc1) {
+  using CT = typename std::conditional<C16, int16_t, int32_t>::type;
+  const int st0 = (int)((C.pass_base + ((unsigned)r0 >> kLogCH)) % Ring<T>::S);
+  const int off = r0 & (kCH - 1);
+  const CT* cp = reinterpret_cast<const CT*>(R.cols(st0)) + off + lane;
+  const T* vp = R.vals(st0) + off + lane;
+  // entry k of the first row is at 32 k; past the stage's end, at the same
+  // distance less kCH from the start of the next stage
+  const int next = st0 + 1 == Ring<T>::S ? -st0 : 1;
+  const int dc = next * (int)(stage_bytes<T>() / sizeof(CT)) - kCH;
+  const int dv = next * (int)(stage_bytes<T>() / sizeof(T)) - kCH;
+  auto col = [&](int k) -> int {
+    return (int)cp[kSlice * k + (kCross && off + kSlice * k >= kCH ? dc : 0)];
+  };
+  auto val = [&](int k) -> T {
+    return vp[kSlice * k + (kCross && off + kSlice * k >= kCH ? dv : 0)];
+  };
+  T x0[W], x1[W];
+#pragma unroll
+  for (int k = 0; k < W; ++k) {
+    x0[k] = G(C16 ? i0 + col(k) : col(k));
+    if (kRows == 2) x1[k] = G(C16 ? i0 + kSlice + col(stride + k) : col(stride + k));
   }
-  if ((wf & kOverflowBit) && i < a.n) {
+#pragma unroll
+  for (int k = 0; k < W; ++k) {
+    acc0 = fma(val(k), x0[k], acc0);
+    if (kRows == 2) acc1 = fma(val(stride + k), x1[k], acc1);
+  }
+}
+template <typename T, int W, int kRows, class Gather>
+__device__ __forceinline__ void row_sums_w(const Ring<T>& R, const Cursor& C, int r0, int lane, int i0,
+                                           Gather G, T& acc0, T& acc1) {
+  const bool cross = (r0 & (kCH - 1)) + kRows * W * kSlice > kCH;
+  if (R.c16) {
+    if (cross) row_sums<T, true, W, kRows, true>(R, C, r0, W, lane, i0, G, acc0, acc1);
+    else row_sums<T, true, W, kRows, false>(R, C, r0, W, lane, i0, G, acc0, acc1);
+  } else {
+    if (cross) row_sums<T, false, W, kRows, true>(R, C, r0, W, lane, i0, G, acc0, acc1);
+    else row_sums<T, false, W, kRows, false>(R, C, r0, W, lane, i0, G, acc0, acc1);
+  }
+}
+template <typename T, int kRows, class Gather>
+__device__ __forceinline__ bool row_sums_any(const Ring<T>& R, const Cursor& C, int r0, int w, int lane,
+                                             int i0, Gather G, T& acc0, T& acc1) {
+  switch (w) {  // warp-uniform
+    case 3: row_sums_w<T, 3, kRows>(R, C, r0, lane, i0, G, acc0, acc1); return true;
+    case 4: row_sums_w<T, 4, kRows>(R, C, r0, lane, i0, G, acc0, acc1); return true;
+    case 5: row_sums_w<T, 5, kRows>(R, C, r0, lane, i0, G, acc0, acc1); return true;
+    case 6: row_sums_w<T, 6, kRows>(R, C, r0, lane, i0, G, acc0, acc1); return true;
+    case 7: row_sums_w<T, 7, kRows>(R, C, r0, lane, i0, G, acc0, acc1); return true;
+    case 8: row_sums_w<T, 8, kRows>(R, C, r0, lane, i0, G, acc0, acc1); return true;
+    case 9: row_sums_w<T, 9, kRows>(R, C, r0, lane, i0, G, acc0, acc1); return true;
+    default: return false;
+  }
+}
+
+// Entries [k, m) of one row or of two (kRows), any number of them, four at a
+// time.  kRows == 2: the second row's entries start `stride` after the first's.
+template <typename T, bool C16, int kRows, class Gather>
+__device__ __forceinline__ void row_sums_range(const Ring<T>& R, const Cursor& C, int r0, int stride, int k,
+                                               int m, int lane, int i0, Gather G, T& acc0, T& acc1) {
+#pragma unroll 1
+  for (; k + 4 <= m; k += 4)
+    row_sums<T, C16, 4, kRows, true>(R, C, r0 + kSlice * k, stride, lane, i0, G, acc0, acc1);
+  switch (m - k) {
+    case 1: row_sums<T, C16, 1, kRows, true>(R, C, r0 + kSlice * k, stride, lane, i0, G, acc0, acc1); break;
+    case 2: row_sums<T, C16, 2, kRows, true>(R, C, r0 + kSlice * k, stride, lane, i0, G, acc0, acc1); break;
+    case 3: row_sums<T, C16, 3, kRows, true>(R, C, r0 + kSlice * k, stride, lane, i0, G, acc0, acc1); break;
+    default: break;
+  }
+}
+// Two adjacent slices (or one: w1 = 0) of any widths: the entries that both
+// rows have side by side, then the rest of the longer row.
+template <typename T, bool C16, class Gather>
+__device__ __forceinline__ void row_sums_mixed(const Ring<T>& R, const Cursor& C, int r0, int w0, int w1,
+                                               int lane, int i0, Gather G, T& acc0, T& acc1) {
+  const int m = min(w0, w1);
+  T none;
+  row_sums_range<T, C16, 2>(R, C, r0, w0, 0, m, lane, i0, G, acc0, acc1);
+  const bool second = w1 > w0;
+  T t = second ? acc1 : acc0;
+  row_sums_range<T, C16, 1>(R, C, second ? r0 + kSlice * w0 : r0, 0, m, max(w0, w1), lane,
+                            second ? i0 + kSlice : i0, G, t, none);
+  if (second) acc1 = t;
+  else acc0 = t;
+}
+// The entries of row i past the slice's width (a row longer than the layout
+// keeps), from the caller's CSR.
+template <typename T, class Gather>
+__device__ __forceinline__ T row_tail(const CgArgs& a, int i, int w, T acc, Gather G) {
+  if (i < a.n) {
     const int e1 = a.rp[i + 1];
     for (int e = a.rp[i] + w; e < e1; ++e) acc = fma((T)a.val[e], G(a.col[e]), acc);
   }
   return acc;
 }
 
-__device__ __forceinline__ bool fast_w(uint32_t wf) {
-  return !(wf & kOverflowBit) && (int)wf <= kFastW;
-}
-
 // One SpMV pass over the block's slices by the consumer warps.  For every
 // row i of the block's slices (padding rows included), Rw(i, acc) receives
-// sum_k v_k G(c_k) in stored order.  A warp takes two slices (s, s + kNC) per
-// step when both fit in two chunks, so that the gathers of both rows are in
-// flight together; a step never needs more than two chunks at once (the ring
-// has at least four), which keeps the producer/consumer ring free of
-// deadlock.  Returns false if a wait failed.
+// sum_k v_k G(c_k) in stored order.  A warp takes two adjacent slices per
+// step (one when the block has no more slices than warps), so that the gathers
+// of both rows are in flight together; their entries are contiguous, at most 2 x 32 x 64 = kCH of them, so a step never
+// needs more than two chunks at once (the ring has at least four), which
+// keeps the producer/consumer ring free of deadlock.  The next step's widths
+// and offsets are loaded a step ahead: they come from L2 (the gathers evict
+// them from L1), and a step would otherwise start with that round trip.
+// Returns false if a wait failed.
 template <int NC, typename T, class Gather, class Row>
 __device__ __forceinline__ bool ring_spmv(const CgArgs& a, Ring<T>& R, Cursor& C, int S0, int S1,
                                           Gather G, Row Rw) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   bool ok = true;
-  for (int s0 = S0 + warp; s0 < S1; s0 += 2 * NC) {
-    const int s1 = s0 + NC;
-    const bool h1 = s1 < S1;
-    const uint32_t wf0 = a.slice_w[s0];
-    const uint32_t wf1 = h1 ? a.slice_w[s1] : 0u;
-    const int w0 = (int)(wf0 & ~kOverflowBit), w1 = (int)(wf1 & ~kOverflowBit);
-    const int r00 = a.slice_ptr[s0] - R.E0;
-    const int r01 = h1 ? a.slice_ptr[s1] - R.E0 : 0;
-    const int i0 = s0 * kSlice + lane, i1 = s1 * kSlice + lane;
-    unsigned lo0 = 0, hi0 = 0, lo1 = 0, hi1 = 0;
-    if (w0 > 0) slice_chunks(r00, w0, lo0, hi0);
-    if (w1 > 0) slice_chunks(r01, w1, lo1, hi1);
-    const bool pair = h1 && w0 > 0 && w1 > 0 && fast_w(wf0) && fast_w(wf1) && hi1 <= lo0 + 1;
-    if (pair) {
-      if (ok) ok = ring_release_below(R, C, C.pass_base + lo0, lane, a.ctl);
-      if (ok) ok = ring_acquire(R, C, C.pass_base + lo0, C.pass_base + hi1, a.ctl);
-      T acc0 = (T)0, acc1 = (T)0;
-      if (ok) {
-        int c0[kFastW], c1[kFastW];
-        T v0[kFastW], v1[kFastW];
-        ring_load(R, C, r00, w0, lane, i0, c0, v0);
-        ring_load(R, C, r01, w1, lane, i1, c1, v1);
-#pragma unroll
-        for (int k = 0; k < kFastW; ++k) {
-          if (k < w0) acc0 = fma(v0[k], G(c0[k]), acc0);
-          if (k < w1) acc1 = fma(v1[k], G(c1[k]), acc1);
-        }
-      }
-      Rw(i0, acc0);
-      Rw(i1, acc1);
-      continue;
+  const int per = S1 - S0 > NC ? 2 : 1;  // slices a step
+  int s0 = S0 + per * warp;
+  uint32_t nf0 = 0u, nf1 = 0u;
+  int np = 0;
+  if (s0 < S1) {
+    nf0 = a.slice_w[s0];
+    np = a.slice_ptr[s0];
+    if (per == 2 && s0 + 1 < S1) nf1 = a.slice_w[s0 + 1];
+  }
+  for (; s0 < S1; s0 += per * NC) {
+    const uint32_t wf0 = nf0, wf1 = nf1;
+    const int r0 = np - R.E0;
+    const bool h1 = per == 2 && s0 + 1 < S1;
+    const int sn = s0 + per * NC;
+    if (sn < S1) {
+      nf0 = a.slice_w[sn];
+      np = a.slice_ptr[sn];
+      nf1 = per == 2 && sn + 1 < S1 ? a.slice_w[sn + 1] : 0u;
     }
-    for (int j = 0; j < 2; ++j) {  // one slice at a time
-      const bool hj = j == 0 || h1;
-      if (!hj) break;
-      const uint32_t wf = j ? wf1 : wf0;
-      const int w = j ? w1 : w0;
-      const int r0 = j ? r01 : r00;
-      const int i = j ? i1 : i0;
-      T acc = (T)0;
-      if (w > 0) {
-        const unsigned lo = j ? lo1 : lo0, hi = j ? hi1 : hi0;
-        if (ok) ok = ring_release_below(R, C, C.pass_base + lo, lane, a.ctl);
-        if (ok) ok = ring_acquire(R, C, C.pass_base + lo, C.pass_base + hi, a.ctl);
-      }
-      if (ok) {
-        if (fast_w(wf)) {
-          int c[kFastW];
-          T v[kFastW];
-          ring_load(R, C, r0, w, lane, i, c, v);
+    const int w0 = (int)(wf0 & ~kOverflowBit), w1 = h1 ? (int)(wf1 & ~kOverflowBit) : 0;
+    const int i0 = s0 * kSlice + lane, i1 = i0 + kSlice;
+    const int end = r0 + kSlice * (w0 + w1);
+    if (end > r0) {
+      const unsigned lo = (unsigned)r0 >> kLogCH, hi = (unsigned)(end - 1) >> kLogCH;
+      if (ok) ok = ring_release_below(R, C, C.pass_base + lo, lane, a.ctl);
+      if (ok) ok = ring_acquire(R, C, C.pass_base + lo, C.pass_base + hi, a.ctl);
+    }
+    T acc0 = (T)0, acc1 = (T)0;
+    if (ok) {
+      // (a width with the overflow flag is none of the listed ones)
+      const bool done = h1 ? wf0 == wf1 && row_sums_any<T, 2>(R, C, r0, (int)wf0, lane, i0, G, acc0, acc1)
+                           : row_sums_any<T, 1>(R, C, r0, (int)wf0, lane, i0, G, acc0, acc1);
+      if (!done) {
+        const int r1 = r0 + kSlice * w0;
+        if (sizeof(T) == 4 && h1 && fast_w(wf0) && fast_w(wf1)) {
+          int c0[kFastW], c1[kFastW];
+          T v0[kFastW], v1[kFastW];
+          ring_load(R, C, r0, w0, lane, i0, c0, v0);
+          ring_load(R, C, r1, w1, lane, i1, c1, v1);
 #pragma unroll
-          for (int k = 0; k < kFastW; ++k)
-            if (k < w) acc = fma(v[k], G(c[k]), acc);
+          for (int k = 0; k < kFastW; ++k) {
+            if (k < w0) acc0 = fma(v0[k], G(c0[k]), acc0);
+            if (k < w1) acc1 = fma(v1[k], G(c1[k]), acc1);
+          }
         } else {
-          acc = ring_row_generic(a, R, C, r0, wf, i, lane, G);
+          if (R.c16) row_sums_mixed<T, true>(R, C, r0, w0, w1, lane, i0, G, acc0, acc1);
+          else row_sums_mixed<T, false>(R, C, r0, w0, w1, lane, i0, G, acc0, acc1);
+          if (wf0 & kOverflowBit) acc0 = row_tail<T>(a, i0, w0, acc0, G);
+          if (h1 && (wf1 & kOverflowBit)) acc1 = row_tail<T>(a, i1, w1, acc1, G);
         }
       }
-      Rw(i, acc);
     }
+    Rw(i0, acc0);
+    if (h1) Rw(i1, acc1);
   }
   C.pass_base += R.nch;
   if (ok) ok = ring_release_below(R, C, C.pass_base, lane, a.ctl);
