@@ -34,9 +34,9 @@
 
 namespace mpcg {
 
-// Set-up of a system: CSR check, b~ = float32(b), sliced layout, ||b||; x = 0
-// when b = 0.  Returns false if the launch aborted.
-static __device__ bool sys_prep(Team& t, const BatchSys& s, const BatchArgs& a, int& red) {
+// Set-up of a system: CSR check, b~ = float32(b), sliced layout (narrow: with
+// the 16-bit copy of the columns), ||b||; x = 0 when b = 0.  Returns false if the launch aborted.
+static __device__ bool sys_prep(Team& t, const BatchSys& s, const BatchArgs& a, int& red, bool narrow) {
   Ctl* ctl = s.w.ctl;
   const bool lead0 = t.rank == 0 && threadIdx.x == 0;
   sys_init(t, s, a);
@@ -46,7 +46,7 @@ static __device__ bool sys_prep(Team& t, const BatchSys& s, const BatchArgs& a, 
   if (sys_status(s) == 0) {
     if (t.rank == 0) block_scan_slices(s.w.slice_w, s.w.slice_ptr, s.nslices);
     if (!team_sync(t)) return false;
-    sys_fill(t, s, true);
+    sys_fill(t, s, narrow);
     // ||b||_2 in double
     double p = 0.0;
     for (int i = team_tid(t); i < s.n; i += team_threads(t)) p = __fma_rn(s.b[i], s.b[i], p);
@@ -74,7 +74,7 @@ static __device__ bool sys_prep(Team& t, const BatchSys& s, const BatchArgs& a, 
 static __device__ bool sys_stage1(Team& t, const BatchSys& s, const BatchArgs& a) {
   Ctl* ctl = s.w.ctl;
   int red = 0;
-  if (!sys_prep(t, s, a, red)) return false;
+  if (!sys_prep(t, s, a, red, true)) return false;
   if (sys_status(s) != 0 || ctl->trivial) return true;
   bool done;
   if (a.auto_eps1) {
@@ -84,7 +84,7 @@ static __device__ bool sys_stage1(Team& t, const BatchSys& s, const BatchArgs& a
     if (!team_sync(t)) return false;
     if (sys_status(s) == 0 && t.rank == 0 && threadIdx.x < 32) {
       const double chi[4] = {(double)s.n, (double)s.nnz, (double)ctl->pdiam, ctl->v};
-      const int cls = knn_warp(a.knn, chi);
+      const int cls = team_vote(&a.knn, chi);
       if (threadIdx.x == 0) {
         if (cls < 0) {
           set_status(ctl, MPCG_ERR_INVALID_ARG);
@@ -103,92 +103,25 @@ static __device__ bool sys_stage1(Team& t, const BatchSys& s, const BatchArgs& a
   return team_sync(t);
 }
 
-// The whole method for one system in one launch (set-up, features or the
-// fixed eps1, both stages, the result record), single-precision SpMV from
-// global memory; with a.part == 2 only the double-precision stage after
-// sys_stage1 and the result record.  Returns false if the launch aborted.
-// Its set-up repeats sys_prep's steps inline on purpose: this kernel's code
-// sets the schedule of its FP64 loops (see k_batch), and this form is the
-// one measured at 305 ms for the FP64-only 512-system batch.
-static __device__ bool sys_solve(Team& t, const BatchSys& s, const BatchArgs& a) {
+// The double-precision stage and the result record: after sys_stage1
+// (a.part == 2), or with the set-up before it (a pure FP64 batch).  Returns
+// false if the launch aborted.
+static __device__ bool sys_stage2(Team& t, const BatchSys& s, const BatchArgs& a) {
   Ctl* ctl = s.w.ctl;
-  const bool lead0 = t.rank == 0 && threadIdx.x == 0;
   int red = 0;
-  if (a.part == 2) {
-    bool done;
-    if (sys_status(s) == 0 && !*reinterpret_cast<volatile int*>(&ctl->trivial) &&
-        !sys_cg64(t, s, 0, red, kNoBudget, false, &done))
-      return false;
-    if (!team_sync(t)) return false;
-    sys_finalize(t, s);
-    return true;
-  }
-  sys_init(t, s, a);
-  if (!team_sync(t)) return false;
-  sys_rows(t, s);
-  if (!team_sync(t)) return false;
-  if (sys_status(s) == 0) {
-    if (t.rank == 0) block_scan_slices(s.w.slice_w, s.w.slice_ptr, s.nslices);
-    if (!team_sync(t)) return false;
-    sys_fill(t, s, false);
-    // ||b||_2 in double
-    double p = 0.0;
-    for (int i = team_tid(t); i < s.n; i += team_threads(t)) p = __fma_rn(s.b[i], s.b[i], p);
-    double bb;
-    if (!team_sum_d(t, p, s.w.partials, red, bb)) return false;  // includes the fill barrier
-    if (lead0) {
-      const double bn = sqrt(bb);
-      ctl->t_prep = globaltimer();
-      ctl->bnorm64 = bn;
-      if (!isfinite(bn)) set_status(ctl, MPCG_ERR_NAN);
-      else if (bn == 0.0) ctl->trivial = 1;
-    }
-    if (!team_sync(t)) return false;
-  }
-  const bool trivial = ctl->trivial != 0;
-  if (sys_status(s) == 0 && trivial) {  // b = 0: x = 0 solves A x = b exactly
-    for (int i = team_tid(t); i < s.n; i += team_threads(t)) s.x[i] = 0.0;
-  } else if (sys_status(s) == 0 && a.o.fp64_only) {  // pure FP64 CG from x0 = 0
-    bool done;
-    if (!sys_cg64(t, s, 1, red, kNoBudget, false, &done)) return false;
-  } else if (sys_status(s) == 0) {
-    if (a.auto_eps1) {
-      // Algorithm II: l~ by 2BFS, v over the first k0 iterations, eps1 by kNN
-      if (!team_pseudo_diameter(t, s, a.smem_bytes)) return false;
-      if (!team_sync(t)) return false;
-      bool done;
-      if (!sys_cg32<false>(t, s, kCgK0, red, kNoBudget, &done)) return false;
-      if (!team_sync(t)) return false;
-      if (sys_status(s) == 0 && t.rank == 0 && threadIdx.x < 32) {
-        const double chi[4] = {(double)s.n, (double)s.nnz, (double)ctl->pdiam, ctl->v};
-        const int cls = knn_warp(a.knn, chi);
-        if (threadIdx.x == 0) {
-          if (cls < 0) {
-            set_status(ctl, MPCG_ERR_INVALID_ARG);
-          } else {
-            ctl->cls = cls;
-            ctl->eps1 = pow10_neg(cls);
-          }
-          ctl->t_features = globaltimer();
-        }
-      }
-      if (!team_sync(t)) return false;
-      if (sys_status(s) == 0 && !sys_cg32<false>(t, s, kCgContinue, red, kNoBudget, &done)) return false;
-    } else {
-      bool done;
-      if (!sys_cg32<false>(t, s, kCgToEps1, red, kNoBudget, &done)) return false;
-    }
-    if (!team_sync(t)) return false;
-    bool done;
-    if (sys_status(s) == 0 && !sys_cg64(t, s, 0, red, kNoBudget, false, &done)) return false;
-  }
+  const bool whole = a.part != 2;
+  if (whole && !sys_prep(t, s, a, red, false)) return false;
+  bool done;
+  if (sys_status(s) == 0 && !*reinterpret_cast<volatile int*>(&ctl->trivial) &&
+      !sys_cg64(t, s, whole ? 1 : 0, red, kNoBudget, false, &done))
+    return false;
   if (!team_sync(t)) return false;
   sys_finalize(t, s);
   return true;
 }
 
 // The persistent team loop of one launch: kPart 1 runs sys_stage1 on every
-// system, kPart 2 sys_solve.  Two kernels, so that the code of one stage
+// system, kPart 2 sys_stage2.  Two kernels, so that the code of one stage
 // does not change the register allocation of the other's loops (measured:
 // with both stages in one kernel, whatever else the kernel held moved the
 // FP64 stage by up to 50 %).
@@ -217,7 +150,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1) k_batch(BatchArgs a) {
     if constexpr (kPart == 1) {
       if (!sys_stage1(t, a.sys[idx], a)) return;
     } else {
-      if (!sys_solve(t, a.sys[idx], a)) return;
+      if (!sys_stage2(t, a.sys[idx], a)) return;
     }
     if (!team_sync(t)) return;  // every block has read next[team]
   }

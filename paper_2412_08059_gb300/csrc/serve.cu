@@ -72,7 +72,7 @@ __device__ bool slot_features(Team& t, const BatchSys& s, const BatchArgs& a, in
   if (!team_sync(t)) return false;
   if (sys_status(s) == 0 && t.rank == 0 && threadIdx.x < 32) {
     const double chi[4] = {(double)s.n, (double)s.nnz, (double)ctl->pdiam, ctl->v};
-    const int cls = knn_warp(a.knn, chi);
+    const int cls = team_vote(&a.knn, chi);
     if (threadIdx.x == 0) {
       if (cls < 0) {
         set_status(ctl, MPCG_ERR_INVALID_ARG);

@@ -80,7 +80,8 @@ struct BatchArgs {
 // Team context: barrier, block-level scratch, deterministic team sums.
 // ---------------------------------------------------------------------------------------
 struct TeamShared {
-  double dpart[kBatchWarps];
+  double dpart[16 * kBatchWarps];
+  double wsum[4];
   float ffp[2 * kBatchWarps];
   double val[4];
   float fval[2];
@@ -152,18 +153,24 @@ struct TeamSyncFn {
 // alternates between two halves of the system's partials array.
 static __device__ bool team_sum_d(Team& t, double v, double* partials, int& red, double& out) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  v = warp_sum(v);
-  if (lane == 0) t.S->dpart[warp] = v;
+  // Folded in half in each warp, then by four warps (one per sub-partition
+  // of the SM): a dependent FP64 add takes 64 clocks of the warp's
+  // sub-partition and 19 of the SM, so 16 butterflies took 1,520 clocks.
+  v += __shfl_xor_sync(0xffffffffu, v, 16);
+  if (lane < 16) t.S->dpart[16 * warp + lane] = v;
+  __syncthreads();
+  if (warp < 4) {
+    double s = t.S->dpart[threadIdx.x] + t.S->dpart[threadIdx.x + 128];
+    s = warp_sum(s);
+    if (lane == 0) t.S->wsum[warp] = s;
+  }
   __syncthreads();
   double* buf = partials + (red & 1) * kMaxGrid;
   ++red;
-  if (threadIdx.x < 32) {
-    double s = lane < kBatchWarps ? t.S->dpart[lane] : 0.0;
-    s = warp_sum(s);
-    if (threadIdx.x == 0) {
-      if (t.size == 1) t.S->val[0] = s;
-      else buf[t.rank] = s;
-    }
+  if (threadIdx.x == 0) {
+    const double s = (t.S->wsum[0] + t.S->wsum[1]) + (t.S->wsum[2] + t.S->wsum[3]);
+    if (t.size == 1) t.S->val[0] = s;
+    else buf[t.rank] = s;
   }
   if (t.size > 1) {
     if (!team_sync(t)) return false;
@@ -660,6 +667,115 @@ __device__ __forceinline__ void team_rows(const Team& t, const BatchSys& s, Ld L
   }
 }
 
+// ---- double precision: forms without predication ----
+// A predicated-off FP64 instruction takes its turn of the FP64 pipe all the
+// same, and that pipe bounds the stage (one warp-wide FMA per 19 clocks and
+// SM: 12 FMAs a row of a 3-D grid are 113 us an iteration at 32,768 rows a
+// block).  So full steps of four slices run unpredicated, and what is left
+// over takes narrower steps.
+
+// One step of U slices: rows i[u] of widths w[u] (entries from p[u] on).
+template <int U, class Gather, class Pre, class Row>
+__device__ __forceinline__ void team_step64(const BatchSys& s, const int (&p)[U], const uint32_t (&wf)[U],
+                                            const int (&i)[U], Gather G, Pre P, Row Rw) {
+  const double* sv = s.w.sv64;
+  const int32_t* sc = s.w.scol;
+  double a[U];
+  decltype(P(0)) own[U];
+  int wmin = 0x7fffffff, wmax = 0;
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int w = (int)(wf[u] & ~kOverflowBit);
+    wmin = min(wmin, w);
+    wmax = max(wmax, w);
+    a[u] = 0.0;
+    own[u] = P(i[u]);  // before the gathers: Rw stores, and loads do not pass stores
+  }
+#pragma unroll 2
+  for (int k = 0; k < wmin; ++k) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) a[u] = fma(sv[p[u] + kSlice * k], G(sc[p[u] + kSlice * k]), a[u]);
+  }
+#pragma unroll 1
+  for (int k = wmin; k < wmax; ++k) {
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (k < (int)(wf[u] & ~kOverflowBit))
+        a[u] = fma(sv[p[u] + kSlice * k], G(sc[p[u] + kSlice * k]), a[u]);
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    if ((wf[u] & kOverflowBit) && i[u] < s.n)
+      a[u] = btail<double>(s, i[u], (int)(wf[u] & ~kOverflowBit), a[u], G);
+    Rw(i[u], a[u], own[u]);
+  }
+}
+
+// SpMV over the team's slices: warp gw owns slices gw, gw + W, ...; lane l
+// owns row 32 s + l.  Rw(i, acc, own) receives row i's sum in stored order
+// (fused multiply-adds from zero, padding rows included) and the row's own
+// values that P(i) loaded before the gathers.  The metadata of 32 of the
+// warp's slices is loaded at once (one slice per lane).
+template <class Gather, class Pre, class Row>
+__device__ __forceinline__ void team_spmv64(const Team& t, const BatchSys& s, Gather G, Pre P, Row Rw) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int gw = team_warp(t), W = team_warps(t);
+  for (int base = gw; base < s.nslices; base += 32 * W) {
+    const int mine = base + lane * W;
+    uint32_t mwf = 0u;
+    int mp = 0;
+    if (mine < s.nslices) {
+      mwf = s.w.slice_w[mine];
+      mp = s.w.slice_ptr[mine];
+    }
+    const int cnt = min(32, (s.nslices - base + W - 1) / W);
+    int j = 0;
+    auto step = [&](auto width) {
+      constexpr int U = decltype(width)::value;
+      int p[U], i[U];
+      uint32_t wf[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        wf[u] = __shfl_sync(full, mwf, j + u);
+        p[u] = __shfl_sync(full, mp, j + u) + lane;
+        i[u] = (base + (j + u) * W) * kSlice + lane;
+      }
+      team_step64<U>(s, p, wf, i, G, P, Rw);
+      j += U;
+    };
+    while (j + 4 <= cnt) step(std::integral_constant<int, 4>{});
+    if (j + 2 <= cnt) step(std::integral_constant<int, 2>{});
+    if (j < cnt) step(std::integral_constant<int, 1>{});
+  }
+}
+
+// Row phases of the double-precision stage: as team_rows, four full slices a
+// step, then two, then one; the ragged last slice by itself.
+template <class Ld, class Op>
+__device__ __forceinline__ void team_rows64(const Team& t, const BatchSys& s, Ld L, Op O) {
+  const int lane = threadIdx.x & 31;
+  const int gw = team_warp(t), W = team_warps(t);
+  const int fs = s.n >> 5;  // slices of 32 rows
+  int sl = gw;
+  auto step = [&](auto width) {
+    constexpr int U = decltype(width)::value;
+    decltype(L(0)) v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) v[u] = L((sl + u * W) * kSlice + lane);
+#pragma unroll
+    for (int u = 0; u < U; ++u) O((sl + u * W) * kSlice + lane, v[u]);
+    sl += U * W;
+  };
+  while (sl + 3 * W < fs) step(std::integral_constant<int, 4>{});
+  if (sl + W < fs) step(std::integral_constant<int, 2>{});
+  if (sl < fs) step(std::integral_constant<int, 1>{});
+  if (sl == fs) {
+    const int i = sl * kSlice + lane;
+    if (i < s.n) O(i, L(i));
+  }
+}
+
 // Broadcast of thread 0's decision (and scalars) to the block.
 __device__ __forceinline__ int bcast_dec(Team& t, int dec) {
   if (threadIdx.x == 0) t.S->ival[0] = dec;
@@ -870,7 +986,7 @@ static __device__ bool sys_cg64(Team& t, const BatchSys& s, int from_zero, int& 
     // restart (CG line 1 from x): r = b - A x, d = r, r^T r
     if (!skip_restart) {
     double p = 0.0;
-    team_spmv<double, false>(
+    team_spmv64(
         t, s, [&](int c) -> double { return x[c]; },
         [&](int i) -> double { return i < n ? b[i] : 0.0; },
         [&](int i, double acc, double bi) {
@@ -917,7 +1033,7 @@ static __device__ bool sys_cg64(Team& t, const BatchSys& s, int from_zero, int& 
       }
       // P1: q = A d, d^T q
       double pq = 0.0;
-      team_spmv<double, false>(
+      team_spmv64(
           t, s, [&](int c) -> double { return d[c]; },
           [&](int i) -> double { return i < n ? d[i] : 0.0; },
           [&](int i, double acc, double di) {
@@ -942,7 +1058,7 @@ static __device__ bool sys_cg64(Team& t, const BatchSys& s, int from_zero, int& 
       const double alpha = t.S->val[2];
       // P2: x += alpha d, r -= alpha q, r^T r
       double pr = 0.0;
-      team_rows(
+      team_rows64(
           t, s, [&](int i) -> double4 { return make_double4(d[i], x[i], q[i], r[i]); },
           [&](int i, double4 v) {
             x[i] = __fma_rn(alpha, v.x, v.y);
@@ -965,7 +1081,7 @@ static __device__ bool sys_cg64(Team& t, const BatchSys& s, int from_zero, int& 
       const double beta = t.S->val[3];
       rr = rrn;
       // P3: d = r + beta d
-      team_rows(
+      team_rows64(
           t, s, [&](int i) -> double2 { return make_double2(d[i], r[i]); },
           [&](int i, double2 v) { d[i] = __fma_rn(beta, v.x, v.y); });
       if (!team_sync(t)) return false;
@@ -974,7 +1090,7 @@ static __device__ bool sys_cg64(Team& t, const BatchSys& s, int from_zero, int& 
     if (failed && failed != MPCG_ERR_NOT_CONVERGED) break;
     // true residual ||b - A x|| (also after the iteration cap)
     double pt = 0.0;
-    team_spmv<double, false>(
+    team_spmv64(
         t, s, [&](int c) -> double { return x[c]; },
         [&](int i) -> double { return i < n ? b[i] : 0.0; },
         [&](int i, double acc, double bi) {
@@ -1080,6 +1196,12 @@ static __device__ __noinline__ void block_bfs_system(const BatchSys* sp, int sme
     }
     ctl->connected = ok ? 1 : 0;
   }
+}
+
+// The kNN vote by one warp.  Not inlined, for the reason block_bfs_system is
+// not.
+static __device__ __noinline__ int team_vote(const KnnSpec* knn, const double* chi) {
+  return knn_warp(*knn, chi);
 }
 
 // 2BFS pseudo-diameter of the system (Sec. 6): ctl->pdiam and ctl->far_t.
