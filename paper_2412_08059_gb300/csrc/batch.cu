@@ -113,7 +113,7 @@ static __device__ bool sys_stage2(Team& t, const BatchSys& s, const BatchArgs& a
   if (whole && !sys_prep(t, s, a, red, false)) return false;
   bool done;
   if (sys_status(s) == 0 && !*reinterpret_cast<volatile int*>(&ctl->trivial) &&
-      !sys_cg64(t, s, whole ? 1 : 0, red, kNoBudget, false, &done))
+      !sys_cg64(t, s, whole ? 1 : 0, red, kNoBudget, false, &done, a.smem_bytes))
     return false;
   if (!team_sync(t)) return false;
   sys_finalize(t, s);
@@ -126,7 +126,7 @@ static __device__ bool sys_stage2(Team& t, const BatchSys& s, const BatchArgs& a
 // with both stages in one kernel, whatever else the kernel held moved the
 // FP64 stage by up to 50 %).
 template <int kPart>
-__global__ void __launch_bounds__(kBatchThreads, 1) k_batch(BatchArgs a) {
+__global__ void __launch_bounds__(kBatchThreads, kBatchPerSm) k_batch(BatchArgs a) {
   __shared__ TeamShared S;
   Team t;
   t.h = a.h;
@@ -172,15 +172,28 @@ int size_class(int n, int rows_per_block) {
 // iteration count that grows like sqrt(n) (CG on discretised operators).
 double work_of(int n, int nnz) { return ((double)nnz + 6.0 * n) * sqrt((double)n); }
 
-int team_smem(const void* kernel, int stage1) {
+int team_smem(const void* kernel) {
   if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTeamSmem) !=
       cudaSuccess)
     return -1;
-  return stage1 ? kTeamSmem : kScanSmem;
+  return kTeamSmem;
+}
+
+int team_grid(const void* kernel, int requested, int smem) {
+  int dev = 0, sms = 0, per_sm = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kBatchThreads, (size_t)smem) !=
+          cudaSuccess)
+    return 0;
+  if (per_sm > kBatchPerSm) per_sm = kBatchPerSm;  // fewer barrier arrivals
+  int full = sms * per_sm / kBatchPerSm;
+  if (full > kMaxGrid / kBatchPerSm) full = kMaxGrid / kBatchPerSm;
+  return requested > 0 && requested < full ? requested : full;
 }
 
 Plan make_plan(int nsys, const int* n, const double* work, int grid, int rows_per_block,
-               const int32_t* rows_sys) {
+               bool whole_blocks, const int32_t* rows_sys) {
   if (rows_per_block <= 0) rows_per_block = kRowsPerBlock;
   Plan P;
   std::vector<int> cls(nsys);
@@ -237,29 +250,24 @@ Plan make_plan(int nsys, const int* n, const double* work, int grid, int rows_pe
     teams[best] += 1;
     used += 1 << best;
   }
-  // Block layout: largest teams first; blocks left over become one-block
-  // teams of class 0.
-  P.team_of_block.assign(grid, 0);
-  P.rank_of_block.assign(grid, 0);
+  // Block layout: largest teams first; the class-0 teams and the blocks left
+  // over are teams of one launch block.
+  P.team_of_block.assign(grid * kBatchPerSm, 0);
+  P.rank_of_block.assign(grid * kBatchPerSm, 0);
   int b = 0;
-  for (int c = kTeamClasses - 1; c >= 0; --c) {
-    for (int k = 0; k < teams[c]; ++k) {
-      const int tm = (int)P.team_size.size();
-      P.team_size.push_back(1 << c);
-      P.team_class.push_back(c);
-      for (int r = 0; r < (1 << c); ++r) {
-        P.team_of_block[b] = tm;
-        P.rank_of_block[b] = r;
-        ++b;
-      }
+  auto add = [&](int c, int size) {  // one team of `size` launch blocks
+    const int tm = (int)P.team_size.size();
+    P.team_size.push_back(size);
+    P.team_class.push_back(c);
+    for (int r = 0; r < size; ++r) {
+      P.team_of_block[b] = tm;
+      P.rank_of_block[b] = r;
+      ++b;
     }
-  }
-  for (; b < grid; ++b) {
-    P.team_of_block[b] = (int)P.team_size.size();
-    P.rank_of_block[b] = 0;
-    P.team_size.push_back(1);
-    P.team_class.push_back(0);
-  }
+  };
+  for (int c = kTeamClasses - 1; c > 0; --c)
+    for (int k = 0; k < teams[c]; ++k) add(c, kBatchPerSm << c);
+  while (b < grid * kBatchPerSm) add(0, whole_blocks ? kBatchPerSm : 1);
   // Queues: class by class, largest work first.
   int base = 0;
   for (int c = 0; c < kTeamClasses; ++c) {
@@ -299,7 +307,7 @@ __global__ void k_pre_records(mpcg_result_t* res, int nsys) {
 }
 
 int batch_grid(int requested, int smem) {
-  return persistent_grid((const void*)k_batch<1>, kBatchThreads, requested, (size_t)smem);
+  return team_grid((const void*)k_batch<1>, requested, smem);
 }
 
 }  // namespace
@@ -334,11 +342,12 @@ extern "C" int32_t mpcg_batch_plan(int32_t nsys, const int32_t* n, const int32_t
   }
   int grid = grid_blocks;
   if (grid == 0) {  // the grid mpcg_solve_batch would launch with these options
-    const int smem = team_smem((const void*)k_batch<1>, 1);
+    const int smem = team_smem((const void*)k_batch<1>);
     grid = smem < 0 ? 0 : batch_grid(opts->grid_blocks, smem);
     if (grid <= 0) return MPCG_ERR_CUDA;
   }
-  const Plan P = make_plan(nsys, nv.data(), work.data(), grid, opts->team_rows, opts->team_rows_sys);
+  const Plan P = make_plan(nsys, nv.data(), work.data(), grid, opts->team_rows, opts->acc32 != 0,
+                           opts->team_rows_sys);
   for (int c = 0; c < kTeamClasses; ++c)
     for (int k = 0; k < P.qlen[c]; ++k) team_blocks_out[P.order[P.qbase[c] + k]] = 1 << c;
   return MPCG_OK;
@@ -366,14 +375,15 @@ extern "C" int32_t mpcg_solve_batch(int32_t nsys, const mpcg_csr_t* A, const dou
   }
   if (mpcg_batch_workspace_bytes(nsys, nv.data(), mv.data(), opts) > ws_bytes)
     return MPCG_ERR_WORKSPACE;
-  const int smem = team_smem((const void*)k_batch<1>, 1);
-  const int smem2 = team_smem((const void*)k_batch<2>, 0);
+  const int smem = team_smem((const void*)k_batch<1>);
+  const int smem2 = team_smem((const void*)k_batch<2>);
   if (smem < 0 || smem2 < 0) return MPCG_ERR_CUDA;
   const int grid = batch_grid(opts->grid_blocks, smem);
   if (grid <= 0) return MPCG_ERR_CUDA;
   std::vector<double> work(nsys);
   for (int32_t i = 0; i < nsys; ++i) work[i] = work_of(nv[i], mv[i]);
-  const Plan P = make_plan(nsys, nv.data(), work.data(), grid, opts->team_rows, opts->team_rows_sys);
+  const Plan P = make_plan(nsys, nv.data(), work.data(), grid, opts->team_rows, opts->acc32 != 0,
+                           opts->team_rows_sys);
 
   // Header blob: [BatchHdr | BatchSys[nsys] | order | team_of_block |
   // rank_of_block | team_size | team_class], then the systems' regions.
@@ -437,7 +447,7 @@ extern "C" int32_t mpcg_solve_batch(int32_t nsys, const mpcg_csr_t* A, const dou
   void* args[] = {&a};
   if (!opts->fp64_only) {  // set-up, features and the single-precision stage
     a.smem_bytes = smem;
-    if (cudaLaunchCooperativeKernel((const void*)k_batch<1>, dim3(grid), dim3(kBatchThreads), args,
+    if (cudaLaunchCooperativeKernel((const void*)k_batch<1>, dim3(grid * kBatchPerSm), dim3(kBatchThreads), args,
                                     (size_t)smem, st) != cudaSuccess)
       return MPCG_ERR_CUDA;
     // fresh barriers and queues for the second launch; an abort stays set
@@ -445,7 +455,7 @@ extern "C" int32_t mpcg_solve_batch(int32_t nsys, const mpcg_csr_t* A, const dou
   }
   a.smem_bytes = smem2;
   a.part = opts->fp64_only ? 0 : 2;
-  const cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_batch<2>, dim3(grid),
+  const cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_batch<2>, dim3(grid * kBatchPerSm),
                                                     dim3(kBatchThreads), args, (size_t)smem2, st);
   return e == cudaSuccess ? MPCG_OK : MPCG_ERR_CUDA;
 }
@@ -508,11 +518,11 @@ double simulate_launch(const Plan& P, const std::vector<SysTimes>& T, int stage)
 constexpr int kTuneMoves = 256;
 std::vector<int32_t> per_system_rows(const std::vector<SysTimes>& T, const std::vector<double>& order_key,
                                      const int* nv, const std::vector<double>& work, int grid,
-                                     const int* cand, int K, int best, bool two_launch) {
+                                     const int* cand, int K, int best, bool two_launch, bool whole_blocks) {
   const int nsys = (int)T.size();
   std::vector<int32_t> rows(nsys, cand[best]);
   auto span = [&]() {
-    const Plan P = make_plan(nsys, nv, work.data(), grid, cand[best], rows.data());
+    const Plan P = make_plan(nsys, nv, work.data(), grid, cand[best], whole_blocks, rows.data());
     return two_launch ? simulate_launch(P, T, 1) + simulate_launch(P, T, 2) : simulate_launch(P, T, 0);
   };
   std::vector<int> idx(nsys);
@@ -570,7 +580,7 @@ extern "C" int32_t mpcg_batch_tune(int32_t nsys, const mpcg_csr_t* A, const doub
     nv[i] = A[i].n;
     work[i] = work_of(A[i].n, A[i].nnz);
   }
-  const int smem = team_smem((const void*)k_batch<1>, 1);
+  const int smem = team_smem((const void*)k_batch<1>);
   const int grid = smem < 0 ? 0 : batch_grid(opts->grid_blocks, smem);
   int32_t status = grid > 0 ? MPCG_OK : MPCG_ERR_CUDA;
   int best = -1;
@@ -614,7 +624,8 @@ extern "C" int32_t mpcg_batch_tune(int32_t nsys, const mpcg_csr_t* A, const doub
     *team_rows_out = kCand[best];
     if (team_rows_sys_out) {
       std::vector<int32_t> rows = per_system_rows(T, key, nv.data(), work, grid, kCand,
-                                                  MPCG_TUNE_CANDIDATES, best, !opts->fp64_only);
+                                                  MPCG_TUNE_CANDIDATES, best, !opts->fp64_only,
+                                                  opts->acc32 != 0);
       mpcg_options_t o = *opts;
       o.team_rows = kCand[best];
       o.team_rows_sys = rows.data();

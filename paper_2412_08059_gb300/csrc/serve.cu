@@ -123,11 +123,13 @@ __device__ bool slot_advance(Team& t, const BatchSys& s, int* phase_p, const Bat
     if (!team_sync(t)) return false;
     ph = sys_status(s) != 0 ? kPhDone : (done ? kPhStage2Start : kPhStage1);
   }
-  if ((ph == kPhStage2Start || ph == kPhStage2) && part != 1) {
-    const bool resume = ph == kPhStage2;
-    if (!sys_cg64(t, s, a.o.fp64_only ? 1 : 0, red, budget, resume, &done)) return false;
-    if (!team_sync(t)) return false;
-    ph = (done || sys_status(s) != 0) ? kPhDone : kPhStage2;
+  if constexpr (!kStage) {  // the staged kernel never runs this stage (part 1)
+    if ((ph == kPhStage2Start || ph == kPhStage2) && part != 1) {
+      const bool resume = ph == kPhStage2;
+      if (!sys_cg64(t, s, a.o.fp64_only ? 1 : 0, red, budget, resume, &done, a.smem_bytes)) return false;
+      if (!team_sync(t)) return false;
+      ph = (done || sys_status(s) != 0) ? kPhDone : kPhStage2;
+    }
   }
   if (!team_sync(t)) return false;
   if (ph == kPhDone) sys_finalize(t, s);
@@ -145,7 +147,7 @@ __device__ bool slot_advance(Team& t, const BatchSys& s, int* phase_p, const Bat
 // iterations, but a step then costs both launches in sequence. The median
 // latency rose from 19 to 30 ms, so the split is off by default.
 template <int kPart>
-__global__ void __launch_bounds__(kBatchThreads, 1) k_serve(ServeArgs sa) {
+__global__ void __launch_bounds__(kBatchThreads, kBatchPerSm) k_serve(ServeArgs sa) {
   __shared__ TeamShared S;
   const BatchArgs& a = sa.b;
   Team t;
@@ -280,11 +282,10 @@ extern "C" int32_t mpcg_server_create(void* ws, size_t ws_bytes, int32_t max_slo
   if (opts->precond || opts->stop_true_residual)  // plain CG, recursive stop test in teams
     return MPCG_ERR_UNIMPLEMENTED;
   if (!ws || ((uintptr_t)ws & 255u) || ws_bytes <= fixed_bytes(max_slots)) return MPCG_ERR_WORKSPACE;
-  const int smem = team_smem((const void*)k_serve<1>, 1);
-  const int smem2 = team_smem((const void*)k_serve<2>, 1);
+  const int smem = team_smem((const void*)k_serve<1>);
+  const int smem2 = team_smem((const void*)k_serve<2>);
   if (smem < 0 || smem2 < 0) return MPCG_ERR_CUDA;
-  const int grid = persistent_grid((const void*)k_serve<1>, kBatchThreads, opts->grid_blocks,
-                                   (size_t)smem);
+  const int grid = team_grid((const void*)k_serve<1>, opts->grid_blocks, smem);
   if (grid <= 0) return MPCG_ERR_CUDA;
   mpcg_server* s = new mpcg_server();
   s->dev = (char*)ws;
@@ -381,7 +382,8 @@ extern "C" int32_t mpcg_batch_step(mpcg_server_t* s, int32_t max_iters, int32_t*
       s->fresh[i] = 0;
     }
   if (!ids.empty()) {
-    const Plan P = make_plan((int)ids.size(), nv.data(), work.data(), s->grid, s->o.team_rows);
+    const Plan P = make_plan((int)ids.size(), nv.data(), work.data(), s->grid, s->o.team_rows,
+                             s->o.acc32 != 0);
     char* m = s->mirror.data();
     BatchHdr* H = (BatchHdr*)m;
     memset(H, 0, sizeof(BatchHdr));
@@ -420,7 +422,7 @@ extern "C" int32_t mpcg_batch_step(mpcg_server_t* s, int32_t max_iters, int32_t*
       a.smem_bytes = s->smem;
       sa.b = a;
       sa.part = 1;
-      if (cudaLaunchCooperativeKernel((const void*)k_serve<1>, dim3(s->grid), dim3(kBatchThreads),
+      if (cudaLaunchCooperativeKernel((const void*)k_serve<1>, dim3(s->grid * kBatchPerSm), dim3(kBatchThreads),
                                       args, (size_t)s->smem, st) != cudaSuccess)
         return MPCG_ERR_CUDA;
       // fresh barriers and queues for the second launch; an abort stays set
@@ -430,7 +432,7 @@ extern "C" int32_t mpcg_batch_step(mpcg_server_t* s, int32_t max_iters, int32_t*
     a.smem_bytes = s->smem2;
     sa.b = a;
     sa.part = split ? 2 : 0;
-    if (cudaLaunchCooperativeKernel((const void*)k_serve<2>, dim3(s->grid), dim3(kBatchThreads),
+    if (cudaLaunchCooperativeKernel((const void*)k_serve<2>, dim3(s->grid * kBatchPerSm), dim3(kBatchThreads),
                                     args, (size_t)s->smem2, st) != cudaSuccess)
       return MPCG_ERR_CUDA;
     k_serve_abort<<<1, 32, 0, st>>>(a.h, a.sys, a.order, (int)ids.size(), s->phase_d);

@@ -1,9 +1,13 @@
 // team_core.cuh -- the whole method for one system, run by a team of blocks
 // of a persistent launch (the batched solve and the serving steps).
 //
-// A team is 1, 2, 4, ..., 128 blocks of one cooperative launch.  Teams
+// A team is 1, 2, 4, ..., 128 blocks of the plan, one plan block an SM.  The
+// launch has two blocks of 256 threads an SM: a plan block is two of them (a
+// plan of one block is two teams of one launch block each).  The two on an SM
+// belong to different teams, so one system's SpMV keeps the FP64 pipe busy
+// while the other waits in a sum, a barrier or a vector phase.  Teams
 // synchronise with a bounded barrier over their own blocks (a block barrier
-// for one-block teams).  Scalars are computed from team-wide sums that every
+// for teams of one).  Scalars are computed from team-wide sums that every
 // block of the team forms in the same order, so all blocks take the same
 // decisions.  The arithmetic is that of the single-system kernels: SpMV rows
 // summed in stored order with fused multiply-adds, float-float dot products
@@ -21,7 +25,8 @@
 
 namespace mpcg {
 
-constexpr int kBatchThreads = 512;
+constexpr int kBatchThreads = 256;
+constexpr int kBatchPerSm = 2;                 // launch blocks an SM (one plan block)
 constexpr int kBatchWarps = kBatchThreads / 32;
 constexpr int kTeamClasses = 8;                // team sizes 1, 2, 4, ..., 128 blocks
 constexpr int kRowsPerBlock = 16384;           // planner default: target rows per block of a team
@@ -32,10 +37,11 @@ constexpr int kStageWarpBytes = 2 * kSpmvStep * kSlice * kTeamFastW * (4 + 4);  
 constexpr int kBScanPer = 8;                   // slice widths per thread in the block scan
 constexpr int kBScanTile = kBatchThreads * kBScanPer;
 constexpr int kScanSmem = kBScanTile * 4 + kBatchThreads * 8;  // the scan's tile and partials
-// Dynamic shared memory of a team launch: the scan at set-up; with a
-// single-precision stage also the SpMV stages and the block-local 2BFS.
-// 128 KB plus the static part keeps the 132 KB shared-memory carve-out, so
-// the L1 cache keeps 124 KB of the 256 KB.
+// Dynamic shared memory of a team launch: the scan at set-up, the stages of
+// the single-precision SpMV, the block-local 2BFS, and r of the
+// double-precision stage, in turn.
+// 2 x 64 KB plus the static parts (under 1 KB each) keep the 132 KB
+// shared-memory carve-out, so the L1 cache keeps 124 KB of the 256 KB.
 constexpr int kTeamSmem = kBatchWarps * kStageWarpBytes;
 static_assert(kTeamSmem >= kScanSmem, "scan buffer");
 constexpr int kBlockBfsMaxN = 1 << 18;         // larger systems run the 2BFS over the whole team
@@ -80,8 +86,8 @@ struct BatchArgs {
 // Team context: barrier, block-level scratch, deterministic team sums.
 // ---------------------------------------------------------------------------------------
 struct TeamShared {
-  double dpart[16 * kBatchWarps];
-  double wsum[4];
+  double dpart[8 * kBatchWarps];
+  double wsum[2];
   float ffp[2 * kBatchWarps];
   double val[4];
   float fval[2];
@@ -153,22 +159,23 @@ struct TeamSyncFn {
 // alternates between two halves of the system's partials array.
 static __device__ bool team_sum_d(Team& t, double v, double* partials, int& red, double& out) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  // Folded in half in each warp, then by four warps (one per sub-partition
-  // of the SM): a dependent FP64 add takes 64 clocks of the warp's
-  // sub-partition and 19 of the SM, so 16 butterflies took 1,520 clocks.
+  // Folded to a quarter in each warp, the rest by two warps: a dependent FP64
+  // add takes 64 clocks of the warp's sub-partition and 19 of the SM, so whole
+  // butterflies in every warp would queue on the pipe.
   v += __shfl_xor_sync(0xffffffffu, v, 16);
-  if (lane < 16) t.S->dpart[16 * warp + lane] = v;
+  v += __shfl_xor_sync(0xffffffffu, v, 8);
+  if (lane < 8) t.S->dpart[8 * warp + lane] = v;
   __syncthreads();
-  if (warp < 4) {
-    double s = t.S->dpart[threadIdx.x] + t.S->dpart[threadIdx.x + 128];
-    s = warp_sum(s);
+  static_assert(8 * kBatchWarps == 64, "two warps sum the folded values");
+  if (warp < 2) {
+    const double s = warp_sum(t.S->dpart[threadIdx.x]);
     if (lane == 0) t.S->wsum[warp] = s;
   }
   __syncthreads();
   double* buf = partials + (red & 1) * kMaxGrid;
   ++red;
   if (threadIdx.x == 0) {
-    const double s = (t.S->wsum[0] + t.S->wsum[1]) + (t.S->wsum[2] + t.S->wsum[3]);
+    const double s = t.S->wsum[0] + t.S->wsum[1];
     if (t.size == 1) t.S->val[0] = s;
     else buf[t.rank] = s;
   }
@@ -192,16 +199,46 @@ static __device__ bool team_sum_ff(Team& t, FF v, double* partials, int& red, do
                                    bool f32) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   v = ff_warp_sum(v, f32);
+  double* buf = partials + (red & 1) * kMaxGrid;
+  ++red;
+  if (f32) {
+    // Option acc32: the float tree is part of the option's meaning (its
+    // results move with it), and its unit is the plan block: a butterfly over
+    // the 16 warps of every plan block, then the plan blocks by 32 lanes and
+    // a butterfly.  The warps' partials meet in global memory.
+    float* fb = reinterpret_cast<float*>(buf);
+    if (lane == 0) fb[t.rank * kBatchWarps + warp] = v.hi;
+    if (!team_sync(t)) return false;
+    if (threadIdx.x < 32) {
+      constexpr int kPlanWarps = kBatchWarps * kBatchPerSm;
+      float sf = 0.0f;
+      for (int r = 0; r < t.size / kBatchPerSm; ++r) {
+        float w = lane < kPlanWarps ? fb[r * kPlanWarps + lane] : 0.0f;
+        w = warp_sum_f(w);
+        if (lane == (r & 31)) sf = __fadd_rn(sf, w);
+      }
+      sf = warp_sum_f(sf);
+      if (threadIdx.x == 0) t.S->val[0] = (double)sf;
+    }
+    __syncthreads();
+    out = t.S->val[0];
+    __syncthreads();
+    return true;
+  }
   if (lane == 0) {
     t.S->ffp[2 * warp] = v.hi;
     t.S->ffp[2 * warp + 1] = v.lo;
   }
   __syncthreads();
-  double* buf = partials + (red & 1) * kMaxGrid;
-  ++red;
   if (threadIdx.x < 32) {
     FF s = lane < kBatchWarps ? FF{t.S->ffp[2 * lane], t.S->ffp[2 * lane + 1]} : FF{0.f, 0.f};
-    s = ff_warp_sum(s, f32);
+#pragma unroll
+    for (int o = kBatchWarps / 2; o > 0; o >>= 1) {
+      FF w;
+      w.hi = __shfl_xor_sync(0xffffffffu, s.hi, o);
+      w.lo = __shfl_xor_sync(0xffffffffu, s.lo, o);
+      s = ff_add(s, w, false);
+    }
     const double bs = (double)s.hi + (double)s.lo;
     if (threadIdx.x == 0) {
       if (t.size == 1) t.S->val[0] = bs;
@@ -212,14 +249,8 @@ static __device__ bool team_sum_ff(Team& t, FF v, double* partials, int& red, do
     if (!team_sync(t)) return false;
     if (threadIdx.x < 32) {
       double s = 0.0;
-      if (f32) {  // option acc32: the blocks' float partials summed in float
-        float sf = 0.0f;
-        for (int i = lane; i < t.size; i += 32) sf = __fadd_rn(sf, (float)buf[i]);
-        s = (double)warp_sum_f(sf);
-      } else {
-        for (int i = lane; i < t.size; i += 32) s += buf[i];
-        s = warp_sum(s);
-      }
+      for (int i = lane; i < t.size; i += 32) s += buf[i];
+      s = warp_sum(s);
       if (threadIdx.x == 0) t.S->val[0] = s;
     }
   }
@@ -358,18 +389,19 @@ static __device__ void block_scan_slices(const uint32_t* slice_w, int32_t* slice
 
 // Sliced arrays: entry k of row i at slice_ptr[s] + 32 k + (i mod 32); short
 // rows padded with value 0 and their own column, the rows past n that fill
-// the last slice with value 0 and column 0 (n - 1 in the 16-bit copy).
-// narrow: the launch's single-precision SpMV is the staged one, which also
-// gets a copy of the columns as 16-bit offsets from the row (Ctl::col16)
+// the last slice with value 0 and column 0 (n - 1 in the 16-bit copy).  A
+// copy of the columns as 16-bit offsets from the row (Ctl::col16) is written
 // when sys_rows found that every one fits and 32-bit columns were not asked
-// for.  Both copies hold the same entries in the same order.
+// for; both copies hold the same entries in the same order.  The
+// double-precision SpMV and the staged single-precision one read the 16-bit
+// copy; narrow: the launch's single-precision SpMV is the staged one.
 static __device__ void sys_fill(const Team& t, const BatchSys& s, bool narrow) {
   const int T = team_threads(t);
   const int32_t* rp = s.A.row_ptr;
-  const bool c16 = narrow && *reinterpret_cast<volatile int*>(&s.w.ctl->colwide) == 0;
+  const bool c16 = *reinterpret_cast<volatile int*>(&s.w.ctl->colwide) == 0;
   if (t.rank == 0 && threadIdx.x == 0) {
     s.w.ctl->col16 = c16 ? 1 : 0;
-    s.w.ctl->colbits = c16 ? 16 : 32;
+    s.w.ctl->colbits = c16 && narrow ? 16 : 32;
   }
   for (int i = team_tid(t); i < s.nslices * kSlice; i += T) {
     const int sl = i >> 5, lane = i & 31;
@@ -675,11 +707,13 @@ __device__ __forceinline__ void team_rows(const Team& t, const BatchSys& s, Ld L
 // over takes narrower steps.
 
 // One step of U slices: rows i[u] of widths w[u] (entries from p[u] on).
-template <int U, class Gather, class Pre, class Row>
+template <bool C16, int U, class Gather, class Pre, class Row>
 __device__ __forceinline__ void team_step64(const BatchSys& s, const int (&p)[U], const uint32_t (&wf)[U],
                                             const int (&i)[U], Gather G, Pre P, Row Rw) {
   const double* sv = s.w.sv64;
-  const int32_t* sc = s.w.scol;
+  const typename std::conditional<C16, int16_t, int32_t>::type* sc;
+  if constexpr (C16) sc = s.w.scol16;
+  else sc = s.w.scol;
   double a[U];
   decltype(P(0)) own[U];
   int wmin = 0x7fffffff, wmax = 0;
@@ -694,14 +728,14 @@ __device__ __forceinline__ void team_step64(const BatchSys& s, const int (&p)[U]
 #pragma unroll 2
   for (int k = 0; k < wmin; ++k) {
 #pragma unroll
-    for (int u = 0; u < U; ++u) a[u] = fma(sv[p[u] + kSlice * k], G(sc[p[u] + kSlice * k]), a[u]);
+    for (int u = 0; u < U; ++u) a[u] = fma(sv[p[u] + kSlice * k], G(col_at<C16>(sc[p[u] + kSlice * k], i[u])), a[u]);
   }
 #pragma unroll 1
   for (int k = wmin; k < wmax; ++k) {
 #pragma unroll
     for (int u = 0; u < U; ++u)
       if (k < (int)(wf[u] & ~kOverflowBit))
-        a[u] = fma(sv[p[u] + kSlice * k], G(sc[p[u] + kSlice * k]), a[u]);
+        a[u] = fma(sv[p[u] + kSlice * k], G(col_at<C16>(sc[p[u] + kSlice * k], i[u])), a[u]);
   }
 #pragma unroll
   for (int u = 0; u < U; ++u) {
@@ -711,13 +745,74 @@ __device__ __forceinline__ void team_step64(const BatchSys& s, const int (&p)[U]
   }
 }
 
+// Steps of two slices of the same width K, for as long as the warp's next two
+// slices have it: all entries and gathers of both rows in flight.  Up to K =
+// 5 the next step's columns are loaded while this step's sums run, so that a
+// step costs one round trip, its gathers; wider rows have no registers left
+// for that and take two.  (A pair of entries at a time took two round trips
+// each.)  j: the first slice's place among the warp's 32 whose metadata is at
+// hand (mwf, mp by lane), of cnt.
+template <bool C16, int K, class Gather, class Pre, class Row>
+__device__ __forceinline__ void team_run64(const BatchSys& s, uint32_t mwf, int mp, int base, int W, int cnt,
+                                           int& j, Gather G, Pre P, Row Rw) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  constexpr bool kAhead = K <= 5;
+  const typename std::conditional<C16, int16_t, int32_t>::type* sc;
+  if constexpr (C16) sc = s.w.scol16;
+  else sc = s.w.scol;
+  int p0, p1, c0[K], c1[K];
+  auto cols = [&]() {
+    p0 = __shfl_sync(full, mp, j) + lane;
+    p1 = __shfl_sync(full, mp, j + 1) + lane;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      c0[k] = sc[p0 + kSlice * k];
+      c1[k] = sc[p1 + kSlice * k];
+    }
+  };
+  if (kAhead) cols();
+  bool more;
+  do {
+    if (!kAhead) cols();
+    const int i0 = (base + j * W) * kSlice + lane, i1 = i0 + W * kSlice;
+    const double* va = s.w.sv64 + p0;
+    const double* vb = s.w.sv64 + p1;
+    double v0[K], v1[K], x0[K], x1[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      v0[k] = va[kSlice * k];
+      v1[k] = vb[kSlice * k];
+    }
+    auto own0 = P(i0);  // before the row callbacks: those store, and loads do not pass stores
+    auto own1 = P(i1);
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      x0[k] = G(C16 ? i0 + c0[k] : c0[k]);
+      x1[k] = G(C16 ? i1 + c1[k] : c1[k]);
+    }
+    j += 2;
+    more = j + 2 <= cnt && __shfl_sync(full, mwf, j & 31) == (uint32_t)K &&
+           __shfl_sync(full, mwf, (j + 1) & 31) == (uint32_t)K;
+    if (kAhead && more) cols();
+    double a0 = 0.0, a1 = 0.0;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      a0 = fma(v0[k], x0[k], a0);
+      a1 = fma(v1[k], x1[k], a1);
+    }
+    Rw(i0, a0, own0);
+    Rw(i1, a1, own1);
+  } while (more);
+}
+
 // SpMV over the team's slices: warp gw owns slices gw, gw + W, ...; lane l
 // owns row 32 s + l.  Rw(i, acc, own) receives row i's sum in stored order
 // (fused multiply-adds from zero, padding rows included) and the row's own
 // values that P(i) loaded before the gathers.  The metadata of 32 of the
 // warp's slices is loaded at once (one slice per lane).
-template <class Gather, class Pre, class Row>
-__device__ __forceinline__ void team_spmv64(const Team& t, const BatchSys& s, Gather G, Pre P, Row Rw) {
+template <bool C16, class Gather, class Pre, class Row>
+__device__ __forceinline__ void team_spmv64_t(const Team& t, const BatchSys& s, Gather G, Pre P, Row Rw) {
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int gw = team_warp(t), W = team_warps(t);
@@ -741,39 +836,86 @@ __device__ __forceinline__ void team_spmv64(const Team& t, const BatchSys& s, Ga
         p[u] = __shfl_sync(full, mp, j + u) + lane;
         i[u] = (base + (j + u) * W) * kSlice + lane;
       }
-      team_step64<U>(s, p, wf, i, G, P, Rw);
+      team_step64<C16, U>(s, p, wf, i, G, P, Rw);
       j += U;
     };
-    while (j + 4 <= cnt) step(std::integral_constant<int, 4>{});
-    if (j + 2 <= cnt) step(std::integral_constant<int, 2>{});
-    if (j < cnt) step(std::integral_constant<int, 1>{});
+    while (j < cnt) {  // warp-uniform
+      const uint32_t w0 = __shfl_sync(full, mwf, j), w1 = __shfl_sync(full, mwf, (j + 1) & 31);
+      if (j + 2 > cnt) {
+        step(std::integral_constant<int, 1>{});
+        break;
+      }
+      switch (w0 == w1 ? w0 : 0u) {  // (a width with the overflow flag is none of these)
+        case 5: team_run64<C16, 5>(s, mwf, mp, base, W, cnt, j, G, P, Rw); break;
+        case 6: team_run64<C16, 6>(s, mwf, mp, base, W, cnt, j, G, P, Rw); break;
+        case 7: team_run64<C16, 7>(s, mwf, mp, base, W, cnt, j, G, P, Rw); break;
+        default:
+          if (j + 4 <= cnt) step(std::integral_constant<int, 4>{});
+          else step(std::integral_constant<int, 2>{});
+      }
+    }
   }
 }
 
-// Row phases of the double-precision stage: as team_rows, four full slices a
-// step, then two, then one; the ragged last slice by itself.
+template <class Gather, class Pre, class Row>
+__device__ __forceinline__ void team_spmv64(const Team& t, const BatchSys& s, bool c16, Gather G, Pre P,
+                                            Row Rw) {
+  if (c16) team_spmv64_t<true>(t, s, G, P, Rw);
+  else team_spmv64_t<false>(t, s, G, P, Rw);
+}
+
+// Row phases of the double-precision stage: as team_rows, eight full slices a
+// step, then four, two and one; the ragged last slice by itself.
+// L(j, i) and O(j, i, v): j is the thread's row number, i the row.
 template <class Ld, class Op>
 __device__ __forceinline__ void team_rows64(const Team& t, const BatchSys& s, Ld L, Op O) {
   const int lane = threadIdx.x & 31;
   const int gw = team_warp(t), W = team_warps(t);
   const int fs = s.n >> 5;  // slices of 32 rows
-  int sl = gw;
+  int sl = gw, j = 0;
   auto step = [&](auto width) {
     constexpr int U = decltype(width)::value;
-    decltype(L(0)) v[U];
+    decltype(L(0, 0)) v[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u) v[u] = L((sl + u * W) * kSlice + lane);
+    for (int u = 0; u < U; ++u) v[u] = L(j + u, (sl + u * W) * kSlice + lane);
 #pragma unroll
-    for (int u = 0; u < U; ++u) O((sl + u * W) * kSlice + lane, v[u]);
+    for (int u = 0; u < U; ++u) O(j + u, (sl + u * W) * kSlice + lane, v[u]);
     sl += U * W;
+    j += U;
   };
-  while (sl + 3 * W < fs) step(std::integral_constant<int, 4>{});
+  while (sl + 7 * W < fs) step(std::integral_constant<int, 8>{});
+  if (sl + 3 * W < fs) step(std::integral_constant<int, 4>{});
   if (sl + W < fs) step(std::integral_constant<int, 2>{});
   if (sl < fs) step(std::integral_constant<int, 1>{});
   if (sl == fs) {
     const int i = sl * kSlice + lane;
-    if (i < s.n) O(i, L(i));
+    if (i < s.n) O(j, i, L(j, i));
   }
+}
+
+// r of the double-precision stage: the first `cap` rows of every thread live
+// in the launch's dynamic shared memory for the length of the stage (only
+// their own thread touches them), the others in the workspace.  At 16,384
+// rows a plan block r fits whole and a row's iteration moves 24 of 150 bytes
+// less through L2 and HBM, which bound the vector phases.
+struct TeamR {
+  double* g;
+  int cap;
+  __device__ __forceinline__ double* sm(int j) const {
+    return reinterpret_cast<double*>(team_dyn) + j * kBatchThreads + threadIdx.x;
+  }
+  __device__ __forceinline__ double ld(int j, int i) const { return j < cap ? *sm(j) : g[i]; }
+  __device__ __forceinline__ void st(int j, int i, double v) const {
+    if (j < cap) *sm(j) = v;
+    else g[i] = v;
+  }
+};
+
+// r from the workspace into shared memory (own rows).
+static __device__ void load_r(const Team& t, const BatchSys& s, const TeamR& R) {
+  team_rows64(
+      t, s, [&](int, int i) -> double { return R.g[i]; },
+      [&](int j, int, double v) { if (j < R.cap) *R.sm(j) = v; });
 }
 
 // Broadcast of thread 0's decision (and scalars) to the block.
@@ -955,7 +1097,7 @@ static __device__ bool sys_cg32(Team& t, const BatchSys& s, int mode, int& red, 
 // iteration state kept in the workspace (x, r, d) and the control block
 // (r^T r, iterations, restarts).  *done is false when the budget ended it.
 static __device__ bool sys_cg64(Team& t, const BatchSys& s, int from_zero, int& red, int budget,
-                         bool resume, bool* done) {
+                                bool resume, bool* done, int smem_bytes) {
   *done = true;
   Ctl* ctl = s.w.ctl;
   const int lane = threadIdx.x & 31;
@@ -969,6 +1111,8 @@ static __device__ bool sys_cg64(Team& t, const BatchSys& s, int from_zero, int& 
   double* d = s.w.d64;
   double* q = s.w.q64;
   const double* b = s.b;
+  const bool c16 = ctl->col16 != 0;
+  const TeamR R{r, smem_bytes / (int)(kBatchThreads * sizeof(double))};
   if (!resume) {
     if (lead0) ctl->t_s2 = globaltimer();
     for (int sl = gw; sl < s.nslices; sl += W) {
@@ -981,136 +1125,132 @@ static __device__ bool sys_cg64(Team& t, const BatchSys& s, int from_zero, int& 
   const int it_start = it;
   double rr = resume ? ctl->rr : 0.0, true_rel = NAN;
   const StopThr thr2 = stop_thr(eps2, bnorm, rel);  // used by thread 0
-  bool skip_restart = resume;
+  // One SpMV pass per round; what it is for:
+  //   kPRestart: r = b - A x, d = r, r^T r        (CG line 1 from x)
+  //   kPIterate: q = A d, d^T q; then the updates
+  //   kPTrueRes: ||b - A x||^2 at convergence; kPFinal: the same after the cap
+  enum { kPRestart = 0, kPIterate = 1, kPTrueRes = 2, kPFinal = 3 };
+  int kind = kPRestart;
+  bool head = resume;  // the next thing is the loop head (stop test), not a pass
+  if (resume) load_r(t, s, R);
   for (;;) {
-    // restart (CG line 1 from x): r = b - A x, d = r, r^T r
-    if (!skip_restart) {
-    double p = 0.0;
-    team_spmv64(
-        t, s, [&](int c) -> double { return x[c]; },
-        [&](int i) -> double { return i < n ? b[i] : 0.0; },
-        [&](int i, double acc, double bi) {
-          if (i < n) {
-            const double ri = bi - acc;
-            r[i] = ri;
-            d[i] = ri;
-            p = __fma_rn(ri, ri, p);
-          }
-        });
-    if (!team_sum_d(t, p, s.w.partials, red, rr)) return false;
-    }
-    skip_restart = false;
-    bool converged = false;
-    for (;;) {
-      int dec = kBGo;
-      if (lead) {
-        if (isnan(rr)) dec = kBNan;
-        else if (stop_pass(thr2, rr)) dec = kBStop;
-        else if (it >= max2) dec = kBCap;
-        else if (it - it_start >= budget) dec = kBSuspend;
-      }
-      dec = bcast_dec(t, dec);
-      if (dec == kBSuspend) {  // keep the iteration state for the next call
-        if (lead0) {
-          ctl->rr = rr;
-          ctl->n2 = it;
-          ctl->restarts = restarts;
-        }
-        *done = false;
-        return true;
-      }
-      if (dec == kBNan) {
-        failed = MPCG_ERR_NAN;
-        break;
-      }
-      if (dec == kBStop) {
-        converged = true;
-        break;
-      }
-      if (dec == kBCap) {
-        failed = MPCG_ERR_NOT_CONVERGED;
-        break;
-      }
-      // P1: q = A d, d^T q
-      double pq = 0.0;
+    if (!head) {
+      const int knd = kind;
+      const double* gv = knd == kPIterate ? d : x;
+      const double* ov = knd == kPIterate ? d : b;
+      double p = 0.0;
       team_spmv64(
-          t, s, [&](int c) -> double { return d[c]; },
-          [&](int i) -> double { return i < n ? d[i] : 0.0; },
-          [&](int i, double acc, double di) {
+          t, s, c16, [&](int c) -> double { return gv[c]; },
+          [&](int i) -> double { return i < n ? ov[i] : 0.0; },
+          [&](int i, double acc, double own) {
             if (i < n) {
-              q[i] = acc;
-              pq = __fma_rn(di, acc, pq);
+              if (knd == kPIterate) {
+                q[i] = acc;
+                p = __fma_rn(own, acc, p);
+              } else {
+                const double ri = own - acc;
+                if (knd == kPRestart) {
+                  r[i] = ri;
+                  d[i] = ri;
+                }
+                p = __fma_rn(ri, ri, p);
+              }
             }
           });
-      double dq;
-      if (!team_sum_d(t, pq, s.w.partials, red, dq)) return false;
-      dec = kBGo;
-      if (lead) {
-        if (!isfinite(dq)) dec = kBNan;
-        else if (!(dq > 0.0)) dec = kBBreakdown;
-        else t.S->val[2] = rr / dq;
+      double tot;
+      if (!team_sum_d(t, p, s.w.partials, red, tot)) return false;
+      if (kind == kPRestart) {
+        rr = tot;
+        load_r(t, s, R);
+      } else if (kind == kPIterate) {
+        int dec = kBGo;
+        if (lead) {
+          if (!isfinite(tot)) dec = kBNan;
+          else if (!(tot > 0.0)) dec = kBBreakdown;
+          else t.S->val[2] = rr / tot;
+        }
+        dec = bcast_dec(t, dec);
+        if (dec != kBGo) {
+          failed = dec == kBNan ? MPCG_ERR_NAN : MPCG_ERR_BREAKDOWN;
+          break;
+        }
+        const double alpha = t.S->val[2];
+        // r -= alpha q, r^T r (x += alpha d waits for the last phase, which reads d anyway)
+        double pr = 0.0;
+        team_rows64(
+            t, s, [&](int j, int i) -> double2 { return make_double2(q[i], R.ld(j, i)); },
+            [&](int j, int i, double2 v) {
+              const double ri = __fma_rn(-alpha, v.x, v.y);
+              R.st(j, i, ri);
+              pr = __fma_rn(ri, ri, pr);
+            });
+        double rrn;
+        if (!team_sum_d(t, pr, s.w.partials, red, rrn)) return false;
+        dec = kBGo;
+        if (lead) {
+          if (!isfinite(rrn)) dec = kBNan;
+          else t.S->val[3] = rrn / rr;
+        }
+        dec = bcast_dec(t, dec);
+        if (dec == kBNan) {
+          failed = MPCG_ERR_NAN;
+          break;
+        }
+        const double beta = t.S->val[3];
+        rr = rrn;
+        // x += alpha d, d = r + beta d
+        team_rows64(
+            t, s, [&](int j, int i) -> double3 { return make_double3(d[i], x[i], R.ld(j, i)); },
+            [&](int, int i, double3 v) {
+              x[i] = __fma_rn(alpha, v.x, v.y);
+              d[i] = __fma_rn(beta, v.x, v.z);
+            });
+        if (!team_sync(t)) return false;
+        ++it;
+      } else {
+        // true residual ||b - A x|| (also after the iteration cap)
+        int again = 0;  // 1: restart from x; 2: the last restart still missed eps2
+        if (lead) {
+          true_rel = bnorm > 0.0 ? sqrt(tot) / bnorm : sqrt(tot);
+          const double tm = rel ? true_rel : sqrt(tot);
+          if (kind == kPTrueRes && tm > eps2) again = restarts < max_restarts ? 1 : 2;
+        }
+        again = bcast_dec(t, again);
+        if (again == 2) failed = MPCG_ERR_NOT_CONVERGED;
+        if (again != 1) break;
+        ++restarts;
+        kind = kPRestart;
+        continue;
       }
-      dec = bcast_dec(t, dec);
-      if (dec != kBGo) {
-        failed = dec == kBNan ? MPCG_ERR_NAN : MPCG_ERR_BREAKDOWN;
-        break;
-      }
-      const double alpha = t.S->val[2];
-      // P2: x += alpha d, r -= alpha q, r^T r
-      double pr = 0.0;
-      team_rows64(
-          t, s, [&](int i) -> double4 { return make_double4(d[i], x[i], q[i], r[i]); },
-          [&](int i, double4 v) {
-            x[i] = __fma_rn(alpha, v.x, v.y);
-            const double ri = __fma_rn(-alpha, v.z, v.w);
-            r[i] = ri;
-            pr = __fma_rn(ri, ri, pr);
-          });
-      double rrn;
-      if (!team_sum_d(t, pr, s.w.partials, red, rrn)) return false;
-      dec = kBGo;
-      if (lead) {
-        if (!isfinite(rrn)) dec = kBNan;
-        else t.S->val[3] = rrn / rr;
-      }
-      dec = bcast_dec(t, dec);
-      if (dec == kBNan) {
-        failed = MPCG_ERR_NAN;
-        break;
-      }
-      const double beta = t.S->val[3];
-      rr = rrn;
-      // P3: d = r + beta d
-      team_rows64(
-          t, s, [&](int i) -> double2 { return make_double2(d[i], r[i]); },
-          [&](int i, double2 v) { d[i] = __fma_rn(beta, v.x, v.y); });
-      if (!team_sync(t)) return false;
-      ++it;
     }
-    if (failed && failed != MPCG_ERR_NOT_CONVERGED) break;
-    // true residual ||b - A x|| (also after the iteration cap)
-    double pt = 0.0;
-    team_spmv64(
-        t, s, [&](int c) -> double { return x[c]; },
-        [&](int i) -> double { return i < n ? b[i] : 0.0; },
-        [&](int i, double acc, double bi) {
-          if (i < n) {
-            const double ri = bi - acc;
-            pt = __fma_rn(ri, ri, pt);
-          }
-        });
-    double tot;
-    if (!team_sum_d(t, pt, s.w.partials, red, tot)) return false;
-    int again = 0;  // 1: restart from x; 2: the last restart still missed eps2
+    head = false;
+    // loop head: the stop test on the recursive residual
+    int dec = kBGo;
     if (lead) {
-      true_rel = bnorm > 0.0 ? sqrt(tot) / bnorm : sqrt(tot);
-      const double tm = rel ? true_rel : sqrt(tot);
-      if (converged && tm > eps2) again = restarts < max_restarts ? 1 : 2;
+      if (isnan(rr)) dec = kBNan;
+      else if (stop_pass(thr2, rr)) dec = kBStop;
+      else if (it >= max2) dec = kBCap;
+      else if (it - it_start >= budget) dec = kBSuspend;
     }
-    again = bcast_dec(t, again);
-    if (again == 2) failed = MPCG_ERR_NOT_CONVERGED;
-    if (again != 1) break;
-    ++restarts;
+    dec = bcast_dec(t, dec);
+    if (dec == kBSuspend) {  // keep the iteration state for the next call
+      team_rows64(
+          t, s, [&](int j, int i) -> double { return R.ld(j, i); },
+          [&](int j, int i, double v) { if (j < R.cap) r[i] = v; });
+      if (lead0) {
+        ctl->rr = rr;
+        ctl->n2 = it;
+        ctl->restarts = restarts;
+      }
+      *done = false;
+      return true;
+    }
+    if (dec == kBNan) {
+      failed = MPCG_ERR_NAN;
+      break;
+    }
+    if (dec == kBCap) failed = MPCG_ERR_NOT_CONVERGED;
+    kind = dec == kBStop ? kPTrueRes : dec == kBCap ? kPFinal : kPIterate;
   }
   if (lead0) {
     if (failed) set_status(ctl, failed);
@@ -1156,7 +1296,7 @@ static __device__ void sys_finalize(const Team& t, const BatchSys& s) {
   res->t_prep_ns = t0;
   res->t_stage2_ns = c->t_s2 ? c->t_s2 : res->t_fp32_ns;
   res->spmv_cols = c->colbits;
-  res->team_blocks = t.size;
+  res->team_blocks = (t.size + 1) / kBatchPerSm;  // plan blocks
 }
 
 // Status of the system as seen after a team barrier (identical in every block).
@@ -1226,19 +1366,24 @@ static __device__ bool team_pseudo_diameter(Team& t, const BatchSys& s, int smem
 // ---------------------------------------------------------------------------------------
 // Host: plan of a team launch (batch.cu).
 // ---------------------------------------------------------------------------------------
+// team_of_block, rank_of_block: by launch block; team_size: launch blocks.
 struct Plan {
   std::vector<int> team_of_block, rank_of_block, team_size, team_class, order;
   int qbase[kTeamClasses], qlen[kTeamClasses];
 };
-// Teams for a grid of `grid` blocks and the class queues of nsys systems of
+// Teams for a grid of `grid` plan blocks (kBatchPerSm * grid launch blocks) and the class queues of nsys systems of
 // n rows with estimated work `work` (largest first within a class); a system
 // goes to the smallest team with at most rows_per_block rows per block, or
 // rows_sys[i] when that array is given and its entry is positive.
+// whole_blocks (option acc32): teams of one plan block are two launch blocks
+// too, so that every team's sums have plan blocks as their unit.
 Plan make_plan(int nsys, const int* n, const double* work, int grid, int rows_per_block,
-               const int32_t* rows_sys = nullptr);
-// Dynamic shared memory of a team launch of `kernel`: kTeamSmem when it runs
-// a single-precision stage (stage1 != 0), else only the scan's kScanSmem.
-// Raises the kernel's limit on the current device; -1 on a CUDA error.
-int team_smem(const void* kernel, int stage1);
+               bool whole_blocks, const int32_t* rows_sys = nullptr);
+// Dynamic shared memory of a team launch of `kernel` (kTeamSmem); raises the
+// kernel's limit on the current device; -1 on a CUDA error.
+int team_smem(const void* kernel);
+// Plan blocks of a team launch of `kernel`: `requested` if positive and
+// smaller than one full wave, else the wave.
+int team_grid(const void* kernel, int requested, int smem);
 
 }  // namespace mpcg
