@@ -1,26 +1,31 @@
-// bfs_block.cuh -- the 2BFS pseudo-diameter of Sec. 6 run by ONE block, for
-// the teams of the batched and serving kernels.
+// bfs_block.cuh -- the 2BFS pseudo-diameter of Sec. 6 run by ONE block: for
+// the teams of the batched and serving kernels, and for small systems.
 //
-// The team version (bfs_core.cuh) pays, per BFS level, a team barrier and a
+// The group version (bfs_core.cuh) pays, per BFS level, a group barrier and a
 // chain of global-memory round trips (queue size, queue entry, row pointers,
 // columns, the claim on dist, the queue counter).  Here a single block runs
 // both searches with block barriers, visited BITMAPS (a claim is one atomicOr
-// on a bit) and frontier queues and counters in shared memory, which leaves
-// two dependent global loads per level (row pointers, then columns).  The
-// other blocks of the team wait at the next team barrier.
+// on a bit), one frontier queue for both searches (entries tagged with their
+// search) and its counters in shared memory.  What bounds a level is its
+// chain of dependent loads, so the neighbours are read from the sliced layout
+// whose slice offsets are kept in shared memory: one global round trip a
+// level instead of two (row pointers, then columns).
 //
-// Storage (given by the caller): the bitmaps of the two searches in shared
-// memory when they fit in half of the block's buffer, else in global scratch
-// of n words; the four queues (A and B, even and odd levels) take the rest of
-// the buffer, and entries past that capacity go to global queues of n
-// entries.  So any n works; shared memory only makes it faster.
+// Storage (given by the caller), by what fits the block's buffer:
+//   * both bitmaps and the slice offsets (3 n / 8 bytes): one round trip a level;
+//   * both bitmaps (n / 4 bytes): neighbours from the caller's CSR;
+//   * one bitmap: the searches run one after the other;
+//   * else bitmaps in global scratch.
+// The queues take the rest of the buffer, and entries past that capacity go
+// to global queues.  So any n works; shared memory only makes it faster.  A
+// matrix with a row longer than the sliced layout keeps uses the CSR.
 //
 // Readings are those of bfs_core.cuh: search A from vertex 0; t = smallest
 // vertex at the largest distance from 0 = smallest vertex of A's last
 // non-empty level; l~ = last non-empty level of the BFS from t; the search
-// from t is started speculatively from n - 1 with A.  Unlike the team
+// from t is started speculatively from n - 1 with A.  Unlike the group
 // version, B is dropped as soon as A ends with t != n - 1.  Only connected
-// graphs are handled; otherwise the caller runs the team version.
+// graphs are handled; otherwise the caller runs the group version.
 #pragma once
 #include <limits.h>
 
@@ -28,61 +33,83 @@
 
 namespace mpcg {
 
-struct BlockBfs {
+// The graph as the block search reads it.
+struct BlockGraph {
   const int32_t* rp;
   const int32_t* col;
-  int n;
-  uint32_t* vis[2];  // visited bitmaps of searches A and B, (n + 31) / 32 words each
-  int32_t* qs[4];    // shared queue heads: A even, A odd, B even, B odd (cap entries)
-  int32_t* qg[4];    // global queues of n entries (entries at index >= cap)
-  int cap;
-  int* cnt;          // shared: A sizes [0..2] and B sizes [3..5] by level mod 3, [6] scratch,
-                     // [7] set when the search is to end
-  Ctl* poll;         // when set: the search ends on an error or the caller's cancel word
+  const int32_t* slice_ptr;
+  const uint32_t* slice_w;
+  const void* scol;  // sliced columns: int16 offsets from the row (c16) or int32
+  int n, c16;
 };
 
-// Partition of a block's shared buffer (bytes, 16-aligned base) for n
-// vertices.  vis_global: scratch of >= 2 * words words for the bitmaps when
-// they do not fit.
-static __device__ BlockBfs block_bfs_layout(const int32_t* rp, const int32_t* col, int n,
-                                            unsigned char* smem, int smem_bytes,
-                                            uint32_t* vis_global, int32_t* const gq[4]) {
+struct BlockBfs {
+  BlockGraph g;
+  uint32_t* vis[2];    // visited bitmaps of searches A and B, (n + 31) / 32 words each
+  const int32_t* sp;   // slice offsets in shared memory, or null: the CSR is read
+  int32_t* qs[2];      // shared queue heads: even and odd levels (cap entries)
+  int32_t* qg[4];      // global queues of n entries: even levels 0 and 1, odd levels 2 and 3
+  int cap;
+  bool dual;           // both searches at once (two bitmaps)
+  int* cnt;            // shared: queue sizes [0..2] and B's part of them [3..5] by level
+                       // mod 3, [6] scratch, [7] set when the search is to end
+  Ctl* poll;           // when set: the search ends on an error or the caller's cancel word
+};
+
+// Partition of a block's shared buffer (bytes, 16-aligned base).  vis_global:
+// scratch of 2 * words words for the bitmaps when they do not fit.  Every
+// thread of the block calls it.
+static __device__ BlockBfs block_bfs_layout(const BlockGraph& g, unsigned char* smem, int smem_bytes,
+                                            uint32_t* vis_global, int32_t* const gq[4], Ctl* poll) {
   BlockBfs b;
-  b.rp = rp;
-  b.col = col;
-  b.n = n;
-  b.poll = nullptr;
-  const int words = (n + 31) >> 5;
+  b.g = g;
+  b.poll = poll;
+  const int words = (g.n + 31) >> 5;
   b.cnt = reinterpret_cast<int*>(smem);
   unsigned char* p = smem + 64;
   int left = smem_bytes - 64;
-  const long long vis_bytes = 2ll * words * 4;
-  if (vis_bytes <= left / 2) {
+  const int one = (words * 4 + 15) & ~15;  // a bitmap; the slice offsets take 16 more at most
+  const int qmin = 4096;                   // bytes the queues get at least
+  b.sp = nullptr;
+  b.dual = true;
+  if (2ll * one + qmin <= left) {
     b.vis[0] = reinterpret_cast<uint32_t*>(p);
-    b.vis[1] = b.vis[0] + words;
-    const int used = (int)((vis_bytes + 15) & ~15ll);
-    p += used;
-    left -= used;
+    b.vis[1] = reinterpret_cast<uint32_t*>(p + one);
+    p += 2 * one;
+    left -= 2 * one;
+    if (one + 16 + qmin <= left) {
+      int32_t* sp = reinterpret_cast<int32_t*>(p);
+      int over = 0;
+      for (int i = threadIdx.x; i <= words; i += blockDim.x) {
+        sp[i] = g.slice_ptr[i];
+        if (i < words && (g.slice_w[i] & kOverflowBit)) over = 1;
+      }
+      if (!__syncthreads_or(over)) {
+        b.sp = sp;
+        p += one + 16;
+        left -= one + 16;
+      }
+    }
+  } else if (one + qmin <= left) {
+    b.vis[0] = b.vis[1] = reinterpret_cast<uint32_t*>(p);
+    p += one;
+    left -= one;
+    b.dual = false;
   } else {
     b.vis[0] = vis_global;
     b.vis[1] = vis_global + words;
   }
-  b.cap = left / 16;
-  if (b.cap > n) b.cap = n;
-  for (int k = 0; k < 4; ++k) {
-    b.qs[k] = reinterpret_cast<int32_t*>(p) + k * b.cap;
-    b.qg[k] = gq[k];
-  }
+  b.cap = left / 8;
+  for (int k = 0; k < 2; ++k) b.qs[k] = reinterpret_cast<int32_t*>(p) + k * b.cap;
+  for (int k = 0; k < 4; ++k) b.qg[k] = gq[k];
   return b;
 }
 
-static __device__ __forceinline__ int bq_get(const BlockBfs& b, int q, int i) {
-  return i < b.cap ? b.qs[q][i] : b.qg[q][i];
-}
-
-static __device__ __forceinline__ void bq_put(const BlockBfs& b, int q, int i, int v) {
-  if (i < b.cap) b.qs[q][i] = v;
-  else b.qg[q][i] = v;
+// Entry i of the queue of a level's parity q.
+static __device__ __forceinline__ int32_t* bq_at(const BlockBfs& b, int q, int i) {
+  if (i < b.cap) return b.qs[q] + i;
+  i -= b.cap;
+  return i < b.g.n ? b.qg[2 * q] + i : b.qg[2 * q + 1] + (i - b.g.n);
 }
 
 // Claim vertex w in a visited bitmap: true for exactly one caller.
@@ -92,12 +119,16 @@ static __device__ __forceinline__ bool bvis_claim(uint32_t* bm, int w) {
   return (atomicOr(&bm[w >> 5], bit) & bit) == 0u;
 }
 
-// Smallest entry of queue q (first `size` entries), in every thread.
+// Smallest vertex of search A in the queue of parity q (first `size`
+// entries), in every thread.
 static __device__ int block_queue_min(const BlockBfs& b, int q, int size) {
   if (threadIdx.x == 0) b.cnt[6] = INT_MAX;
   __syncthreads();
   int m = INT_MAX;
-  for (int i = threadIdx.x; i < size; i += blockDim.x) m = min(m, bq_get(b, q, i));
+  for (int i = threadIdx.x; i < size; i += blockDim.x) {
+    const int e = *bq_at(b, q, i);
+    if (!(e & 1)) m = min(m, e >> 1);
+  }
   m = __reduce_min_sync(0xffffffffu, m);
   if ((threadIdx.x & 31) == 0 && m != INT_MAX) atomicMin(&b.cnt[6], m);
   __syncthreads();
@@ -109,15 +140,20 @@ static __device__ int block_queue_min(const BlockBfs& b, int q, int size) {
 struct BlockBfsOut {
   int la, lb;        // last non-empty level of A and of B (B: valid if !dropped)
   int t;             // smallest vertex of A's last level
-  long long reached; // vertices reached by A
+  long long reached; // vertices reached by A; -1 if the search was stopped
   bool dropped;      // B was dropped because t != srcB
 };
 
 // Searches A from srcA and (srcB >= 0) B from srcB, level-synchronous, in
-// the calling block; every thread of the block calls it.
-static __device__ BlockBfsOut block_bfs2(const BlockBfs& b, int srcA, int srcB) {
+// the calling block (the sliced columns may have been written in this launch,
+// so they are read past the read-only cache); every thread of the block calls it.  kSliced: neighbours
+// from the sliced layout (b.sp), kC16: as int16 offsets.
+template <bool kSliced, bool kC16>
+static __device__ BlockBfsOut block_bfs2_t(const BlockBfs& b, int srcA, int srcB) {
   const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31, wbase = tid - lane;
-  const int words = (b.n + 31) >> 5;
+  const int words = (b.g.n + 31) >> 5;
+  const int16_t* s16 = reinterpret_cast<const int16_t*>(b.g.scol);
+  const int32_t* s32 = reinterpret_cast<const int32_t*>(b.g.scol);
   for (int i = tid; i < words; i += T) {
     b.vis[0][i] = 0u;
     b.vis[1][i] = 0u;
@@ -126,30 +162,32 @@ static __device__ BlockBfsOut block_bfs2(const BlockBfs& b, int srcA, int srcB) 
   __syncthreads();
   if (tid == 0) {
     b.vis[0][srcA >> 5] |= 1u << (srcA & 31);
-    bq_put(b, 0, 0, srcA);
+    *bq_at(b, 0, 0) = srcA << 1;
     b.cnt[0] = 1;
     if (srcB >= 0) {
       b.vis[1][srcB >> 5] |= 1u << (srcB & 31);
-      bq_put(b, 2, 0, srcB);
+      *bq_at(b, 0, 1) = (srcB << 1) | 1;
+      b.cnt[0] = 2;
       b.cnt[3] = 1;
     }
   }
   __syncthreads();
   BlockBfsOut o{0, 0, -1, 0, false};
   bool liveB = srcB >= 0, doneA = false;
-  int lastsa = 1;
+  int lastsize = 0;  // entries of the previous level's queue
   for (int level = 0;; ++level) {
-    const int sa = *reinterpret_cast<volatile int*>(&b.cnt[level % 3]);
-    int sb = liveB ? *reinterpret_cast<volatile int*>(&b.cnt[3 + level % 3]) : 0;
+    const int size = *reinterpret_cast<volatile int*>(&b.cnt[level % 3]);
+    int sb = *reinterpret_cast<volatile int*>(&b.cnt[3 + level % 3]);
+    const int sa = size - sb;
     if (sa == 0 && !doneA) {  // A has ended: its last level is known
       doneA = true;
-      o.t = block_queue_min(b, o.la & 1, lastsa);
+      o.t = block_queue_min(b, (level & 1) ^ 1, lastsize);
       if (liveB && o.t != srcB) {
         liveB = false;
         o.dropped = true;
-        sb = 0;
       }
     }
+    if (!liveB) sb = 0;
     if (sa == 0 && sb == 0) break;
     if (b.poll && (level & 255) == 255) {
       if (tid == 0 && (volatile_status(b.poll) != 0 || poll_cancel(b.poll))) b.cnt[7] = 1;
@@ -160,37 +198,43 @@ static __device__ BlockBfsOut block_bfs2(const BlockBfs& b, int srcA, int srcB) 
       }
     }
     o.reached += sa;
-    if (sa) {
-      o.la = level;
-      lastsa = sa;
-    }
+    if (sa) o.la = level;
     if (sb) o.lb = level;
+    lastsize = size;
     if (tid == 0) {
       b.cnt[(level + 2) % 3] = 0;
       b.cnt[3 + (level + 2) % 3] = 0;
     }
-    const int qa = level & 1, qb = 2 + (level & 1);
-    int* cntA = &b.cnt[(level + 1) % 3];
+    const int q = level & 1;
+    int* cnt = &b.cnt[(level + 1) % 3];
     int* cntB = &b.cnt[3 + (level + 1) % 3];
-    const int total = sa + sb;
     // Two frontier vertices per lane per round, so that their loads overlap.
-    for (int base = wbase; base < total; base += 2 * T) {  // warp-uniform bound
-      int u[2], e0[2], deg[2];
-      bool isB[2];
+    for (int base = wbase; base < size; base += 2 * T) {  // warp-uniform bound
+      int u[2], e0[2], deg[2], tag[2];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int idx = base + h * T + lane;
-        isB[h] = idx >= sa;
         u[h] = -1;
-        if (idx < total) u[h] = isB[h] ? bq_get(b, qb, idx - sa) : bq_get(b, qa, idx);
+        e0[h] = 0;
+        deg[h] = 0;
+        tag[h] = 0;
+        if (idx < size) {
+          const int e = *bq_at(b, q, idx);
+          tag[h] = e & 1;
+          if (!tag[h] || liveB) u[h] = e >> 1;
+        }
       }
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        e0[h] = 0;
-        deg[h] = 0;
         if (u[h] >= 0) {
-          e0[h] = __ldg(&b.rp[u[h]]);
-          deg[h] = __ldg(&b.rp[u[h] + 1]) - e0[h];
+          if (kSliced) {
+            const int s = u[h] >> 5;
+            e0[h] = b.sp[s] + (u[h] & 31);
+            deg[h] = (b.sp[s + 1] - b.sp[s]) >> 5;  // the slice's width: padding entries name the row itself
+          } else {
+            e0[h] = __ldg(&b.g.rp[u[h]]);
+            deg[h] = __ldg(&b.g.rp[u[h] + 1]) - e0[h];
+          }
         }
       }
       const int maxdeg = __reduce_max_sync(0xffffffffu, max(deg[0], deg[1]));
@@ -199,49 +243,43 @@ static __device__ BlockBfsOut block_bfs2(const BlockBfs& b, int srcA, int srcB) 
 #pragma unroll
         for (int h = 0; h < 2; ++h)
 #pragma unroll
-          for (int j = 0; j < 8; ++j) w[h][j] = (k0 + j < deg[h]) ? __ldg(&b.col[e0[h] + k0 + j]) : -1;
-        bool push[2][8];
-        int mA = 0, mB = 0;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          uint32_t* vis = b.vis[isB[h] ? 1 : 0];
-#pragma unroll
           for (int j = 0; j < 8; ++j) {
-            push[h][j] = w[h][j] >= 0 && bvis_claim(vis, w[h][j]);
-            if (push[h][j]) {
-              if (isB[h]) ++mB;
-              else ++mA;
+            w[h][j] = -1;
+            if (k0 + j < deg[h]) {
+              if (!kSliced) w[h][j] = __ldg(&b.g.col[e0[h] + k0 + j]);
+              else if (kC16) w[h][j] = u[h] + (int)__ldcg(&s16[e0[h] + kSlice * (k0 + j)]);
+              else w[h][j] = __ldcg(&s32[e0[h] + kSlice * (k0 + j)]);
             }
           }
+        unsigned push[2] = {0u, 0u};
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          uint32_t* vis = b.vis[tag[h]];
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            if (w[h][j] >= 0 && bvis_claim(vis, w[h][j])) push[h] |= 1u << j;
         }
-        int incA = mA, incB = mB;
+        const int m0 = __popc(push[0]), m1 = __popc(push[1]);
+        int inc = m0 + m1;
 #pragma unroll
         for (int o2 = 1; o2 < 32; o2 <<= 1) {
-          const int ta = __shfl_up_sync(0xffffffffu, incA, o2);
-          const int tb = __shfl_up_sync(0xffffffffu, incB, o2);
-          if (lane >= o2) {
-            incA += ta;
-            incB += tb;
-          }
+          const int t = __shfl_up_sync(0xffffffffu, inc, o2);
+          if (lane >= o2) inc += t;
         }
-        const int totA = __shfl_sync(0xffffffffu, incA, 31);
-        const int totB = __shfl_sync(0xffffffffu, incB, 31);
-        int bA = 0, bB = 0;
+        const int tot = __shfl_sync(0xffffffffu, inc, 31);
+        if (tot == 0) continue;  // warp-uniform
+        const int totB = __reduce_add_sync(0xffffffffu, (tag[0] ? m0 : 0) + (tag[1] ? m1 : 0));
+        int at = 0;
         if (lane == 0) {
-          if (totA > 0) bA = atomicAdd(cntA, totA);
-          if (totB > 0) bB = atomicAdd(cntB, totB);
+          at = atomicAdd(cnt, tot);
+          if (totB) atomicAdd(cntB, totB);
         }
-        int posA = __shfl_sync(0xffffffffu, bA, 0) + incA - mA;
-        int posB = __shfl_sync(0xffffffffu, bB, 0) + incB - mB;
+        int pos = __shfl_sync(0xffffffffu, at, 0) + inc - m0 - m1;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            if (push[h][j]) {
-              if (isB[h]) bq_put(b, qb ^ 1, posB++, w[h][j]);
-              else bq_put(b, qa ^ 1, posA++, w[h][j]);
-            }
-          }
+          for (int j = 0; j < 8; ++j)
+            if ((push[h] >> j) & 1u) *bq_at(b, q ^ 1, pos++) = (w[h][j] << 1) | tag[h];
         }
       }
     }
@@ -249,21 +287,32 @@ static __device__ BlockBfsOut block_bfs2(const BlockBfs& b, int srcA, int srcB) 
   }
   return o;  // unless stopped, the loop ends only after A has ended, so o.t is set
 }
+static __device__ BlockBfsOut block_bfs2(const BlockBfs& b, int srcA, int srcB) {
+  if (!b.sp) return block_bfs2_t<false, false>(b, srcA, srcB);
+  if (b.g.c16) return block_bfs2_t<true, true>(b, srcA, srcB);
+  return block_bfs2_t<true, false>(b, srcA, srcB);
+}
 
 // 2BFS of a connected graph in one block.  Returns false (in every thread)
-// if vertex 0 does not reach all n vertices; then nothing is written.
+// if vertex 0 does not reach all n vertices, or the search was stopped; then
+// nothing is written.
 static __device__ bool block_pseudo_diameter(const BlockBfs& b, int* pdiam, int* t_out) {
-  if (b.n <= 0) return false;
-  const int guess = b.n - 1;
-  const BlockBfsOut o = block_bfs2(b, 0, guess);
-  if (o.reached != b.n) return false;
-  *t_out = o.t;
-  if (o.t == guess && !o.dropped) {
-    *pdiam = o.lb;
-  } else {
-    const BlockBfsOut o2 = block_bfs2(b, o.t, -1);
-    if (o2.reached != b.n) return false;  // stopped
-    *pdiam = o2.la;
+  if (b.g.n <= 0) return false;
+  const int guess = b.dual ? b.g.n - 1 : -1;
+  int src = 0;
+  for (int pass = 0; pass < 2; ++pass) {
+    const BlockBfsOut o = block_bfs2(b, src, pass == 0 ? guess : -1);
+    if (o.reached != b.g.n) return false;
+    if (pass == 1) {
+      *pdiam = o.la;
+    } else {
+      *t_out = o.t;
+      if (guess >= 0 && o.t == guess && !o.dropped) {
+        *pdiam = o.lb;
+        break;
+      }
+      src = o.t;
+    }
   }
   return true;
 }

@@ -347,9 +347,8 @@ struct BlockSync {
 __device__ __noinline__ void cl_bfs(const ClusterArgs& a, unsigned char* smem) {
   Ctl* ctl = a.ctl;
   int32_t* const gq[4] = {a.g.fq0, a.g.fq1, a.g.fq2, a.g.fq3};
-  BlockBfs b = block_bfs_layout(a.rp, a.col, a.n, smem, a.smem_bytes,
-                                reinterpret_cast<uint32_t*>(a.g.ckey), gq);
-  b.poll = ctl;
+  const BlockGraph g{a.rp, a.col, a.slice_ptr, a.slice_w, a.scol, a.n, ctl->col16};
+  const BlockBfs b = block_bfs_layout(g, smem, a.smem_bytes, reinterpret_cast<uint32_t*>(a.g.ckey), gq, ctl);
   int pd = 0, tv = 0;
   bool ok = block_pseudo_diameter(b, &pd, &tv);
   __syncthreads();

@@ -1324,8 +1324,10 @@ static __device__ __noinline__ void block_bfs_system(const BatchSys* sp, int sme
   const BatchSys& s = *sp;
   Ctl* ctl = s.w.ctl;
   int32_t* const gq[4] = {s.w.fq0, s.w.fq1, s.w.fq2, s.w.fq3};
-  const BlockBfs b = block_bfs_layout(s.A.row_ptr, s.A.col, s.n, team_dyn, smem_bytes,
-                                      reinterpret_cast<uint32_t*>(s.w.ckey), gq);
+  const bool c16 = ctl->col16 != 0;
+  const BlockGraph g{s.A.row_ptr, s.A.col, s.w.slice_ptr, s.w.slice_w,
+                     c16 ? (const void*)s.w.scol16 : (const void*)s.w.scol, s.n, c16 ? 1 : 0};
+  const BlockBfs b = block_bfs_layout(g, team_dyn, smem_bytes, reinterpret_cast<uint32_t*>(s.w.ckey), gq, nullptr);
   int pd = 0, tv = 0;
   const bool ok = block_pseudo_diameter(b, &pd, &tv);
   if (threadIdx.x == 0) {
