@@ -148,7 +148,7 @@ int32_t mpcg_features(const mpcg_csr_t* A, const double* b, const mpcg_options_t
   if ((e = launch_init(L, *opts, 0)) != cudaSuccess) return cuda_status(e);
   if ((e = launch_prep(L, b)) != cudaSuccess) return cuda_status(e);
   if (L.precond && (e = launch_jacobi(L)) != cudaSuccess) return cuda_status(e);
-  if ((e = launch_pseudo_diameter(L, kSlotPd)) != cudaSuccess) return cuda_status(e);
+  if ((e = launch_pseudo_diameter(L, kSlotPd, opts->bfs_starts)) != cudaSuccess) return cuda_status(e);
   if ((e = launch_cg32(L, kCgK0, kSlotCgK0)) != cudaSuccess) return cuda_status(e);
   return cuda_status(launch_finalize(L, nullptr, out));
 }
@@ -199,7 +199,7 @@ int32_t mpcg_solve(const mpcg_csr_t* A, const double* b, double* x, const mpcg_s
     // Algorithm II with Jacobi PCG or with the stop test on b - A x, its
     // steps as separate launches in the paper's order: 2BFS, k0 iterations
     // (v), kNN, stage 1 from iterate k0
-    if ((e = launch_pseudo_diameter(L, kSlotPd)) != cudaSuccess) return cuda_status(e);
+    if ((e = launch_pseudo_diameter(L, kSlotPd, opts->bfs_starts)) != cudaSuccess) return cuda_status(e);
     if ((e = launch_cg32(L, kCgK0, kSlotCgK0)) != cudaSuccess) return cuda_status(e);
     if ((e = launch_knn(L.st, nullptr, *sample, *opts, L.ws.ctl, nullptr, nullptr)) != cudaSuccess)
       return cuda_status(e);
@@ -256,7 +256,7 @@ int32_t mpcg_pseudo_diameter(const mpcg_csr_t* A, int32_t* out, void* ws, size_t
   cudaError_t e;
   if ((e = launch_init(L, o, 0)) != cudaSuccess) return cuda_status(e);
   if ((e = launch_prep(L, nullptr)) != cudaSuccess) return cuda_status(e);
-  if ((e = launch_pseudo_diameter(L, kSlotPd)) != cudaSuccess) return cuda_status(e);
+  if ((e = launch_pseudo_diameter(L, kSlotPd, o.bfs_starts)) != cudaSuccess) return cuda_status(e);
   return cuda_status(launch_copy_pdiam(L, out));
 }
 

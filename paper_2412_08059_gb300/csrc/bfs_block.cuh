@@ -45,15 +45,17 @@ struct BlockGraph {
 
 struct BlockBfs {
   BlockGraph g;
-  uint32_t* vis[2];    // visited bitmaps of searches A and B, (n + 31) / 32 words each
+  uint32_t *visA, *visB;  // visited bitmaps of searches A and B, (n + 31) / 32 words each
   const int32_t* sp;   // slice offsets in shared memory, or null: the CSR is read
-  int32_t* qs[2];      // shared queue heads: even and odd levels (cap entries)
-  int32_t* qg[4];      // global queues of n entries: even levels 0 and 1, odd levels 2 and 3
+  int32_t* qs;         // shared queue heads: even levels, then odd levels (cap entries each)
+  int32_t *qg0, *qg1, *qg2, *qg3;  // global queues of n entries: even levels 0 and 1, odd 2 and 3
   int cap;
   bool dual;           // both searches at once (two bitmaps)
   int* cnt;            // shared: queue sizes [0..2] and B's part of them [3..5] by level
                        // mod 3, [6] scratch, [7] set when the search is to end
   Ctl* poll;           // when set: the search ends on an error or the caller's cancel word
+  int wide, grow;      // wide set: the search ends at a frontier of more than wide entries,
+                       // with grow also at one of more than 128 + grow * level
 };
 
 // Partition of a block's shared buffer (bytes, 16-aligned base).  vis_global:
@@ -64,6 +66,8 @@ static __device__ BlockBfs block_bfs_layout(const BlockGraph& g, unsigned char* 
   BlockBfs b;
   b.g = g;
   b.poll = poll;
+  b.wide = 0;
+  b.grow = 0;
   const int words = (g.n + 31) >> 5;
   b.cnt = reinterpret_cast<int*>(smem);
   unsigned char* p = smem + 64;
@@ -73,8 +77,8 @@ static __device__ BlockBfs block_bfs_layout(const BlockGraph& g, unsigned char* 
   b.sp = nullptr;
   b.dual = true;
   if (2ll * one + qmin <= left) {
-    b.vis[0] = reinterpret_cast<uint32_t*>(p);
-    b.vis[1] = reinterpret_cast<uint32_t*>(p + one);
+    b.visA = reinterpret_cast<uint32_t*>(p);
+    b.visB = reinterpret_cast<uint32_t*>(p + one);
     p += 2 * one;
     left -= 2 * one;
     if (one + 16 + qmin <= left) {
@@ -91,32 +95,29 @@ static __device__ BlockBfs block_bfs_layout(const BlockGraph& g, unsigned char* 
       }
     }
   } else if (one + qmin <= left) {
-    b.vis[0] = b.vis[1] = reinterpret_cast<uint32_t*>(p);
+    b.visA = b.visB = reinterpret_cast<uint32_t*>(p);
     p += one;
     left -= one;
     b.dual = false;
   } else {
-    b.vis[0] = vis_global;
-    b.vis[1] = vis_global + words;
+    b.visA = vis_global;
+    b.visB = vis_global + words;
   }
   b.cap = left / 8;
-  for (int k = 0; k < 2; ++k) b.qs[k] = reinterpret_cast<int32_t*>(p) + k * b.cap;
-  for (int k = 0; k < 4; ++k) b.qg[k] = gq[k];
+  b.qs = reinterpret_cast<int32_t*>(p);
+  b.qg0 = gq[0];
+  b.qg1 = gq[1];
+  b.qg2 = gq[2];
+  b.qg3 = gq[3];
   return b;
 }
 
 // Entry i of the queue of a level's parity q.
 static __device__ __forceinline__ int32_t* bq_at(const BlockBfs& b, int q, int i) {
-  if (i < b.cap) return b.qs[q] + i;
+  if (i < b.cap) return b.qs + q * b.cap + i;
   i -= b.cap;
-  return i < b.g.n ? b.qg[2 * q] + i : b.qg[2 * q + 1] + (i - b.g.n);
-}
-
-// Claim vertex w in a visited bitmap: true for exactly one caller.
-static __device__ __forceinline__ bool bvis_claim(uint32_t* bm, int w) {
-  const uint32_t bit = 1u << (w & 31);
-  if (*reinterpret_cast<volatile uint32_t*>(&bm[w >> 5]) & bit) return false;
-  return (atomicOr(&bm[w >> 5], bit) & bit) == 0u;
+  if (i < b.g.n) return (q ? b.qg2 : b.qg0) + i;
+  return (q ? b.qg3 : b.qg1) + (i - b.g.n);
 }
 
 // Smallest vertex of search A in the queue of parity q (first `size`
@@ -144,28 +145,109 @@ struct BlockBfsOut {
   bool dropped;      // B was dropped because t != srcB
 };
 
-// Searches A from srcA and (srcB >= 0) B from srcB, level-synchronous, in
-// the calling block (the sliced columns may have been written in this launch,
-// so they are read past the read-only cache); every thread of the block calls it.  kSliced: neighbours
-// from the sliced layout (b.sp), kC16: as int16 offsets.
-template <bool kSliced, bool kC16>
-static __device__ BlockBfsOut block_bfs2_t(const BlockBfs& b, int srcA, int srcB) {
-  const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31, wbase = tid - lane;
-  const int words = (b.g.n + 31) >> 5;
+// One level: the `size` entries of the queue of parity q; claimed neighbours go
+// to the other queue, their number to *cnt and B's part of it to *cntB.
+// kN: neighbours a lane takes of its vertex, 8 / kN lanes a vertex.  A warp
+// issues a level's instructions one after the other, and with two vertices of
+// eight neighbours a lane those took most of a level (about 5,500 clocks, a
+// third of it waiting for memory); a narrow frontier therefore spreads its
+// neighbours over the block's lanes.  kSliced: neighbours from the sliced
+// layout (b.sp), kC16: as int16 offsets; it may have been written in this
+// launch, so it is read past the read-only cache.
+template <bool kSliced, bool kC16, int kN>
+static __device__ __forceinline__ void block_level(const BlockBfs& b, int q, int size, bool liveB, int* cnt,
+                                                   int* cntB) {
+  constexpr int kL = 8 / kN, kPer = 32 / kL;  // lanes a vertex, vertices a warp
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
   const int16_t* s16 = reinterpret_cast<const int16_t*>(b.g.scol);
   const int32_t* s32 = reinterpret_cast<const int32_t*>(b.g.scol);
+  const int sub = (lane % kL) * kN;
+  for (int base = warp * kPer; base < size; base += warps * kPer) {  // warp-uniform bound
+    const int idx = base + lane / kL;
+    int u = -1, e0 = 0, deg = 0, tag = 0;
+    if (idx < size) {
+      const int e = *bq_at(b, q, idx);
+      tag = e & 1;
+      if (!tag || liveB) u = e >> 1;
+    }
+    if (u >= 0) {
+      if (kSliced) {
+        const int a0 = b.sp[u >> 5], a1 = b.sp[(u >> 5) + 1];
+        e0 = a0 + (u & 31);
+        deg = (a1 - a0) >> 5;  // the slice's width: padding entries name the row itself
+      } else {
+        e0 = __ldg(&b.g.rp[u]);
+        deg = __ldg(&b.g.rp[u + 1]) - e0;
+      }
+    }
+    uint32_t* vis = tag ? b.visB : b.visA;
+    const int maxdeg = __reduce_max_sync(0xffffffffu, deg);
+    for (int k0 = 0; k0 < maxdeg; k0 += 8) {
+      int w[kN];
+#pragma unroll
+      for (int j = 0; j < kN; ++j) {
+        const int k = k0 + sub + j;
+        w[j] = -1;
+        if (k < deg) {
+          if (!kSliced) w[j] = __ldg(&b.g.col[e0 + k]);
+          else if (kC16) w[j] = u + (int)__ldcg(&s16[e0 + kSlice * k]);
+          else w[j] = __ldcg(&s32[e0 + kSlice * k]);
+        }
+      }
+      // the bitmap words of all candidates first, then the atomics of those
+      // not visited yet
+      unsigned open = 0u, push = 0u;
+#pragma unroll
+      for (int j = 0; j < kN; ++j)
+        if (w[j] >= 0) open |= (~(*reinterpret_cast<const volatile uint32_t*>(&vis[w[j] >> 5]) >> (w[j] & 31)) & 1u) << j;
+#pragma unroll
+      for (int j = 0; j < kN; ++j) {
+        if ((open >> j) & 1u) {
+          const uint32_t bit = 1u << (w[j] & 31);
+          if (!(atomicOr(&vis[w[j] >> 5], bit) & bit)) push |= 1u << j;
+        }
+      }
+      const int m = __popc(push);
+      if (!__any_sync(0xffffffffu, m)) continue;  // warp-uniform
+      int inc = m;
+#pragma unroll
+      for (int o2 = 1; o2 < 32; o2 <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, inc, o2);
+        if (lane >= o2) inc += t;
+      }
+      const int totB = __reduce_add_sync(0xffffffffu, tag ? m : 0);
+      int at = 0;
+      if (lane == 31) {
+        at = atomicAdd(cnt, inc);
+        if (totB) atomicAdd(cntB, totB);
+      }
+      int pos = __shfl_sync(0xffffffffu, at, 31) + inc - m;
+#pragma unroll
+      for (int j = 0; j < kN; ++j)
+        if ((push >> j) & 1u) *bq_at(b, q ^ 1, pos++) = (w[j] << 1) | tag;
+    }
+  }
+}
+
+// Searches A from srcA and (srcB >= 0) B from srcB, level-synchronous, in
+// the calling block; every thread of the block calls it.  Not inlined: the
+// search then leaves the register allocation of the kernel around it alone.
+template <bool kSliced, bool kC16>
+static __device__ __noinline__ BlockBfsOut block_bfs2_t(const BlockBfs b, int srcA, int srcB) {
+  const int tid = threadIdx.x, T = blockDim.x;
+  const int words = (b.g.n + 31) >> 5;
   for (int i = tid; i < words; i += T) {
-    b.vis[0][i] = 0u;
-    b.vis[1][i] = 0u;
+    b.visA[i] = 0u;
+    b.visB[i] = 0u;
   }
   if (tid < 8) b.cnt[tid] = 0;
   __syncthreads();
   if (tid == 0) {
-    b.vis[0][srcA >> 5] |= 1u << (srcA & 31);
+    b.visA[srcA >> 5] |= 1u << (srcA & 31);
     *bq_at(b, 0, 0) = srcA << 1;
     b.cnt[0] = 1;
     if (srcB >= 0) {
-      b.vis[1][srcB >> 5] |= 1u << (srcB & 31);
+      b.visB[srcB >> 5] |= 1u << (srcB & 31);
       *bq_at(b, 0, 1) = (srcB << 1) | 1;
       b.cnt[0] = 2;
       b.cnt[3] = 1;
@@ -189,6 +271,10 @@ static __device__ BlockBfsOut block_bfs2_t(const BlockBfs& b, int srcA, int srcB
     }
     if (!liveB) sb = 0;
     if (sa == 0 && sb == 0) break;
+    if (b.wide && (size > b.wide || (b.grow && size > 128 + b.grow * level))) {
+      o.reached = -1;
+      break;
+    }
     if (b.poll && (level & 255) == 255) {
       if (tid == 0 && (volatile_status(b.poll) != 0 || poll_cancel(b.poll))) b.cnt[7] = 1;
       __syncthreads();
@@ -208,81 +294,10 @@ static __device__ BlockBfsOut block_bfs2_t(const BlockBfs& b, int srcA, int srcB
     const int q = level & 1;
     int* cnt = &b.cnt[(level + 1) % 3];
     int* cntB = &b.cnt[3 + (level + 1) % 3];
-    // Two frontier vertices per lane per round, so that their loads overlap.
-    for (int base = wbase; base < size; base += 2 * T) {  // warp-uniform bound
-      int u[2], e0[2], deg[2], tag[2];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int idx = base + h * T + lane;
-        u[h] = -1;
-        e0[h] = 0;
-        deg[h] = 0;
-        tag[h] = 0;
-        if (idx < size) {
-          const int e = *bq_at(b, q, idx);
-          tag[h] = e & 1;
-          if (!tag[h] || liveB) u[h] = e >> 1;
-        }
-      }
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        if (u[h] >= 0) {
-          if (kSliced) {
-            const int s = u[h] >> 5;
-            e0[h] = b.sp[s] + (u[h] & 31);
-            deg[h] = (b.sp[s + 1] - b.sp[s]) >> 5;  // the slice's width: padding entries name the row itself
-          } else {
-            e0[h] = __ldg(&b.g.rp[u[h]]);
-            deg[h] = __ldg(&b.g.rp[u[h] + 1]) - e0[h];
-          }
-        }
-      }
-      const int maxdeg = __reduce_max_sync(0xffffffffu, max(deg[0], deg[1]));
-      for (int k0 = 0; k0 < maxdeg; k0 += 8) {
-        int w[2][8];
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            w[h][j] = -1;
-            if (k0 + j < deg[h]) {
-              if (!kSliced) w[h][j] = __ldg(&b.g.col[e0[h] + k0 + j]);
-              else if (kC16) w[h][j] = u[h] + (int)__ldcg(&s16[e0[h] + kSlice * (k0 + j)]);
-              else w[h][j] = __ldcg(&s32[e0[h] + kSlice * (k0 + j)]);
-            }
-          }
-        unsigned push[2] = {0u, 0u};
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          uint32_t* vis = b.vis[tag[h]];
-#pragma unroll
-          for (int j = 0; j < 8; ++j)
-            if (w[h][j] >= 0 && bvis_claim(vis, w[h][j])) push[h] |= 1u << j;
-        }
-        const int m0 = __popc(push[0]), m1 = __popc(push[1]);
-        int inc = m0 + m1;
-#pragma unroll
-        for (int o2 = 1; o2 < 32; o2 <<= 1) {
-          const int t = __shfl_up_sync(0xffffffffu, inc, o2);
-          if (lane >= o2) inc += t;
-        }
-        const int tot = __shfl_sync(0xffffffffu, inc, 31);
-        if (tot == 0) continue;  // warp-uniform
-        const int totB = __reduce_add_sync(0xffffffffu, (tag[0] ? m0 : 0) + (tag[1] ? m1 : 0));
-        int at = 0;
-        if (lane == 0) {
-          at = atomicAdd(cnt, tot);
-          if (totB) atomicAdd(cntB, totB);
-        }
-        int pos = __shfl_sync(0xffffffffu, at, 0) + inc - m0 - m1;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-#pragma unroll
-          for (int j = 0; j < 8; ++j)
-            if ((push[h] >> j) & 1u) *bq_at(b, q ^ 1, pos++) = (w[h][j] << 1) | tag[h];
-        }
-      }
-    }
+    if (8 * size <= T) block_level<kSliced, kC16, 1>(b, q, size, liveB, cnt, cntB);
+    else if (4 * size <= T) block_level<kSliced, kC16, 2>(b, q, size, liveB, cnt, cntB);
+    else if (2 * size <= T) block_level<kSliced, kC16, 4>(b, q, size, liveB, cnt, cntB);
+    else block_level<kSliced, kC16, 8>(b, q, size, liveB, cnt, cntB);
     __syncthreads();
   }
   return o;  // unless stopped, the loop ends only after A has ended, so o.t is set

@@ -59,6 +59,7 @@ struct Ctl {
   alignas(128) int cls;
   int eps1_ready;  // fused stage 1: 0 pending, t + 1 when the kNN chose t, -1 on failure
   int x32_src;     // stage-1 result: -1 = x32, s >= 0 = snapshot slot s
+  int pd_done;     // the one-block 2BFS has succeeded
   int feat_sides;  // cluster kernel: sides of the features (l~, v) that are complete
   // device clock marks (ns)
   unsigned long long t_start, t_prep, t_features, t_fp32, t_fp64, t_end;

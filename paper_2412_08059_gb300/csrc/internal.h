@@ -70,7 +70,7 @@ cudaError_t launch_cluster(const Launch& L, const double* b, double* x, const mp
 
 // bfs.cu
 BfsGraph bfs_graph(const Launch& L);
-cudaError_t launch_pseudo_diameter(const Launch& L, int slot);
+cudaError_t launch_pseudo_diameter(const Launch& L, int slot, int starts);
 cudaError_t launch_bfs_only(const Launch& L, int src, int32_t* dist, int slot);
 cudaError_t launch_copy_pdiam(const Launch& L, int32_t* out);
 const void* bfs_kernel();

@@ -1,0 +1,57 @@
+"""The one-block 2BFS of mpcg_pseudo_diameter and mpcg_features (GPU) against
+the oracle: long thin graphs it finishes, graphs whose frontier grows past its
+limits (the grid-wide search then does the work), the sizes at which its
+limits change, disconnected graphs, rows past the sliced layout's cap, and
+both column formats (columns further than 32,767 from their row)."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def mp():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2412_08059_gb300 import build, mpcg
+    build.build()
+    mpcg.load()
+    return mpcg
+
+
+def _two(A, B):
+    return synth.CSR(np.concatenate([A.row_ptr, A.nnz + B.row_ptr[1:]]).astype(np.int32),
+                     np.concatenate([A.col, A.n + B.col]).astype(np.int32),
+                     np.concatenate([A.val, B.val]))
+
+
+CASES = {
+    "one": lambda: synth.laplacian_2d(1, 1),
+    "path_3000": lambda: synth.path(3000),
+    "thin_2000x40": lambda: synth.laplacian_2d(2000, 40),
+    "thin_40x2000": lambda: synth.laplacian_2d(40, 2000),
+    "square_128": lambda: synth.laplacian_2d(128, 128),        # n = 16384
+    "square_130": lambda: synth.laplacian_2d(130, 130),        # past it
+    "square_540": lambda: synth.laplacian_2d(540, 540),        # n = 291600
+    "square_550": lambda: synth.laplacian_2d(550, 550),        # past the largest
+    "cube_30": lambda: synth.laplacian_3d(30),                 # given up for the grid
+    "star_5000": lambda: synth.star(5000, 1.1),                # a row past the width cap
+    "rreg_40000": lambda: synth.random_regular_laplacian(40000, 8, 1e-3, seed=5),
+    "band_20000": lambda: synth.banded(20000, 15, 0.6, 1.1, seed=7),
+    "two_parts": lambda: _two(synth.laplacian_2d(300, 20), synth.laplacian_2d(50, 50)),
+}
+
+
+@pytest.mark.parametrize("name", sorted(CASES))
+def test_block_pdiam(mp, name):
+    A = CASES[name]()
+    dA = mp.DeviceCSR.from_host(A)
+    want, t = oracle.pseudo_diameter(A, return_t=True)
+    assert mp.pseudo_diameter(dA) == (want, t)
+    _, b = synth.rhs(A, seed=3)
+    f = mp.features(dA, torch.from_numpy(b).cuda())
+    assert f["pdiam"] == want and f["status"] in (mp.OK, mp.WARN_EPS1_NOT_REACHED)
