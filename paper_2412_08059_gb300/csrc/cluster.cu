@@ -119,6 +119,7 @@ struct ClShared {
   float fval;
   int dec, aux_i;
   int2 tab[kClWarps * kClMaxRpt];  // first entry and width | overflow flag, by slice
+  int tail;                        // entries of row tails kept past the slices'
   // Algorithm II, thread 0's record of the candidate crossings (as k_stage1)
   double s_lo[17], s_hi[17], res_at[16];
   int nt[16], snap_it[kClSnaps];
@@ -222,15 +223,32 @@ struct ClMat {
   uint16_t* c;
 };
 
-// Columns once, values at the start of each stage.
-template <typename T>
+__device__ __forceinline__ uint16_t cl_pack(int nslices, int c) {
+  const int o = cl_owner(nslices, c >> 5);
+  return (uint16_t)((o << 12) | (c - kSlice * cl_first(nslices, o)));
+}
+
+// Columns once (`cols`), values at the start of each stage.  The entries of a
+// row past the layout's width cap go behind the slices' where there is room
+// (tail[j]: first entry | number << 16; 0: none, or read from the CSR).  Read
+// from the caller's CSR at every pass, with a division for the owner of each,
+// they made a random tree's SpMV three times as long as its other rows need.
+template <typename T, int RPT>
 __device__ __forceinline__ void cl_load(const ClusterArgs& a, ClShared& S, const ClMat& M, int S0,
-                                        int ns, const T* sv, bool cols) {
+                                        int ns, const T* sv, bool cols, uint32_t (&tail)[RPT]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int E0 = a.slice_ptr[S0];
+  const int E0 = a.slice_ptr[S0], E = a.slice_ptr[S0 + ns] - E0;
   const bool c16 = a.ctl->col16 != 0;
   T* vd = reinterpret_cast<T*>(M.v);
-  for (int s = warp; s < ns; s += kClWarps) {
+  if (cols) {
+    if (threadIdx.x == 0) S.tail = 0;
+    __syncthreads();
+  }
+#pragma unroll
+  for (int j = 0; j < RPT; ++j) {
+    const int s = warp + kClWarps * j;
+    if (cols) tail[j] = 0u;
+    if (s >= ns) continue;
     const uint32_t wf = a.slice_w[S0 + s];
     const int w = (int)(wf & ~kOverflowBit), p = a.slice_ptr[S0 + s];
     if (lane == 0) S.tab[s] = make_int2(p - E0, (int)wf);
@@ -240,19 +258,46 @@ __device__ __forceinline__ void cl_load(const ClusterArgs& a, ClShared& S, const
       vd[e - E0] = sv[e];
       if (cols) {
         const int c = c16 ? i + (int)reinterpret_cast<const int16_t*>(a.scol)[e] : a.scol[e];
-        const int o = cl_owner(a.nslices, c >> 5);
-        M.c[e - E0] = (uint16_t)((o << 12) | (c - kSlice * cl_first(a.nslices, o)));
+        M.c[e - E0] = cl_pack(a.nslices, c);
+      }
+    }
+    if ((wf & kOverflowBit) && i < a.n) {
+      const int e0 = a.rp[i] + w, cnt = a.rp[i + 1] - e0;
+      if (cols && cnt > 0 && cnt < (1 << 15)) {
+        const int at = E + atomicAdd(&S.tail, cnt);
+        if (at + cnt <= a.ent_cap && at < (1 << 16)) tail[j] = (uint32_t)at | ((uint32_t)cnt << 16);
+      }
+      const int at = (int)(tail[j] & 0xffffu), m = (int)(tail[j] >> 16);
+      for (int k = 0; k < m; ++k) {
+        vd[at + k] = (T)a.val[e0 + k];
+        if (cols) M.c[at + k] = cl_pack(a.nslices, a.col[e0 + k]);
       }
     }
   }
   __syncthreads();
 }
 
+// acc + the sum over K entries of a row, from shared memory: all columns, then
+// all gathers, then the chain of fused multiply-adds, so that a row waits once
+// for its columns and once for its gathers.
+template <typename T, int K>
+__device__ __forceinline__ T cl_entries(uint32_t gb, const uint16_t* cp, const T* vp, T acc) {
+  uint32_t c[K];
+  T x[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) c[k] = cp[kSlice * k];
+#pragma unroll
+  for (int k = 0; k < K; ++k) cl_ld(cl_map(gb, c[k] >> 12) + (c[k] & 4095u) * (uint32_t)sizeof(T), x[k]);
+#pragma unroll
+  for (int k = 0; k < K; ++k) acc = fma(vp[kSlice * k], x[k], acc);
+  return acc;
+}
+
 // Row sums of the block's slices: q[j] = sum_k v_k g(c_k) of row
-// 32 (warp + 16 j) + lane, in stored order.
+// 32 (warp + 16 j) + lane, in stored order (0 where the thread has no row).
 template <typename T, int RPT>
 __device__ __forceinline__ void cl_spmv(const ClusterArgs& a, const ClShared& S, const ClMat& M, int S0,
-                                        int ns, T (&q)[RPT]) {
+                                        int ns, const uint32_t (&tail)[RPT], T (&q)[RPT]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t gb = smem_addr(M.g);
 #pragma unroll
@@ -265,30 +310,58 @@ __device__ __forceinline__ void cl_spmv(const ClusterArgs& a, const ClShared& S,
       const int w = (int)(wf & ~kOverflowBit);
       const uint16_t* cp = M.c + t.x + lane;
       const T* vp = reinterpret_cast<const T*>(M.v) + t.x + lane;
-      for (int k0 = 0; k0 < w; k0 += 8) {  // warp-uniform
-        T v[8], x[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          if (k0 + k < w) {
-            const uint32_t c = cp[kSlice * (k0 + k)];
-            v[k] = vp[kSlice * (k0 + k)];
-            cl_ld(cl_map(gb, c >> 12) + (c & 4095u) * (uint32_t)sizeof(T), x[k]);
-          }
-        }
-#pragma unroll
-        for (int k = 0; k < 8; ++k)
-          if (k0 + k < w) acc = fma(v[k], x[k], acc);
+      int k = 0;
+      while (w - k > 9) {  // warp-uniform
+        acc = cl_entries<T, 6>(gb, cp + kSlice * k, vp + kSlice * k, acc);
+        k += 6;
+      }
+      cp += kSlice * k;
+      vp += kSlice * k;
+      switch (w - k) {
+        case 1: acc = cl_entries<T, 1>(gb, cp, vp, acc); break;
+        case 2: acc = cl_entries<T, 2>(gb, cp, vp, acc); break;
+        case 3: acc = cl_entries<T, 3>(gb, cp, vp, acc); break;
+        case 4: acc = cl_entries<T, 4>(gb, cp, vp, acc); break;
+        case 5: acc = cl_entries<T, 5>(gb, cp, vp, acc); break;
+        case 6: acc = cl_entries<T, 6>(gb, cp, vp, acc); break;
+        case 7: acc = cl_entries<T, 7>(gb, cp, vp, acc); break;
+        case 8: acc = cl_entries<T, 8>(gb, cp, vp, acc); break;
+        case 9: acc = cl_entries<T, 9>(gb, cp, vp, acc); break;
+        default: break;
       }
       const int i = (S0 + s) * kSlice + lane;
-      if ((wf & kOverflowBit) && i < a.n) {  // the row's tail from the caller's CSR
-        const int e1 = a.rp[i + 1];
-        for (int e = a.rp[i] + w; e < e1; ++e) {
-          const int c = a.col[e], o = cl_owner(a.nslices, c >> 5);
+      if (wf & kOverflowBit) {
+        const int m = (int)(tail[j] >> 16);
+        const uint16_t* tc = M.c + (tail[j] & 0xffffu);
+        const T* tv = reinterpret_cast<const T*>(M.v) + (tail[j] & 0xffffu);
+        int e = 0;
+        for (; e + 4 <= m; e += 4) {
+          T x[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const uint32_t c = tc[e + u];
+            cl_ld(cl_map(gb, c >> 12) + (c & 4095u) * (uint32_t)sizeof(T), x[u]);
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u) acc = fma(tv[e + u], x[u], acc);
+        }
+        for (; e < m; ++e) {
+          const uint32_t c = tc[e];
           T x;
-          cl_ld(cl_map(gb, o) + (uint32_t)(c - kSlice * cl_first(a.nslices, o)) * (uint32_t)sizeof(T), x);
-          acc = fma((T)a.val[e], x, acc);
+          cl_ld(cl_map(gb, c >> 12) + (c & 4095u) * (uint32_t)sizeof(T), x);
+          acc = fma(tv[e], x, acc);
+        }
+        if (m == 0 && i < a.n) {  // no room: from the caller's CSR
+          const int e1 = a.rp[i + 1];
+          for (int f = a.rp[i] + w; f < e1; ++f) {
+            const uint32_t c = cl_pack(a.nslices, a.col[f]);
+            T x;
+            cl_ld(cl_map(gb, c >> 12) + (c & 4095u) * (uint32_t)sizeof(T), x);
+            acc = fma((T)a.val[f], x, acc);
+          }
         }
       }
+      if (i >= a.n) acc = (T)0;
     }
     q[j] = acc;
   }
@@ -415,13 +488,14 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
     const int s = warp + kClWarps * j, i = (S0 + s) * kSlice + lane;
     row[j] = s < ns && i < n ? i : -1;
   }
+  uint32_t tail[RPT];  // where the entries past the width cap are (cl_load)
   double xd[RPT];
 #pragma unroll
   for (int j = 0; j < RPT; ++j) xd[j] = 0.0;
 
   // =================== single-precision stage ===================
   if (a.mode != 2) {
-    cl_load<float>(a, S, M, S0, ns, a.sv32, true);
+    cl_load<float, RPT>(a, S, M, S0, ns, a.sv32, true, tail);
     float* g = reinterpret_cast<float*>(M.g);
     const bool autom = a.mode == 1;
     const int max1 = ctl->max1, k0 = ctl->k0;
@@ -485,13 +559,13 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
         if (cancelled) {
           dec = kClFail;
           if (lead0) set_status(ctl, MPCG_ERR_CANCELLED);
-        } else if (isnan(rr)) {
+        } else if (bits_nan(rr)) {
           dec = kClFail;
           if (lead0) set_status(ctl, MPCG_ERR_NAN);
         } else if (!autom) {
           if (stop_pass(thr, rr) || it >= max1) dec = kClStop;
         } else {
-          if (in_k0 && (it >= min(k0, max1) || rr == 0.0 || stop_pass(thr, rr))) {
+          if (in_k0 && (it >= min(k0, max1) || dbits(rr) == 0 || stop_pass(thr, rr))) {
             in_k0 = 0;  // end of the k0 phase: v of Eq. (13)
             if (rank == 0) {
               if (lane == 0) {
@@ -508,7 +582,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
             bool fresh = false;
             const unsigned open = S.cmask & ~S.met;
             __syncwarp();
-            if (open && rr <= S.s_hi[__ffs(open) - 1]) {
+            if (open && dbits(rr) <= dbits(S.s_hi[__ffs(open) - 1])) {
               unsigned met = S.met;
               __syncwarp();
               for (int t = 0; t < 16; ++t) {
@@ -579,7 +653,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
         cw = cancel_word(ctl);
         if (autom && cls < 0) label_now = *reinterpret_cast<volatile int*>(&ctl->eps1_ready);
       }
-      cl_spmv<float, RPT>(a, S, M, S0, ns, q);
+      cl_spmv<float, RPT>(a, S, M, S0, ns, tail, q);
       FF pdq{0.f, 0.f};
       float d[RPT];
 #pragma unroll
@@ -593,10 +667,10 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
       const double dq = cl_total_ff(S, rank, ns, red, pdq);
       if (warp == 0) {
         int d2 = kClGo;
-        if (!isfinite(dq)) {
+        if (!bits_finite(dq)) {
           d2 = kClFail;
           if (lead0) set_status(ctl, MPCG_ERR_NAN);
-        } else if (!(dq > 0.0)) {
+        } else if (!bits_positive(dq)) {
           d2 = kClBroke;  // stage 1 ends here; x~ and r are unchanged
         } else if (lane == 0) {
           S.fval = (float)(rr / dq);
@@ -627,7 +701,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
         cancelled = word == 100;
         if (word < 0) {
           d3 = kClFail;
-        } else if (!isfinite(rrn)) {
+        } else if (!bits_finite(rrn)) {
           d3 = kClFail;
           if (lead0) set_status(ctl, MPCG_ERR_NAN);
         } else {
@@ -727,7 +801,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
   }
 
   // =================== double-precision stage ===================
-  cl_load<double>(a, S, M, S0, ns, a.sv64, a.mode == 2);
+  cl_load<double, RPT>(a, S, M, S0, ns, a.sv64, a.mode == 2, tail);
   double* g = reinterpret_cast<double*>(M.g);
   const double bnorm = ctl->bnorm64, eps2 = ctl->eps2;
   const int max2 = ctl->max2, max_restarts = ctl->max_restarts;
@@ -743,12 +817,15 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
     for (int j = 0; j < RPT; ++j)
       if (warp + kClWarps * j < ns) g[(warp + kClWarps * j) * kSlice + lane] = xd[j];
     cl_sync();
-    cl_spmv<double, RPT>(a, S, M, S0, ns, q);
+    cl_spmv<double, RPT>(a, S, M, S0, ns, tail, q);
     double p = 0.0;
 #pragma unroll
     for (int j = 0; j < RPT; ++j) {
-      q[j] = row[j] >= 0 ? a.b64[row[j]] - q[j] : 0.0;
-      p = __fma_rn(q[j], q[j], p);
+      if (warp + kClWarps * j < ns) {
+        __syncwarp();
+        q[j] = row[j] >= 0 ? a.b64[row[j]] - q[j] : 0.0;
+        p = __fma_rn(q[j], q[j], p);
+      }
     }
     int cw = lead0 ? cancel_word(ctl) : 0;
     int half = red & 1;
@@ -759,7 +836,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
         failed = MPCG_ERR_CANCELLED;
         return kClFail;
       }
-      if (isnan(rrv)) {
+      if (bits_nan(rrv)) {
         failed = MPCG_ERR_NAN;
         return kClFail;
       }
@@ -784,7 +861,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
       }
       if (dec == kClGo) {
         rr = tot;
-        dec = head(rr, it, S.aux[half] != 0.0);
+        dec = head(rr, it, dbits(S.aux[half]) != 0);
       }
       if (lane == 0) S.dec = dec;
     }
@@ -802,21 +879,25 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
     while (dec == kClGo) {
       if (lead0) cw = cancel_word(ctl);  // used with the r^T r sum
       // ---- q = A d, d^T q ----
-      cl_spmv<double, RPT>(a, S, M, S0, ns, q);
+      cl_spmv<double, RPT>(a, S, M, S0, ns, tail, q);
+      // (A predicated-off FP64 instruction takes its turn of the FP64 pipe:
+      // warps without a slice branch around these.  The __syncwarp keeps the
+      // compiler from predicating the short bodies.)
       double pq = 0.0, d[RPT];
 #pragma unroll
       for (int j = 0; j < RPT; ++j) {
         d[j] = 0.0;
-        if (row[j] >= 0) {
-          d[j] = g[row[j] - S0 * kSlice];
+        if (warp + kClWarps * j < ns) {
+          __syncwarp();
+          d[j] = g[(warp + kClWarps * j) * kSlice + lane];
           pq = __fma_rn(d[j], q[j], pq);
         }
       }
       const double dq = cl_total(S, rank, ns, red, pq);
       if (warp == 0) {
         int d2 = kClGo;
-        if (!isfinite(dq)) failed = MPCG_ERR_NAN;
-        else if (!(dq > 0.0)) failed = MPCG_ERR_BREAKDOWN;
+        if (!bits_finite(dq)) failed = MPCG_ERR_NAN;
+        else if (!bits_positive(dq)) failed = MPCG_ERR_BREAKDOWN;
         else if (lane == 0) S.val = rr / dq;
         if (failed) d2 = kClFail;
         if (lane == 0) S.dec = d2;
@@ -829,7 +910,8 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
       double pr = 0.0;
 #pragma unroll
       for (int j = 0; j < RPT; ++j) {
-        if (row[j] >= 0) {
+        if (warp + kClWarps * j < ns) {
+          __syncwarp();
           r[j] = __fma_rn(-alpha, q[j], r[j]);
           pr = __fma_rn(r[j], r[j], pr);
         }
@@ -838,11 +920,11 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
       const double rrn = cl_total(S, rank, ns, red, pr, (double)cw);
       if (warp == 0) {
         int d3 = kClFail;
-        if (!isfinite(rrn)) {
+        if (!bits_finite(rrn)) {
           failed = MPCG_ERR_NAN;
           if (lane == 0) S.aux_i = 0;  // x keeps the iterate before the failing step
         } else {
-          d3 = head(rrn, it + 1, S.aux[half] != 0.0);
+          d3 = head(rrn, it + 1, dbits(S.aux[half]) != 0);
           if (lane == 0) {
             S.val = rrn / rr;  // beta
             S.aux_i = 1;
@@ -859,13 +941,21 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
       // ---- d = r + beta d, x += alpha d ----
       if (dec == kClGo) {
 #pragma unroll
-        for (int j = 0; j < RPT; ++j)
-          if (row[j] >= 0) g[row[j] - S0 * kSlice] = __fma_rn(beta, d[j], r[j]);
+        for (int j = 0; j < RPT; ++j) {
+          if (warp + kClWarps * j < ns) {
+            __syncwarp();
+            g[(warp + kClWarps * j) * kSlice + lane] = __fma_rn(beta, d[j], r[j]);
+          }
+        }
         cl_arrive();
       }
 #pragma unroll
-      for (int j = 0; j < RPT; ++j)
-        if (row[j] >= 0) xd[j] = __fma_rn(alpha, d[j], xd[j]);
+      for (int j = 0; j < RPT; ++j) {
+        if (warp + kClWarps * j < ns) {
+          __syncwarp();
+          xd[j] = __fma_rn(alpha, d[j], xd[j]);
+        }
+      }
       ++it;
       if (dec == kClGo) cl_wait();
     }

@@ -127,6 +127,22 @@ __device__ __forceinline__ double stop_measure(double rr, double bnorm, int rel)
   return rel ? sqrt(rr) / bnorm : sqrt(rr);
 }
 
+// Comparisons of doubles by their bit patterns: an FP64 comparison takes its
+// turn of the FP64 pipe (about 80 clocks in a chain), an integer one does not.
+// Values that are not negative order like their bits; every NaN is above
+// infinity there.
+__device__ __forceinline__ long long dbits(double v) { return __double_as_longlong(v); }
+__device__ __forceinline__ bool bits_finite(double v) {
+  return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000;
+}
+__device__ __forceinline__ bool bits_nan(double v) {
+  return (dbits(v) & 0x7fffffffffffffffll) > 0x7ff0000000000000ll;
+}
+// v > 0 (false for NaN)
+__device__ __forceinline__ bool bits_positive(double v) {
+  return dbits(v) > 0 && dbits(v) <= 0x7ff0000000000000ll;
+}
+
 // The stop test stop_measure(rr) <= eps without a square root and a division
 // per iteration.  stop_measure is non-decreasing in rr, so the test passes
 // exactly for rr up to some threshold near t = (eps ||b||)^2 (or eps^2).
@@ -149,8 +165,10 @@ __device__ __forceinline__ StopThr stop_thr(double eps, double bnorm, int rel) {
   return T;
 }
 __device__ __forceinline__ bool stop_pass(const StopThr& T, double rr) {
-  if (rr <= T.lo) return true;
-  if (rr > T.hi) return false;
+  // rr is a sum of squares (not negative) or NaN, for which the test fails; lo
+  // is -1 where it never passes by itself
+  if (dbits(rr) <= dbits(T.lo)) return true;
+  if (dbits(rr) > dbits(T.hi)) return false;
   return stop_measure(rr, T.bnorm, T.rel) <= T.eps;
 }
 
