@@ -41,6 +41,7 @@
 
 #include <type_traits>
 
+#include "feature_block.cuh"
 #include "internal.h"
 
 namespace mpcg {
@@ -124,6 +125,7 @@ struct CShared {
   int dec;
   int ok;
   int aux;
+  int nb;  // blocks of the CG group (the barriers' and sums' blocks)
 };
 
 // Block partial of float-float sums, valid in thread 0 (float ops only until
@@ -196,18 +198,18 @@ __device__ __noinline__ int cgrid_wait(Ctl* ctl, int slot, unsigned long long ta
 // when another block has recorded an error.
 template <int NC>
 __device__ __forceinline__ bool cgrid_barrier(Ctl* ctl, int slot, unsigned long long& round,
-                                              int* s_ok) {
+                                              CShared<NC>& S) {
   cbar<NC>();
   round += 1;
   if (threadIdx.x == 0) {
-    const unsigned long long target = round * (unsigned long long)gridDim.x;
+    const unsigned long long target = round * (unsigned long long)S.nb;
     red_release_add(&ctl->bar[slot].v, 1ull);
     int ok = 1;
     if (ld_acquire(&ctl->bar[slot].v) < target) ok = cgrid_wait(ctl, slot, target);
-    *s_ok = ok;
+    S.ok = ok;
   }
   cbar<NC>();
-  return *s_ok != 0;
+  return S.ok != 0;
 }
 
 // Grid-wide sum of the block partials (block partial valid in thread 0;
@@ -221,18 +223,30 @@ __device__ __forceinline__ double cgrid_total(double block_part, double* partial
   double* buf = partials + (red & 1) * kMaxGrid;
   ++red;
   if (threadIdx.x == 0) buf[blockIdx.x] = block_part;
-  ok = cgrid_barrier<NC>(ctl, slot, round, &S.ok);
+  ok = cgrid_barrier<NC>(ctl, slot, round, S);
+  const int nb = S.nb;
   // extra (thread 0): the slot after the partials, which block 0 wrote before
   // the barrier; loaded beside them rather than after the sum
-  if (extra && threadIdx.x == 0) *extra = buf[gridDim.x];
+  if (extra && threadIdx.x == 0) *extra = buf[nb];
   double s = 0.0;
   if (threadIdx.x < 32) {
     if (f32) {  // option acc32: the blocks' float partials summed in float
       float sf = 0.0f;
-      for (int i = threadIdx.x; i < (int)gridDim.x; i += 32) sf = __fadd_rn(sf, (float)buf[i]);
+      for (int i = threadIdx.x; i < nb; i += 32) sf = __fadd_rn(sf, (float)buf[i]);
       s = (double)warp_sum_f(sf);
     } else {
-      for (int i = threadIdx.x; i < (int)gridDim.x; i += 32) s += buf[i];
+      // a lane's partials all in flight before the first add
+      constexpr int kU = 5;  // 160 blocks a round
+      for (int i0 = 0; i0 < nb; i0 += 32 * kU) {
+        double v[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+          const int i = i0 + 32 * u + (int)threadIdx.x;
+          v[u] = i < nb ? buf[i] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < kU; ++u) s += v[u];
+      }
       s = warp_sum(s);
     }
   }
@@ -567,15 +581,15 @@ __device__ __forceinline__ bool ring_spmv(const CgArgs& a, Ring<T>& R, Cursor& C
 // Set-up common to both stages: the ring in dynamic shared memory, the
 // block's slice range and element range, barrier initialisation.
 template <int NC, typename T>
-__device__ __forceinline__ void ring_setup(const CgArgs& a, char* smem, Ring<T>& R, int& S0,
-                                           int& S1) {
+__device__ __forceinline__ void ring_setup(const CgArgs& a, char* smem, Ring<T>& R, CShared<NC>& S_,
+                                           int nb, int& S0, int& S1) {
   constexpr int S = Ring<T>::S;
   R.base = smem;
   R.full = reinterpret_cast<unsigned long long*>(smem + S * stage_bytes<T>());
   R.empty = R.full + S;
   R.stop = reinterpret_cast<volatile int*>(R.empty + S);
-  S0 = (int)((long long)a.nslices * blockIdx.x / gridDim.x);
-  S1 = (int)((long long)a.nslices * (blockIdx.x + 1) / gridDim.x);
+  S0 = (int)((long long)a.nslices * blockIdx.x / nb);
+  S1 = (int)((long long)a.nslices * (blockIdx.x + 1) / nb);
   R.E0 = a.slice_ptr[S0];
   R.E1 = a.slice_ptr[S1];
   R.nch = (unsigned)((R.E1 - R.E0 + kCH - 1) >> kLogCH);
@@ -586,6 +600,7 @@ __device__ __forceinline__ void ring_setup(const CgArgs& a, char* smem, Ring<T>&
       mbar_init(&R.empty[s], NC);
     }
     *R.stop = 0;
+    S_.nb = nb;
     mbar_fence_init();
   }
   __syncthreads();
@@ -741,7 +756,7 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_cg32(CgArgs a) {
   }
   Ring<float> R;
   int S0, S1;
-  ring_setup<NC>(a, smem, R, S0, S1);
+  ring_setup<NC>(a, smem, R, S, (int)gridDim.x, S0, S1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (warp == NC) {
     if (lane == 0) ring_producer(a, R);
@@ -1109,7 +1124,7 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_cg64(CgArgs a) {
   if (volatile_status(ctl) != 0) return;
   Ring<double> R;
   int S0, S1;
-  ring_setup<NC>(a, smem, R, S0, S1);
+  ring_setup<NC>(a, smem, R, S, (int)gridDim.x, S0, S1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n = a.n;
   if (ctl->trivial) {  // b = 0: x = 0 solves A x = b exactly
@@ -1151,7 +1166,7 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_cg64(CgArgs a) {
     const float* xs = src >= 0 ? a.snap + (size_t)src * n : a.x32;
     for (int i = R0 + lane; i < R1; i += kSlice) a.x64[i] = a.mode ? 0.0 : (double)xs[i];
   }
-  ok = cgrid_barrier<NC>(ctl, a.slot, round, &S.ok);
+  ok = cgrid_barrier<NC>(ctl, a.slot, round, S);
 
   // One SpMV pass per step; its kind is decided by thread 0 and broadcast.
   //   kRestart:  r = b - A x, d = r, r^T r      (CG line 1 from x)
@@ -1279,7 +1294,7 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_cg64(CgArgs a) {
       // ---- P3: x += alpha d, d = r + beta d (kPc: d = dinv r + beta d) ----
       if constexpr (kPc) p3_64_pc(a, R0, R1, lane, alpha, S.val);
       else p3_64(a, R0, R1, lane, alpha, S.val);
-      ok = cgrid_barrier<NC>(ctl, a.slot, round, &S.ok);
+      ok = cgrid_barrier<NC>(ctl, a.slot, round, S);
       ++it;
       next = -1;
     } else if (next == kTrueRes + 100) {
@@ -1300,7 +1315,7 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_cg64(CgArgs a) {
         const double tz = cgrid_total(block_d(pzr, S), a.partials, red, ctl, a.slot, round, S, ok);
         if (lead) rz = tz;
       } else {
-        ok = cgrid_barrier<NC>(ctl, a.slot, round, &S.ok);
+        ok = cgrid_barrier<NC>(ctl, a.slot, round, S);
       }
       next = -1;
     }
@@ -1389,8 +1404,47 @@ __device__ __noinline__ bool stage1_pdiam(const BfsGraph g, int32_t* d1, int32_t
   return ok;
 }
 
+// The feature block: the 2BFS in this block, then v (bounded wait for block 0's
+// consumers) and the vote.  Every block of the launch is resident (cooperative
+// launch), so the wait ends.
+__device__ __noinline__ void stage1_feature_block(const Stage1Args& sa, unsigned char* smem) {
+  const CgArgs& a = sa.a;
+  Ctl* ctl = a.ctl;
+  const bool ok = block_pdiam_any(ctl, a.rp, a.col, a.slice_ptr, a.slice_w, a.scol, a.n, sa.g, sa.d1, sa.d2, smem,
+                                  (int)ring_smem_bytes<float>());
+  __syncthreads();
+  if (threadIdx.x >= 32) return;
+  int have_v = 0;
+  if (ok && threadIdx.x == 0) {
+    const volatile int* flag = &ctl->feat_sides;
+    const unsigned long long t0 = globaltimer();
+    unsigned spins = 0;
+    while (!(have_v = *flag)) {
+      if ((++spins & 255u) == 0) {
+        if (volatile_status(ctl) != 0 || poll_cancel(ctl)) break;
+        if (globaltimer() - t0 > (unsigned long long)ctl->timeout_ns) {
+          set_status(ctl, MPCG_ERR_TIMEOUT);
+          break;
+        }
+      }
+    }
+    __threadfence();
+  }
+  have_v = __shfl_sync(0xffffffffu, have_v, 0);
+  if (have_v) feature_vote(sa.knn, ctl);
+  else if (threadIdx.x == 0) atomicExch(&ctl->eps1_ready, -1);
+}
+
+// kFeat: one block, the last of the grid, runs the 2BFS alone (bfs_block.cuh)
+// and the vote; the others run CG with fifteen consumer warps.  For systems of
+// up to kFeatBlockN rows: the one-warp-a-block search costs 5 us a level there
+// and slows the iterations beside it from 9.5 to 19 us (301 x 203 grid, 502
+// levels; this form: 3 us a level, 9.5 us an iteration).  Wide graphs of more
+// rows are too much work for one block.
+constexpr int kFeatBlockN = 80000;
+template <bool kFeat>
 __global__ void __launch_bounds__(kTmaThreads, 1) k_stage1(Stage1Args sa) {
-  constexpr int NC = kNC1;
+  constexpr int NC = kFeat ? kNC : kNC1;
   extern __shared__ __align__(128) char smem[];
   __shared__ CShared<NC> S;
   __shared__ volatile int s_k0_ready;
@@ -1407,15 +1461,20 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_stage1(Stage1Args sa) {
     s_help = kHelpNone;
     s_hl.cmd = 0;
   }
+  const int nb = kFeat ? (int)gridDim.x - 1 : (int)gridDim.x;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (kFeat && (int)blockIdx.x == nb) {
+    stage1_feature_block(sa, reinterpret_cast<unsigned char*>(smem));
+    return;
+  }
   Ring<float> R;
   int S0, S1;
-  ring_setup<NC>(a, smem, R, S0, S1);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (warp == NC + 1) {
+  ring_setup<NC>(a, smem, R, S, nb, S0, S1);
+  if (warp == (kFeat ? NC : NC + 1)) {
     if (lane == 0) ring_producer(a, R);
     return;
   }
-  if (warp == NC) {
+  if (!kFeat && warp == NC) {
     // ---- feature warp: 2BFS over the grid's feature warps ----
     const bool ok = stage1_pdiam(sa.g, sa.d1, sa.d2, ctl, sa.bfs_slot, &s_help, &s_hl, NC);
     if (blockIdx.x != 0) return;
@@ -1510,10 +1569,10 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_stage1(Stage1Args sa) {
   {
     double* buf = a.partials + (red & 1) * kMaxGrid;
     const double bp = block_ff(acc, S, f32);  // all consumer warps past the mask
-    if (lead0) buf[gridDim.x] = (double)s_cmask;
+    if (lead0) buf[nb] = (double)s_cmask;
     const double tot = cgrid_total(bp, a.partials, red, ctl, a.slot, round, S, ok, f32);
     if (lead) {
-      cmask = (unsigned)buf[gridDim.x];
+      cmask = (unsigned)buf[nb];
       met = 0u;
       S.rr = tot;
       S.val = sqrt(tot);
@@ -1576,9 +1635,14 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_stage1(Stage1Args sa) {
             ctl->k0_done = k0done;
             ctl->vsum = vsum;
             ctl->v = k0done > 0 ? vsum / (double)k0done : 0.0;
-            s_v = ctl->v;
-            __threadfence_block();
-            s_k0_ready = 1;
+            if (kFeat) {  // for the feature block
+              __threadfence();
+              atomicExch(&ctl->feat_sides, 1);
+            } else {
+              s_v = ctl->v;
+              __threadfence_block();
+              s_k0_ready = 1;
+            }
           }
         }
         if (!in_k0) {
@@ -1692,7 +1756,7 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_stage1(Stage1Args sa) {
     {
       double* buf = a.partials + (red & 1) * kMaxGrid;
       const double bp = block_ff(prr, S, f32);
-      if (lead0) buf[gridDim.x] = (double)label_now;
+      if (lead0) buf[nb] = (double)label_now;
       double label_slot = 0.0;
       const double rrn = cgrid_total(bp, a.partials, red, ctl, a.slot, round, S, ok, f32, &label_slot);
       if (lead) {
@@ -1727,7 +1791,7 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_stage1(Stage1Args sa) {
     ++it;
   }
 
-  if (ok && help) {  // the consumers join the 2BFS levels unless the search has ended
+  if (!kFeat && ok && help) {  // the consumers join the 2BFS levels unless the search has ended
     if (lead) S.aux = atomicCAS(&s_help, kHelpNone, kHelpJoined);
     cbar<NC>();
     if (S.aux == kHelpNone) bfs_help(sa.g, &s_hl, NC, warp + 1);
@@ -1737,9 +1801,14 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_stage1(Stage1Args sa) {
       ctl->k0_done = k0done;
       ctl->vsum = vsum;
       ctl->v = k0done > 0 ? vsum / (double)k0done : 0.0;
-      s_v = ctl->v;
-      __threadfence_block();
-      s_k0_ready = 1;
+      if (kFeat) {
+        __threadfence();
+        atomicExch(&ctl->feat_sides, 1);
+      } else {
+        s_v = ctl->v;
+        __threadfence_block();
+        s_k0_ready = 1;
+      }
     }
     if (ok && cls < 0) {
       cls = wait_label(ctl);
@@ -1856,9 +1925,10 @@ int cg_grid(int requested) {
     struct K {
       const void* f;
       size_t smem;
-    } ks[9] = {{(const void*)k_cg32<false, false>, ring_smem_bytes<float>()},
+    } ks[10] = {{(const void*)k_cg32<false, false>, ring_smem_bytes<float>()},
                {(const void*)k_cg64<false, false>, ring_smem_bytes<double>()},
-               {(const void*)k_stage1, ring_smem_bytes<float>()},
+               {(const void*)k_stage1<false>, ring_smem_bytes<float>()},
+               {(const void*)k_stage1<true>, ring_smem_bytes<float>()},
                {(const void*)k_cg32<true, false>, ring_smem_bytes<float>()},
                {(const void*)k_cg64<true, false>, ring_smem_bytes<double>()},
                {(const void*)k_cg32<false, true>, ring_smem_bytes<float>()},
@@ -1888,7 +1958,6 @@ int cg_grid(int requested) {
 
 const void* cg32_kernel() { return (const void*)k_cg32<false, false>; }
 const void* cg64_kernel() { return (const void*)k_cg64<false, false>; }
-const void* stage1_kernel() { return (const void*)k_stage1; }
 
 cudaError_t launch_cg32(const Launch& L, int mode, int slot) {
   CgArgs a = make_args(L, slot, mode);
@@ -1928,7 +1997,11 @@ cudaError_t launch_stage1(const Launch& L, const mpcg_sample_t& S, const mpcg_op
   void* args[] = {&sa};
   const int g = cg_grid(L.grid_req);
   if (g <= 0) return cudaErrorInvalidConfiguration;
-  return cudaLaunchCooperativeKernel((const void*)k_stage1, dim3(g), dim3(kTmaThreads), args,
+  // (a grid asked for, repeated searches, and float sums, whose tree has the
+  // blocks as leaves, keep the one-warp-a-block search)
+  const bool feat = L.d.n <= kFeatBlockN && g >= 2 && L.grid_req == 0 && o.bfs_starts <= 1 && !o.acc32;
+  const void* k = feat ? (const void*)k_stage1<true> : (const void*)k_stage1<false>;
+  return cudaLaunchCooperativeKernel(k, dim3(g), dim3(kTmaThreads), args,
                                     ring_smem_bytes<float>(), L.st);
 }
 

@@ -33,7 +33,7 @@
 // part of the features, so the 2BFS block never waits.
 #include <math.h>
 
-#include "bfs_block.cuh"
+#include "feature_block.cuh"
 #include "internal.h"
 
 namespace mpcg {
@@ -370,26 +370,6 @@ __device__ __forceinline__ void cl_spmv(const ClusterArgs& a, const ClShared& S,
 // ---------------------------------------------------------------------------------------
 // Algorithm II: the 2BFS block and the vote
 // ---------------------------------------------------------------------------------------
-// The vote from the features in the control block, by one warp; publishes
-// the label (or the failure).
-__device__ __noinline__ void cl_vote(const KnnSpec& knn, Ctl* ctl) {
-  const volatile Ctl* c = ctl;
-  const double chi[4] = {(double)c->n, (double)c->nnz, (double)c->pdiam, c->v};
-  const int t = knn_warp(knn, chi);
-  if ((threadIdx.x & 31) == 0) {
-    if (t >= 0) {
-      ctl->cls = t;
-      ctl->eps1 = pow10_neg(t);
-    } else {
-      set_status(ctl, MPCG_ERR_INVALID_ARG);  // invalid query, sample or label
-    }
-    ctl->t_features = globaltimer();
-    __threadfence();
-    atomicExch(&ctl->eps1_ready, t >= 0 ? t + 1 : -1);
-  }
-  __syncwarp();
-}
-
 // One side of the features is complete (called by a whole warp).  The second
 // of the two sides to say so runs the vote.
 __device__ __forceinline__ void cl_feature_ready(const KnnSpec& knn, Ctl* ctl) {
@@ -399,47 +379,16 @@ __device__ __forceinline__ void cl_feature_ready(const KnnSpec& knn, Ctl* ctl) {
     second = atomicAdd(&ctl->feat_sides, 1);
     __threadfence();
   }
-  if (__shfl_sync(0xffffffffu, second, 0) == 1) cl_vote(knn, ctl);
+  if (__shfl_sync(0xffffffffu, second, 0) == 1) feature_vote(knn, ctl);
 }
 
-// The block's own barrier as the group barrier of the 2BFS routines.
-struct BlockSync {
-  static constexpr bool kWholeBlock = true;
-  static constexpr bool kNarrow = false;
-  static constexpr bool kHelpers = false;
-  Ctl* ctl;
-  __device__ bool operator()() {
-    __shared__ int s_ok;
-    __syncthreads();
-    if (threadIdx.x == 0) s_ok = volatile_status(ctl) == 0 && !poll_cancel(ctl);
-    __syncthreads();
-    return s_ok != 0;
-  }
-};
-
 __device__ __noinline__ void cl_bfs(const ClusterArgs& a, unsigned char* smem) {
-  Ctl* ctl = a.ctl;
-  int32_t* const gq[4] = {a.g.fq0, a.g.fq1, a.g.fq2, a.g.fq3};
-  const BlockGraph g{a.rp, a.col, a.slice_ptr, a.slice_w, a.scol, a.n, ctl->col16};
-  const BlockBfs b = block_bfs_layout(g, smem, a.smem_bytes, reinterpret_cast<uint32_t*>(a.g.ckey), gq, ctl);
-  int pd = 0, tv = 0;
-  bool ok = block_pseudo_diameter(b, &pd, &tv);
-  __syncthreads();
-  if (ok) {
-    if (threadIdx.x == 0) {
-      ctl->pdiam = pd;
-      ctl->far_t = tv;
-      ctl->reached = a.n;
-      ctl->connected = 1;
-    }
-  } else {  // more than one component (or an error, which the group barrier reports)
-    BlockSync sync{ctl};
-    ok = pseudo_diameter_run<BlockSync, false>(a.g, a.d1, a.d2, threadIdx.x, kClThreads, sync);
-  }
+  const bool ok = block_pdiam_any(a.ctl, a.rp, a.col, a.slice_ptr, a.slice_w, a.scol, a.n, a.g, a.d1, a.d2, smem,
+                                  a.smem_bytes);
   __syncthreads();
   if (threadIdx.x < 32) {
-    if (ok) cl_feature_ready(a.knn, ctl);
-    else if (threadIdx.x == 0) atomicExch(&ctl->eps1_ready, -1);
+    if (ok) cl_feature_ready(a.knn, a.ctl);
+    else if (threadIdx.x == 0) atomicExch(&a.ctl->eps1_ready, -1);
   }
 }
 

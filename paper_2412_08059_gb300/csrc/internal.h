@@ -58,7 +58,6 @@ cudaError_t launch_promote(const Launch& L, double* x);
 // Fused stage 1 of Algorithm II: 2BFS + k0 iterations + kNN + CG to eps1.
 cudaError_t launch_stage1(const Launch& L, const mpcg_sample_t& S, const mpcg_options_t& o,
                           int slot, int bfs_slot);
-const void* stage1_kernel();
 const void* cg32_kernel();
 const void* cg64_kernel();
 int cg_grid(int requested);
