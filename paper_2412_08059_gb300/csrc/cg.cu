@@ -847,7 +847,7 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_cg32(CgArgs a) {
     if (lead) {
       const double rs = kTrue ? trr : rr;  // the stop test's r^T r
       int dec = kGo;
-      if (isnan(rr) || isnan(rs)) dec = kNan;
+      if (bits_nan(rr) || bits_nan(rs)) dec = kNan;
       else if (stop_pass(thr, rs) || it >= limit || (a.mode == kCgK0 && rr == 0.0) ||
                (kTrue && rr <= kStagnationRR * rs))
         dec = kStop;
@@ -888,8 +888,8 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_cg32(CgArgs a) {
       const double dq = cgrid_total(block_ff(pdq, S, f32), a.partials, red, ctl, a.slot, round, S, ok, f32);
       if (lead) {
         int dec = kGo;
-        if (!isfinite(dq)) dec = kNan;
-        else if (!(dq > 0.0)) dec = kBroke;  // stage 1 ends here; x and r are unchanged
+        if (!bits_finite(dq)) dec = kNan;
+        else if (!bits_positive(dq)) dec = kBroke;  // stage 1 ends here; x and r are unchanged
         else S.alpha = (float)((kPc ? rz : rr) / dq);
         S.dec = dec;
         if (dec == kNan && lead0) set_status(ctl, MPCG_ERR_NAN);
@@ -915,7 +915,7 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_cg32(CgArgs a) {
         rzn = cgrid_total(block_ff(prz, S, f32), a.partials, red, ctl, a.slot, round, S, ok, f32);
       if (lead) {
         int dec = kGo;
-        if (!isfinite(rrn) || (kPc && !isfinite(rzn))) {
+        if (!bits_finite(rrn) || (kPc && !bits_finite(rzn))) {
           dec = kNan;
           if (lead0) set_status(ctl, MPCG_ERR_NAN);
         } else {
@@ -1246,9 +1246,9 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_cg64(CgArgs a) {
           }
         }
       } else if (kind == kIterate) {
-        if (!isfinite(tot)) {
+        if (!bits_finite(tot)) {
           failed = MPCG_ERR_NAN;
-        } else if (!(tot > 0.0)) {
+        } else if (!bits_positive(tot)) {
           failed = MPCG_ERR_BREAKDOWN;
         } else {
           S.val = (kPc ? rz : rr) / tot;  // alpha
@@ -1275,7 +1275,7 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_cg64(CgArgs a) {
       if constexpr (kPc)
         rzn = cgrid_total(block_d(przl, S), a.partials, red, ctl, a.slot, round, S, ok);
       if (lead) {
-        if (!isfinite(rrn) || (kPc && !isfinite(rzn))) {
+        if (!bits_finite(rrn) || (kPc && !bits_finite(rzn))) {
           failed = MPCG_ERR_NAN;
           S.dec = kDone;
         } else {
@@ -1326,7 +1326,7 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_cg64(CgArgs a) {
           failed = MPCG_ERR_CANCELLED;
           set_status(ctl, MPCG_ERR_CANCELLED);
           nk = kDone;
-        } else if (isnan(rr)) {
+        } else if (bits_nan(rr)) {
           failed = MPCG_ERR_NAN;
           nk = kDone;
         } else if (kTrue) {
@@ -1624,12 +1624,12 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_stage1(Stage1Args sa) {
       if (lead0 && cw != 0) {  // the caller cancelled; the other blocks stop at their next wait
         dec = kFailed;
         set_status(ctl, MPCG_ERR_CANCELLED);
-      } else if (isnan(rr)) {
+      } else if (bits_nan(rr)) {
         dec = kFailed;
         if (lead0) set_status(ctl, MPCG_ERR_NAN);
       } else {
-        if (in_k0 && (it >= min(k0, max1) || rr == 0.0 || rr <= s_lo[16] ||
-                      (rr <= s_hi[16] && stop_measure(rr, bnorm, rel) <= eps2))) {
+        if (in_k0 && (it >= min(k0, max1) || dbits(rr) == 0 || dbits(rr) <= dbits(s_lo[16]) ||
+                      (dbits(rr) <= dbits(s_hi[16]) && stop_measure(rr, bnorm, rel) <= eps2))) {
           in_k0 = 0;  // end of the k0 phase: v of Eq. (13) for the kNN
           if (lead0) {
             ctl->k0_done = k0done;
@@ -1651,7 +1651,7 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_stage1(Stage1Args sa) {
           // the lowest present class not met yet, none is met this iteration.
           bool fresh = false;
           const unsigned open = cmask & ~met;
-          if (open && rr <= s_hi[__ffs(open) - 1]) {
+          if (open && dbits(rr) <= dbits(s_hi[__ffs(open) - 1])) {
             for (int t = 0; t < 16; ++t) {
               if (!((open >> t) & 1u)) continue;
               if (rr <= s_lo[t] ||
@@ -1724,10 +1724,10 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_stage1(Stage1Args sa) {
       const double dq = cgrid_total(block_ff(pdq, S, f32), a.partials, red, ctl, a.slot, round, S, ok, f32);
       if (lead) {
         int d2 = kGoOn;
-        if (!isfinite(dq)) {
+        if (!bits_finite(dq)) {
           d2 = kFailed;
           if (lead0) set_status(ctl, MPCG_ERR_NAN);
-        } else if (!(dq > 0.0)) {
+        } else if (!bits_positive(dq)) {
           d2 = kBrokeDown;  // stage 1 ends here; x~ and r are unchanged
         } else {
           S.alpha = (float)(rr / dq);
@@ -1764,7 +1764,7 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_stage1(Stage1Args sa) {
         int d3 = kGoOn;
         if (label < 0) {
           d3 = kFailed;
-        } else if (!isfinite(rrn)) {
+        } else if (!bits_finite(rrn)) {
           d3 = kFailed;
           if (lead0) set_status(ctl, MPCG_ERR_NAN);
         } else {

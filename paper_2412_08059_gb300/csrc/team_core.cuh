@@ -996,14 +996,15 @@ static __device__ bool sys_cg32(Team& t, const BatchSys& s, int mode, int& red, 
   const int limit = mode == kCgK0 ? min(ctl->k0, ctl->max1) : ctl->max1;
   const int it_start = it;
   // Every thread holds the team sums (identical in every block), so every
-  // thread takes the loop's decisions itself, with no broadcast barrier.
+  // thread takes the loop's decisions itself (integer tests), with no
+  // broadcast barrier.
   const StopThr thr = stop_thr(eps, bnorm, rel);
   double vsum = 0.0;  // thread 0
   int k0done = 0, broke = 0, suspended = 0;
   while (true) {
     int dec = kBGo;
-    if (isnan(rr)) dec = kBNan;
-    else if (stop_pass(thr, rr) || it >= limit || (mode == kCgK0 && rr == 0.0)) dec = kBStop;
+    if (bits_nan(rr)) dec = kBNan;
+    else if (stop_pass(thr, rr) || it >= limit || (mode == kCgK0 && dbits(rr) == 0)) dec = kBStop;
     else if (mode != kCgK0 && it - it_start >= budget) dec = kBSuspend;
     if (dec == kBSuspend) {
       suspended = 1;
@@ -1032,8 +1033,8 @@ static __device__ bool sys_cg32(Team& t, const BatchSys& s, int mode, int& red, 
     double dq;
     if (!team_sum_ff(t, pdq, s.w.partials, red, dq, f32)) return false;
     dec = kBGo;
-    if (!isfinite(dq)) dec = kBNan;
-    else if (!(dq > 0.0)) dec = kBBroke;
+    if (!bits_finite(dq)) dec = kBNan;
+    else if (!bits_positive(dq)) dec = kBBroke;
     if (dec == kBNan) {
       if (lead0) set_status(ctl, MPCG_ERR_NAN);
       break;
@@ -1042,7 +1043,11 @@ static __device__ bool sys_cg32(Team& t, const BatchSys& s, int mode, int& red, 
       broke = 1;
       break;
     }
-    const float alpha = (float)(rr / dq);
+    // One thread divides: an FP64 division in every warp would queue ten times
+    // as long on the pipe as the barrier takes.
+    if (lead) t.S->fval[0] = (float)(rr / dq);
+    __syncthreads();
+    const float alpha = t.S->fval[0];
     // P2: x += alpha d_k, r -= alpha q, r^T r
     FF prr{0.f, 0.f};
     team_rows(
@@ -1055,12 +1060,14 @@ static __device__ bool sys_cg32(Team& t, const BatchSys& s, int mode, int& red, 
         });
     double rrn;
     if (!team_sum_ff(t, prr, s.w.partials, red, rrn, f32)) return false;
-    if (!isfinite(rrn)) {
+    if (!bits_finite(rrn)) {
       if (lead0) set_status(ctl, MPCG_ERR_NAN);
       break;
     }
     if (lead && mode == kCgK0) vsum += sqrt(rrn) / sqrt(rr);  // Eq. (13) ratio
-    beta = (float)(rrn / rr);
+    if (lead) t.S->fval[1] = (float)(rrn / rr);
+    __syncthreads();
+    beta = t.S->fval[1];
     rr = rrn;
     if (mode == kCgK0) ++k0done;
     parity ^= 1;
@@ -1165,8 +1172,8 @@ static __device__ bool sys_cg64(Team& t, const BatchSys& s, int from_zero, int& 
       } else if (kind == kPIterate) {
         int dec = kBGo;
         if (lead) {
-          if (!isfinite(tot)) dec = kBNan;
-          else if (!(tot > 0.0)) dec = kBBreakdown;
+          if (!bits_finite(tot)) dec = kBNan;
+          else if (!bits_positive(tot)) dec = kBBreakdown;
           else t.S->val[2] = rr / tot;
         }
         dec = bcast_dec(t, dec);
@@ -1188,7 +1195,7 @@ static __device__ bool sys_cg64(Team& t, const BatchSys& s, int from_zero, int& 
         if (!team_sum_d(t, pr, s.w.partials, red, rrn)) return false;
         dec = kBGo;
         if (lead) {
-          if (!isfinite(rrn)) dec = kBNan;
+          if (!bits_finite(rrn)) dec = kBNan;
           else t.S->val[3] = rrn / rr;
         }
         dec = bcast_dec(t, dec);
@@ -1227,7 +1234,7 @@ static __device__ bool sys_cg64(Team& t, const BatchSys& s, int from_zero, int& 
     // loop head: the stop test on the recursive residual
     int dec = kBGo;
     if (lead) {
-      if (isnan(rr)) dec = kBNan;
+      if (bits_nan(rr)) dec = kBNan;
       else if (stop_pass(thr2, rr)) dec = kBStop;
       else if (it >= max2) dec = kBCap;
       else if (it - it_start >= budget) dec = kBSuspend;
