@@ -191,7 +191,7 @@ int32_t mpcg_solve(const mpcg_csr_t* A, const double* b, double* x, const mpcg_s
   const bool small = opts->grid_blocks == 0 && !L.precond && !L.true_res && !opts->stage1_only &&
                      !opts->acc32 && !(auto_eps1 && opts->bfs_starts > 1) && cluster_fits(L.d);
   if (small) {
-    if ((e = launch_cluster(L, b, x, sample, *opts, fp64_only ? 2 : (auto_eps1 ? 1 : 0))) != cudaSuccess)
+    if ((e = launch_cluster(L, b, x, sample, *opts, fp64_only ? 2 : (auto_eps1 ? 1 : 0), kSlotPd)) != cudaSuccess)
       return cuda_status(e);
     return cuda_status(launch_finalize(L, res, nullptr));
   }

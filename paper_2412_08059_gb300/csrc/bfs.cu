@@ -2,8 +2,7 @@
 // (the routines are in bfs_core.cuh and bfs_block.cuh): the 2BFS
 // pseudo-diameter, with the per-component rule, by one block or in one
 // cooperative launch, and a plain BFS.
-#include "bfs_block.cuh"
-#include "bfs_core.cuh"
+#include "feature_block.cuh"
 #include "internal.h"
 
 namespace mpcg {
@@ -14,33 +13,15 @@ namespace mpcg {
 // together) and 5.3 us at 1,000, so long thin graphs gain most (4096 x 64
 // grid, 4,158 levels: 21.7 ms by the grid, 11.4 here).  A frontier that grows
 // like a cube's or a random graph's is soon wide and better off with the
-// grid: the search gives up (see PdArgs) and k_pdiam, launched behind it,
+// grid: the search gives up (feature_block.cuh) and k_pdiam, launched behind it,
 // does the work; that one leaves at once when this one has succeeded.
 constexpr int kPdThreads = 1024;
 constexpr int kPdSmem = 200 * 1024;
-struct PdArgs {
-  BlockGraph g;
-  BfsGraph q;  // queues and scratch
-  int wide, grow;  // limits of the frontier (BlockBfs)
-};
-__global__ void __launch_bounds__(kPdThreads, 1) k_pdiam_block(PdArgs a) {
+__global__ void __launch_bounds__(kPdThreads, 1) k_pdiam_block(BlockGraph g, BfsGraph q) {
   extern __shared__ __align__(16) unsigned char pd_smem[];
-  Ctl* ctl = a.q.ctl;
-  if (volatile_status(ctl) != 0) return;
-  a.g.c16 = ctl->col16;
-  int32_t* const gq[4] = {a.q.fq0, a.q.fq1, a.q.fq2, a.q.fq3};
-  BlockBfs b = block_bfs_layout(a.g, pd_smem, kPdSmem, reinterpret_cast<uint32_t*>(a.q.ckey), gq, ctl);
-  b.wide = a.wide;
-  b.grow = a.grow;
-  int pd = 0, tv = 0;
-  if (!block_pseudo_diameter(b, &pd, &tv)) return;
-  if (threadIdx.x == 0) {
-    ctl->pdiam = pd;
-    ctl->far_t = tv;
-    ctl->reached = a.g.n;
-    ctl->connected = 1;
-    ctl->pd_done = 1;
-  }
+  if (volatile_status(q.ctl) != 0) return;
+  g.c16 = q.ctl->col16;
+  block_pdiam(g, q, pd_smem, kPdSmem);
 }
 
 __global__ void __launch_bounds__(kCgThreads, 1) k_pdiam(BfsGraph g, int32_t* d1, int32_t* d2,
@@ -82,29 +63,14 @@ BfsGraph bfs_graph(const Launch& L) {
 
 const void* bfs_kernel() { return (const void*)k_pdiam; }
 
-// Sizes the one-block search takes.  Up to kPdSmallN vertices a frontier of up
-// to 2,048 entries: a whole cube is then no slower than by the grid (features
-// of 24^3: 0.58 ms against 0.67; of 32^3 0.95 against 0.84).  Past it a
-// frontier of 128 + 8 level entries, at most 1,280: a 2-D grid (2 level) of up
-// to kPdMaxN vertices stays within that (512 x 512: 5.5 against 5.9 ms), a
-// cube leaves it at level 16 (level^2), some 50 us into a search of a
-// millisecond.  A larger square grid would leave it late (700 x 700: 12.8 ms
-// against 8.8), so larger graphs go to the grid at once.
-constexpr int kPdMaxN = 300000;
-constexpr int kPdSmallN = 16384;
-
 cudaError_t launch_pseudo_diameter(const Launch& L, int slot, int starts) {
   BfsGraph g = bfs_graph(L);
   // (repeated searches, and a grid asked for, keep to the grid-wide kernel)
   if (L.d.n <= kPdMaxN && starts <= 1 && L.grid_req == 0) {
     cudaError_t e = cudaFuncSetAttribute(k_pdiam_block, cudaFuncAttributeMaxDynamicSharedMemorySize, kPdSmem);
     if (e != cudaSuccess) return e;
-    PdArgs a{};
-    a.g = BlockGraph{L.A->row_ptr, L.A->col, L.ws.slice_ptr, L.ws.slice_w, L.ws.scol, L.d.n, 0};
-    a.q = g;
-    a.wide = L.d.n <= kPdSmallN ? 2048 : 1280;
-    a.grow = L.d.n <= kPdSmallN ? 0 : 8;
-    k_pdiam_block<<<1, kPdThreads, kPdSmem, L.st>>>(a);
+    const BlockGraph b{L.A->row_ptr, L.A->col, L.ws.slice_ptr, L.ws.slice_w, L.ws.scol, L.d.n, 0};
+    k_pdiam_block<<<1, kPdThreads, kPdSmem, L.st>>>(b, g);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   int32_t* d1 = L.ws.dist;

@@ -19,6 +19,8 @@
 // jumping) and 2BFS runs in every component at once from multi-source
 // frontiers; l~ is the largest second-BFS level.
 #pragma once
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace mpcg {
@@ -54,6 +56,24 @@ struct GridSync {
   int slot;
   unsigned long long round;
   __device__ bool operator()() { return grid_barrier(ctl, slot, round); }
+  __device__ int first() const { return 0; }               // the group's first block
+  __device__ int* scratch() const { return nullptr; }      // no memory of its own for narrow levels
+};
+
+// Whole blocks `first_block` .. `first_block` + `blocks` - 1 of the grid; the
+// narrow levels' memory is the caller's (kNarrowScratch ints).
+struct BlockGroupSync {
+  static constexpr bool kWholeBlock = true;
+  static constexpr bool kNarrow = true;
+  static constexpr bool kHelpers = false;
+  Ctl* ctl;
+  int slot;
+  unsigned long long round;
+  int first_block, blocks;
+  int* mem;
+  __device__ bool operator()() { return grid_barrier(ctl, slot, round, blocks); }
+  __device__ int first() const { return first_block; }
+  __device__ int* scratch() const { return mem; }
 };
 
 // One warp per block: lane 0 arrives on the counter and polls (bounded).
@@ -64,6 +84,8 @@ struct WarpGroupSync {
   Ctl* ctl;
   int slot;
   unsigned long long round;
+  __device__ int first() const { return 0; }
+  __device__ int* scratch() const { return nullptr; }
   __device__ bool operator()() {
     __syncwarp();
     round += 1;
@@ -437,6 +459,9 @@ __device__ bool bfs_run(const BfsGraph& g, int32_t* dist, int sources, int src, 
 constexpr int kNarrowItems = 64;
 constexpr int kNarrowHash = 2048;  // shared-memory set of the level's claims (load <= 1/2)
 constexpr int kNarrowHashDeg = 16; // levels with a wider row claim by compare-and-swap
+// Memory of the one-warp levels: the current and next frontiers, the set, and
+// the block's copy of the mode word.
+constexpr int kNarrowScratch = 4 * kNarrowItems + kNarrowHash + 4;
 enum { kNmResume = 1, kNmDone = 2 };
 
 // Whether the mode word ends the wait of the group left at level L: the
@@ -447,9 +472,9 @@ __device__ __forceinline__ bool nm_ends(int m, int L) {
 }
 
 template <bool kBlk>
-__device__ int nm_wait(Ctl* ctl, int L, volatile int* s_mode) {
+__device__ int nm_wait(Ctl* ctl, int L, volatile int* s_mode, int first) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const bool poller = !kBlk || warp == (blockIdx.x == 0 ? 1 : 0);
+  const bool poller = !kBlk || warp == ((int)blockIdx.x == first ? 1 : 0);
   int m = 0;
   if (lane == 0) {
     const unsigned long long t0 = globaltimer();
@@ -699,18 +724,23 @@ __device__ bool bfs_dual(const BfsGraph& g, int32_t* dA, int32_t* dB, int srcA, 
     if constexpr (Sync::kNarrow) {
     if (sa + sb <= kNarrowItems) {
       // ---- narrow frontiers: one warp runs the next levels alone ----
-      __shared__ int s_nbuf[4][kNarrowItems];  // the warp's current and next frontiers
-      __shared__ int s_hash[kNarrowHash];      // the warp's set of a level's claims
-      __shared__ volatile int s_nmode;         // whole-block groups: the block's copy of the mode word
+      int* nmem;
+      if constexpr (std::is_same<Sync, BlockGroupSync>::value) {
+        nmem = sync.scratch();
+      } else {
+        __shared__ int s_narrow[kNarrowScratch];
+        nmem = s_narrow;
+      }
+      int (*const nbuf)[kNarrowItems] = reinterpret_cast<int (*)[kNarrowItems]>(nmem);
+      int* const nhash = nmem + 4 * kNarrowItems;
+      volatile int* const nmode = nmem + 4 * kNarrowItems + kNarrowHash;  // whole-block groups
       if constexpr (Sync::kWholeBlock) {
-        if (threadIdx.x == 0) s_nmode = 0;
+        if (threadIdx.x == 0) *nmode = 0;
         __syncthreads();  // every thread of the block is here (same level, same decision)
       }
       int resume;
       if (tid < 32) {
-        resume = narrow_levels(g, dA, dB, level, sa, sb, la, lb, reached,
-                               reinterpret_cast<int (*)[kNarrowItems]>(&s_nbuf[0][0]),
-                               reinterpret_cast<int (*)[kNarrowItems]>(&s_nbuf[2][0]), s_hash);
+        resume = narrow_levels(g, dA, dB, level, sa, sb, la, lb, reached, nbuf, nbuf + 2, nhash);
         if (lane == 0) {
           ctl->nla = la;
           ctl->nlb = lb;
@@ -720,7 +750,7 @@ __device__ bool bfs_dual(const BfsGraph& g, int32_t* dA, int32_t* dB, int srcA, 
         }
         __syncwarp();
       } else {
-        const int m = nm_wait<Sync::kWholeBlock>(ctl, level, &s_nmode);
+        const int m = nm_wait<Sync::kWholeBlock>(ctl, level, nmode, sync.first());
         if (m == -1) return false;
         la = *reinterpret_cast<volatile int*>(&ctl->nla);
         lb = *reinterpret_cast<volatile int*>(&ctl->nlb);

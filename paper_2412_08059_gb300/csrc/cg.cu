@@ -1404,14 +1404,24 @@ __device__ __noinline__ bool stage1_pdiam(const BfsGraph g, int32_t* d1, int32_t
   return ok;
 }
 
-// The feature block: the 2BFS in this block, then v (bounded wait for block 0's
-// consumers) and the vote.  Every block of the launch is resident (cooperative
-// launch), so the wait ends.
-__device__ __noinline__ void stage1_feature_block(const Stage1Args& sa, unsigned char* smem) {
+// kFeat: the last kFeatBlocks blocks of the grid run the 2BFS and the vote; the
+// others run CG with fifteen consumer warps.  The search by one warp a block
+// cost 5 to 17 us a level and slowed the iterations beside it: 301 x 203 grid
+// (502 levels) 19 us an iteration against 9.5 without it, label at 2.3 ms
+// against 1.0 here (25,000 rows less: 200 x 250); 128^3 (381 levels) 46 us
+// against 38 on the remaining 136 blocks, stage 1 6.9 against 5.7 ms.  Eight
+// blocks are too few for wide levels (random 8-regular graph of 2^20 vertices,
+// 2BFS alone: 4.8 ms, 2.4 by sixteen), thirty-two cost CG a fifth of the chip.
+constexpr int kFeatBlocks = 16;
+// The feature blocks: the 2BFS; then, in the first, v (bounded wait for block 0's consumers) and the vote.  Every block
+// of the launch is resident (cooperative launch), so the wait ends.
+__device__ __noinline__ void stage1_feature_block(const Stage1Args& sa, unsigned char* smem, int first) {
   const CgArgs& a = sa.a;
   Ctl* ctl = a.ctl;
-  const bool ok = block_pdiam_any(ctl, a.rp, a.col, a.slice_ptr, a.slice_w, a.scol, a.n, sa.g, sa.d1, sa.d2, smem,
-                                  (int)ring_smem_bytes<float>());
+  const BlockGraph g{a.rp, a.col, a.slice_ptr, a.slice_w, a.scol, a.n, ctl->col16};
+  const bool ok = feature_pdiam(g, sa.g, sa.d1, sa.d2, smem, (int)ring_smem_bytes<float>(), sa.bfs_slot, first,
+                                kFeatBlocks);
+  if ((int)blockIdx.x != first) return;
   __syncthreads();
   if (threadIdx.x >= 32) return;
   int have_v = 0;
@@ -1435,13 +1445,6 @@ __device__ __noinline__ void stage1_feature_block(const Stage1Args& sa, unsigned
   else if (threadIdx.x == 0) atomicExch(&ctl->eps1_ready, -1);
 }
 
-// kFeat: one block, the last of the grid, runs the 2BFS alone (bfs_block.cuh)
-// and the vote; the others run CG with fifteen consumer warps.  For systems of
-// up to kFeatBlockN rows: the one-warp-a-block search costs 5 us a level there
-// and slows the iterations beside it from 9.5 to 19 us (301 x 203 grid, 502
-// levels; this form: 3 us a level, 9.5 us an iteration).  Wide graphs of more
-// rows are too much work for one block.
-constexpr int kFeatBlockN = 80000;
 template <bool kFeat>
 __global__ void __launch_bounds__(kTmaThreads, 1) k_stage1(Stage1Args sa) {
   constexpr int NC = kFeat ? kNC : kNC1;
@@ -1461,10 +1464,10 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_stage1(Stage1Args sa) {
     s_help = kHelpNone;
     s_hl.cmd = 0;
   }
-  const int nb = kFeat ? (int)gridDim.x - 1 : (int)gridDim.x;
+  const int nb = kFeat ? (int)gridDim.x - kFeatBlocks : (int)gridDim.x;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (kFeat && (int)blockIdx.x == nb) {
-    stage1_feature_block(sa, reinterpret_cast<unsigned char*>(smem));
+  if (kFeat && (int)blockIdx.x >= nb) {
+    stage1_feature_block(sa, reinterpret_cast<unsigned char*>(smem), nb);
     return;
   }
   Ring<float> R;
@@ -1999,7 +2002,7 @@ cudaError_t launch_stage1(const Launch& L, const mpcg_sample_t& S, const mpcg_op
   if (g <= 0) return cudaErrorInvalidConfiguration;
   // (a grid asked for, repeated searches, and float sums, whose tree has the
   // blocks as leaves, keep the one-warp-a-block search)
-  const bool feat = L.d.n <= kFeatBlockN && g >= 2 && L.grid_req == 0 && o.bfs_starts <= 1 && !o.acc32;
+  const bool feat = g >= 4 * kFeatBlocks && L.grid_req == 0 && o.bfs_starts <= 1 && !o.acc32;
   const void* k = feat ? (const void*)k_stage1<true> : (const void*)k_stage1<false>;
   return cudaLaunchCooperativeKernel(k, dim3(g), dim3(kTmaThreads), args,
                                     ring_smem_bytes<float>(), L.st);

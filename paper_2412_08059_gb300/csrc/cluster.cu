@@ -26,11 +26,10 @@
 // stored order by fused multiply-adds, float-float inner products in single
 // precision, alpha and beta the double quotients rounded once to float.
 //
-// Algorithm II: a second cluster of the same launch runs the 2BFS in one of
-// its blocks meanwhile, and the iterations past k0 are speculative with
+// Algorithm II: a second cluster of the same launch runs the 2BFS meanwhile, and the iterations past k0 are speculative with
 // snapshots at every candidate eps1, as in k_stage1.  The kNN vote is run by
-// whichever of the two, the 2BFS block or the cluster, comes second with its
-// part of the features, so the 2BFS block never waits.
+// whichever of the two clusters comes second with its part of the features,
+// so the 2BFS never waits for CG.
 #include <math.h>
 
 #include "feature_block.cuh"
@@ -66,7 +65,7 @@ struct ClusterArgs {
   BfsGraph g;    // Algorithm II
   int32_t *d1, *d2;
   KnnSpec knn;
-  int smem_bytes;
+  int smem_bytes, bfs_slot;
 };
 
 // ---------------------------------------------------------------------------------------
@@ -368,7 +367,7 @@ __device__ __forceinline__ void cl_spmv(const ClusterArgs& a, const ClShared& S,
 }
 
 // ---------------------------------------------------------------------------------------
-// Algorithm II: the 2BFS block and the vote
+// Algorithm II: the 2BFS cluster and the vote
 // ---------------------------------------------------------------------------------------
 // One side of the features is complete (called by a whole warp).  The second
 // of the two sides to say so runs the vote.
@@ -383,10 +382,10 @@ __device__ __forceinline__ void cl_feature_ready(const KnnSpec& knn, Ctl* ctl) {
 }
 
 __device__ __noinline__ void cl_bfs(const ClusterArgs& a, unsigned char* smem) {
-  const bool ok = block_pdiam_any(a.ctl, a.rp, a.col, a.slice_ptr, a.slice_w, a.scol, a.n, a.g, a.d1, a.d2, smem,
-                                  a.smem_bytes);
+  const BlockGraph g{a.rp, a.col, a.slice_ptr, a.slice_w, a.scol, a.n, a.ctl->col16};
+  const bool ok = feature_pdiam(g, a.g, a.d1, a.d2, smem, a.smem_bytes, a.bfs_slot, 0, kClBlocks);
   __syncthreads();
-  if (threadIdx.x < 32) {
+  if (blockIdx.x == 0 && threadIdx.x < 32) {
     if (ok) cl_feature_ready(a.knn, a.ctl);
     else if (threadIdx.x == 0) atomicExch(&a.ctl->eps1_ready, -1);
   }
@@ -402,8 +401,8 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
   __shared__ ClShared S;
   Ctl* ctl = a.ctl;
   const bool trivial = *reinterpret_cast<volatile int*>(&ctl->trivial) != 0;
-  if (a.mode == 1 && blockIdx.x < kClBlocks) {  // the 2BFS cluster: one block of it works
-    if (blockIdx.x == 0 && !trivial && volatile_status(ctl) == 0) cl_bfs(a, cl_smem);
+  if (a.mode == 1 && blockIdx.x < kClBlocks) {  // the 2BFS cluster
+    if (!trivial && volatile_status(ctl) == 0) cl_bfs(a, cl_smem);
     return;
   }
   const int rank = (int)(blockIdx.x & (kClBlocks - 1));
@@ -416,7 +415,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
     return;
   }
   // The blocks of the cluster leave together: block 0's view of the status
-  // decides for all (the 2BFS block may set it at any time).  The first
+  // decides for all (the 2BFS cluster may set it at any time).  The first
   // barrier makes sure that every block runs before its memory is written to.
   cl_sync();
   int red = 1;
@@ -1009,8 +1008,9 @@ bool cluster_fits(const Dims& d) {
 }
 
 cudaError_t launch_cluster(const Launch& L, const double* b, double* x, const mpcg_sample_t* S,
-                           const mpcg_options_t& o, int mode) {
+                           const mpcg_options_t& o, int mode, int bfs_slot) {
   ClusterArgs a{};
+  a.bfs_slot = bfs_slot;
   a.ctl = L.ws.ctl;
   a.slice_w = L.ws.slice_w;
   a.slice_ptr = L.ws.slice_ptr;
@@ -1032,7 +1032,7 @@ cudaError_t launch_cluster(const Launch& L, const double* b, double* x, const mp
   a.d2 = L.ws.dist2;
   if (mode == 1) a.knn = knn_spec(*S, o);
   size_t smem = cluster_smem(L.d, &a.rows_cap, &a.ent_cap);
-  if (mode == 1) smem = kClSmem;  // the 2BFS block's bitmaps and queues
+  if (mode == 1) smem = kClSmem;  // the 2BFS's bitmaps and queues
   a.smem_bytes = (int)smem;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[1];

@@ -223,12 +223,13 @@ __device__ __forceinline__ double ld_stream(const double* p) { return __ldcs(p);
 // Ordering: the block's writes are ordered before thread 0's release-add by
 // the CTA barrier; thread 0's acquire load, followed by the second CTA
 // barrier, orders every thread's later loads after all blocks' writes.
-__device__ __forceinline__ bool grid_barrier(Ctl* ctl, int slot, unsigned long long& round) {
+// `blocks` > 0: the barrier of that many blocks of the grid.
+__device__ __forceinline__ bool grid_barrier(Ctl* ctl, int slot, unsigned long long& round, int blocks = 0) {
   __shared__ int s_ok;
   __syncthreads();
   round += 1;
   if (threadIdx.x == 0) {
-    const unsigned long long target = round * (unsigned long long)gridDim.x;
+    const unsigned long long target = round * (unsigned long long)(blocks > 0 ? blocks : (int)gridDim.x);
     red_release_add(&ctl->bar[slot].v, 1ull);
     int ok = 1;
     if (ld_acquire(&ctl->bar[slot].v) < target) {

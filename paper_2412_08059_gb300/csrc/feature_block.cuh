@@ -27,45 +27,53 @@ static __device__ __noinline__ void feature_vote(const KnnSpec& knn, Ctl* ctl) {
   __syncwarp();
 }
 
-// The block's own barrier as the group barrier of the 2BFS routines.
-struct BlockSync {
-  static constexpr bool kWholeBlock = true;
-  static constexpr bool kNarrow = false;
-  static constexpr bool kHelpers = false;
-  Ctl* ctl;
-  __device__ bool operator()() {
-    __shared__ int s_ok;
-    __syncthreads();
-    if (threadIdx.x == 0) s_ok = volatile_status(ctl) == 0 && !poll_cancel(ctl);
-    __syncthreads();
-    return s_ok != 0;
-  }
-};
+// Sizes the one-block search takes (bfs_block.cuh) before the blocks of a
+// group, or of the grid, search together, and the frontiers at which it gives
+// up for them (entries of both searches).  Up to kPdSmallN vertices 2,048: a
+// whole cube is then no slower than by the grid (features of 24^3: 0.58 ms
+// against 0.67; of 32^3 0.95 against 0.84).  Past it 128 + 8 level, at most
+// 1,280: a 2-D grid (2 level) of up to kPdMaxN vertices stays within that (512 x
+// 512: 5.5 against 5.9 ms), a cube leaves it at level 16 (level^2), some 50 us
+// into a search of a millisecond.  A larger square grid would leave it late
+// (700 x 700: 12.8 ms against 8.8), so larger graphs are not tried.
+constexpr int kPdMaxN = 300000;
+constexpr int kPdSmallN = 16384;
 
-// l~ by the calling block, into the control block: the one-block search, or,
-// where the graph has more than one component, the group's routines over this
-// block.  False (in every thread) on an error or a cancel.
-static __device__ bool block_pdiam_any(Ctl* ctl, const int32_t* rp, const int32_t* col, const int32_t* slice_ptr,
-                                       const uint32_t* slice_w, const void* scol, int n, const BfsGraph& q,
-                                       int32_t* d1, int32_t* d2, unsigned char* smem, int smem_bytes) {
+// l~ by the calling block, into the control block (pd_done set).  False (in
+// every thread) if the graph has more than one component, its frontier grows
+// past the limits, or on an error or a cancel; then nothing is written.
+static __device__ bool block_pdiam(const BlockGraph& g, const BfsGraph& q, unsigned char* smem, int smem_bytes) {
+  Ctl* ctl = q.ctl;
   int32_t* const gq[4] = {q.fq0, q.fq1, q.fq2, q.fq3};
-  const BlockGraph g{rp, col, slice_ptr, slice_w, scol, n, ctl->col16};
-  const BlockBfs b = block_bfs_layout(g, smem, smem_bytes, reinterpret_cast<uint32_t*>(q.ckey), gq, ctl);
+  BlockBfs b = block_bfs_layout(g, smem, smem_bytes, reinterpret_cast<uint32_t*>(q.ckey), gq, ctl);
+  b.wide = g.n <= kPdSmallN ? 2048 : 1280;
+  b.grow = g.n <= kPdSmallN ? 0 : 8;
   int pd = 0, tv = 0;
-  bool ok = block_pseudo_diameter(b, &pd, &tv);
+  const bool ok = block_pseudo_diameter(b, &pd, &tv);
   __syncthreads();
-  if (ok) {
-    if (threadIdx.x == 0) {
-      ctl->pdiam = pd;
-      ctl->far_t = tv;
-      ctl->reached = n;
-      ctl->connected = 1;
-    }
-  } else {  // more than one component (or an error, which the group barrier reports)
-    BlockSync sync{ctl};
-    ok = pseudo_diameter_run<BlockSync, false>(q, d1, d2, threadIdx.x, blockDim.x, sync);
+  if (ok && threadIdx.x == 0) {
+    ctl->pdiam = pd;
+    ctl->far_t = tv;
+    ctl->reached = g.n;
+    ctl->connected = 1;
+    ctl->pd_done = 1;
   }
   return ok;
+}
+
+// l~ by a group of blocks of a launch that run beside the CG blocks: `blocks`
+// of them from `first` on.  The first tries the one-block search while the
+// others wait at the group's (bounded) barrier; where it gives up, they search
+// together.  False (in every thread) on an error or a cancel.
+static __device__ bool feature_pdiam(const BlockGraph& g, const BfsGraph& q, int32_t* d1, int32_t* d2,
+                                     unsigned char* smem, int smem_bytes, int slot, int first, int blocks) {
+  const int rank = (int)blockIdx.x - first;
+  if (rank == 0 && g.n <= kPdMaxN) block_pdiam(g, q, smem, smem_bytes);
+  BlockGroupSync sync{q.ctl, slot, 0ull, first, blocks, reinterpret_cast<int*>(smem)};
+  if (!sync()) return false;
+  if (*reinterpret_cast<volatile int*>(&q.ctl->pd_done)) return true;
+  return pseudo_diameter_run<BlockGroupSync, false>(q, d1, d2, rank * (int)blockDim.x + (int)threadIdx.x,
+                                                    blocks * (int)blockDim.x, sync);
 }
 
 }  // namespace mpcg

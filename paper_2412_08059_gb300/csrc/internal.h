@@ -65,7 +65,7 @@ int cg_grid(int requested);
 // cluster.cu: both stages of a small system in one cluster of blocks
 bool cluster_fits(const Dims& d);
 cudaError_t launch_cluster(const Launch& L, const double* b, double* x, const mpcg_sample_t* S,
-                           const mpcg_options_t& o, int mode);
+                           const mpcg_options_t& o, int mode, int bfs_slot);
 
 // bfs.cu
 BfsGraph bfs_graph(const Launch& L);
