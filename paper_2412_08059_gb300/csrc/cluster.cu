@@ -60,7 +60,7 @@ struct ClusterArgs {
   float* snap;
   int n, nslices;
   int mode;      // 0: Algorithm I, 1: Algorithm II, 2: double precision only
-  int rows_cap;  // rows a block has room for (the same in every block)
+  int rows_cap;  // rows of the gathered vector a block has room for (the same in every block)
   int ent_cap;   // stored entries a block has room for
   BfsGraph g;    // Algorithm II
   int32_t *d1, *d2;
@@ -81,6 +81,11 @@ __device__ __forceinline__ void cl_sync() {
   cl_arrive();
   cl_wait();
 }
+__device__ __forceinline__ uint32_t cl_rank() {
+  uint32_t r;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
 __device__ __forceinline__ uint32_t cl_map(uint32_t addr, uint32_t rank) {
   uint32_t r;
   asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
@@ -91,6 +96,9 @@ __device__ __forceinline__ void cl_ld(uint32_t addr, double& v) {
 }
 __device__ __forceinline__ void cl_ld(uint32_t addr, float& v) {
   asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr));
+}
+__device__ __forceinline__ void cl_st(uint32_t addr, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
 }
 __device__ __forceinline__ void cl_st(uint32_t addr, double v) {
   asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(addr), "d"(v) : "memory");
@@ -216,11 +224,36 @@ __device__ __forceinline__ double cl_total_ff(ClShared& S, int rank, int ns, int
 // ---------------------------------------------------------------------------------------
 // A block's part: the gathered vector, the entries' values and packed
 // columns (owner << 12 | row in the owner; rows_cap <= 3072).
+//
+// Where most entries lie in other blocks' rows (random graphs), a gather
+// through distributed shared memory costs 52 clocks a warp (32 lanes, up to 16
+// targets), and a row's gathers bound the iteration (n = 3,001 random tree:
+// 4,900 of 15,500 clocks).  (8-regular graph of 2,000 rows: 6.6 us a
+// double-precision iteration that way, 5.7 with whole copies; tree of 4,000
+// rows 7.9 and 7.2, in single precision 7.6 and 6.1.)  Up to kClRepN rows every block then keeps the whole
+// vector: the owner writes each value to all sixteen, the entries' owner is
+// the block itself, and a gather stays in its own shared memory.
+constexpr int kClRepN = 4096;
 struct ClMat {
   unsigned char* g;   // gathered vector: rows_cap values (float or double)
+  int base;           // first row of the block in g: 0, or its first row where g is whole
+  bool rep;           // g is whole in every block
   unsigned char* v;   // values of the entries (float or double)
   uint16_t* c;
 };
+
+// Publish the value of one of the block's rows (`local`) in the gathered vector.
+template <typename T>
+__device__ __forceinline__ void cl_put(const ClMat& M, int local, T v) {
+  T* g = reinterpret_cast<T*>(M.g) + M.base + local;
+  if (!M.rep) {
+    *g = v;
+    return;
+  }
+  const uint32_t addr = smem_addr(g);
+#pragma unroll
+  for (int o = 0; o < kClBlocks; ++o) cl_st(cl_map(addr, o), v);
+}
 
 __device__ __forceinline__ uint16_t cl_pack(int nslices, int c) {
   const int o = cl_owner(nslices, c >> 5);
@@ -234,7 +267,7 @@ __device__ __forceinline__ uint16_t cl_pack(int nslices, int c) {
 // they made a random tree's SpMV three times as long as its other rows need.
 template <typename T, int RPT>
 __device__ __forceinline__ void cl_load(const ClusterArgs& a, ClShared& S, const ClMat& M, int S0,
-                                        int ns, const T* sv, bool cols, uint32_t (&tail)[RPT]) {
+                                        int rank, int ns, const T* sv, bool cols, uint32_t (&tail)[RPT]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int E0 = a.slice_ptr[S0], E = a.slice_ptr[S0 + ns] - E0;
   const bool c16 = a.ctl->col16 != 0;
@@ -257,7 +290,7 @@ __device__ __forceinline__ void cl_load(const ClusterArgs& a, ClShared& S, const
       vd[e - E0] = sv[e];
       if (cols) {
         const int c = c16 ? i + (int)reinterpret_cast<const int16_t*>(a.scol)[e] : a.scol[e];
-        M.c[e - E0] = cl_pack(a.nslices, c);
+        M.c[e - E0] = M.rep ? (uint16_t)((rank << 12) | c) : cl_pack(a.nslices, c);
       }
     }
     if ((wf & kOverflowBit) && i < a.n) {
@@ -269,7 +302,10 @@ __device__ __forceinline__ void cl_load(const ClusterArgs& a, ClShared& S, const
       const int at = (int)(tail[j] & 0xffffu), m = (int)(tail[j] >> 16);
       for (int k = 0; k < m; ++k) {
         vd[at + k] = (T)a.val[e0 + k];
-        if (cols) M.c[at + k] = cl_pack(a.nslices, a.col[e0 + k]);
+        if (cols) {
+          const int c = a.col[e0 + k];
+          M.c[at + k] = M.rep ? (uint16_t)((rank << 12) | c) : cl_pack(a.nslices, c);
+        }
       }
     }
   }
@@ -353,9 +389,9 @@ __device__ __forceinline__ void cl_spmv(const ClusterArgs& a, const ClShared& S,
         if (m == 0 && i < a.n) {  // no room: from the caller's CSR
           const int e1 = a.rp[i + 1];
           for (int f = a.rp[i] + w; f < e1; ++f) {
-            const uint32_t c = cl_pack(a.nslices, a.col[f]);
+            const uint32_t c = M.rep ? (uint32_t)a.col[f] : cl_pack(a.nslices, a.col[f]);
             T x;
-            cl_ld(cl_map(gb, c >> 12) + (c & 4095u) * (uint32_t)sizeof(T), x);
+            cl_ld(cl_map(gb, M.rep ? cl_rank() : c >> 12) + (c & 4095u) * (uint32_t)sizeof(T), x);
             acc = fma((T)a.val[f], x, acc);
           }
         }
@@ -428,6 +464,33 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
   M.g = cl_smem;
   M.v = M.g + (size_t)a.rows_cap * sizeof(double);
   M.c = reinterpret_cast<uint16_t*>(M.v + (size_t)a.ent_cap * sizeof(double));
+  M.rep = false;
+  if (n <= kClRepN) {  // uniform: count the entries in other blocks' rows
+    const int E0 = a.slice_ptr[S0], E1 = a.slice_ptr[S0 + ns];
+    const bool c16 = ctl->col16 != 0;
+    int far = 0;
+    for (int s = warp; s < ns; s += kClWarps) {
+      const int w = (int)(a.slice_w[S0 + s] & ~kOverflowBit), p = a.slice_ptr[S0 + s];
+      const int i = (S0 + s) * kSlice + lane;
+      for (int k = 0; k < w; ++k) {
+        const int e = p + kSlice * k + lane;
+        const int c = c16 ? i + (int)reinterpret_cast<const int16_t*>(a.scol)[e] : a.scol[e];
+        if (c < S0 * kSlice || c >= (S0 + ns) * kSlice) ++far;
+      }
+    }
+    if (tid == 0) S.tail = 0;
+    __syncthreads();
+    far = __reduce_add_sync(0xffffffffu, far);
+    if (lane == 0 && far) atomicAdd(&S.tail, far);
+    __syncthreads();
+    const int half = red & 1;
+    ++red;
+    cl_exchange(S, rank, half, (double)(3 * S.tail - (E1 - E0)), 0.0);
+    double sum = 0.0;
+    for (int o = 0; o < kClBlocks; ++o) sum += S.slot[half][o];  // exact: small whole numbers
+    M.rep = sum > 0.0;  // more than a third of the stored entries (padding included)
+  }
+  M.base = M.rep ? S0 * kSlice : 0;
   const int rel = ctl->tol_relative;
   bool ok = true;
   int row[RPT];  // the thread's rows, or -1
@@ -443,8 +506,8 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
 
   // =================== single-precision stage ===================
   if (a.mode != 2) {
-    cl_load<float, RPT>(a, S, M, S0, ns, a.sv32, true, tail);
-    float* g = reinterpret_cast<float*>(M.g);
+    cl_load<float, RPT>(a, S, M, S0, rank, ns, a.sv32, true, tail);
+    const float* g = reinterpret_cast<const float*>(M.g) + M.base;
     const bool autom = a.mode == 1;
     const int max1 = ctl->max1, k0 = ctl->k0;
     const double eps2 = ctl->eps2;
@@ -469,7 +532,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
     for (int j = 0; j < RPT; ++j) {
       x[j] = 0.0f;
       r[j] = row[j] >= 0 ? a.b32[row[j]] : 0.0f;
-      if (warp + kClWarps * j < ns) g[(warp + kClWarps * j) * kSlice + lane] = r[j];
+      if (warp + kClWarps * j < ns) cl_put(M, (warp + kClWarps * j) * kSlice + lane, r[j]);
       if (row[j] >= 0) ff_add_prod(acc, r[j], r[j], false);
     }
     double rr = cl_total_ff(S, rank, ns, red, acc);  // the barrier also publishes d
@@ -672,7 +735,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
       // ---- d = r + beta d ----
 #pragma unroll
       for (int j = 0; j < RPT; ++j)
-        if (row[j] >= 0) g[row[j] - S0 * kSlice] = __fmaf_rn(beta, d[j], r[j]);
+        if (row[j] >= 0) cl_put(M, row[j] - S0 * kSlice, __fmaf_rn(beta, d[j], r[j]));
       ++it;
       cl_sync();
     }
@@ -749,8 +812,8 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
   }
 
   // =================== double-precision stage ===================
-  cl_load<double, RPT>(a, S, M, S0, ns, a.sv64, a.mode == 2, tail);
-  double* g = reinterpret_cast<double*>(M.g);
+  cl_load<double, RPT>(a, S, M, S0, rank, ns, a.sv64, a.mode == 2, tail);
+  const double* g = reinterpret_cast<const double*>(M.g) + M.base;
   const double bnorm = ctl->bnorm64, eps2 = ctl->eps2;
   const int max2 = ctl->max2, max_restarts = ctl->max_restarts;
   const StopThr thr2 = stop_thr(eps2, bnorm, rel);
@@ -763,7 +826,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
     cl_sync();  // every block has read d (and loaded its entries)
 #pragma unroll
     for (int j = 0; j < RPT; ++j)
-      if (warp + kClWarps * j < ns) g[(warp + kClWarps * j) * kSlice + lane] = xd[j];
+      if (warp + kClWarps * j < ns) cl_put(M, (warp + kClWarps * j) * kSlice + lane, xd[j]);
     cl_sync();
     cl_spmv<double, RPT>(a, S, M, S0, ns, tail, q);
     double p = 0.0;
@@ -820,7 +883,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
 #pragma unroll
       for (int j = 0; j < RPT; ++j) {
         r[j] = q[j];
-        if (warp + kClWarps * j < ns) g[(warp + kClWarps * j) * kSlice + lane] = r[j];
+        if (warp + kClWarps * j < ns) cl_put(M, (warp + kClWarps * j) * kSlice + lane, r[j]);
       }
       cl_sync();
     }
@@ -892,7 +955,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
         for (int j = 0; j < RPT; ++j) {
           if (warp + kClWarps * j < ns) {
             __syncwarp();
-            g[(warp + kClWarps * j) * kSlice + lane] = __fma_rn(beta, d[j], r[j]);
+            cl_put(M, (warp + kClWarps * j) * kSlice + lane, __fma_rn(beta, d[j], r[j]));
           }
         }
         cl_arrive();
@@ -950,9 +1013,9 @@ int cluster_rpt(int nslices) {
 
 size_t cluster_smem(const Dims& d, int* rows_cap, int* ent_cap) {
   const int rows = (d.nslices + kClBlocks - 1) / kClBlocks * kSlice;
-  *rows_cap = rows;
+  *rows_cap = d.n <= kClRepN ? d.nslices * kSlice : rows;
   *ent_cap = rows * d.wcap;
-  return (size_t)rows * sizeof(double) + (size_t)*ent_cap * (sizeof(double) + sizeof(uint16_t));
+  return (size_t)*rows_cap * sizeof(double) + (size_t)*ent_cap * (sizeof(double) + sizeof(uint16_t));
 }
 
 // Whether the device takes a cluster of kClBlocks blocks of every instance

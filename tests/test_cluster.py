@@ -45,6 +45,11 @@ CASES = {f"grid{n}": (lambda n=n: _grid(n)) for n in
 CASES.update({
     "star_1001": lambda: synth.star(1001, 1.1),          # one row past the width cap
     "rtree_5000": lambda: synth.random_tree_plus(5000, 0.5, 1.1, seed=3),
+    # whole copies of the gathered vector up to 4,096 rows, where columns are far away
+    "rreg_300": lambda: synth.random_regular_laplacian(300, 6, 1e-2, seed=4),
+    "rreg_4096": lambda: synth.random_regular_laplacian(4096, 8, 1e-3, seed=4),
+    "rreg_4097": lambda: synth.random_regular_laplacian(4097, 8, 1e-3, seed=4),
+    "rtree_3001": lambda: synth.random_tree_plus(3001, 0.5, 1.1, seed=8),
     "rreg_20000": lambda: synth.random_regular_laplacian(20000, 8, 1e-3, seed=4),  # columns far away
     "band_9000_b29": lambda: synth.banded(9000, 29, 0.6, 1.1, seed=7),
     "two_3000": lambda: _two(2000),
