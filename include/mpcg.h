@@ -117,7 +117,9 @@ typedef struct {
                                 MPCG_ERR_NOT_CONVERGED (x holds the last iterate) */
   uint32_t feat_mask;        /* bit c: feature c enters the distance (default 0xF) */
   int32_t fp64_only;         /* 1: pure FP64 CG from x0 = 0 (the baseline); no stage 1 */
-  int32_t grid_blocks;       /* persistent grid size; 0 = one full wave of the device */
+  int32_t grid_blocks;       /* persistent grid size; 0 = one full wave of the device (and small
+                                systems may run in one thread-block cluster, and the 2BFS in one
+                                block) */
   int32_t timeout_ms;        /* limit of every device-side wait (default 20000) */
   int32_t stage1_only;       /* 1: stop after the single-precision stage; x = float64(x~) */
   int32_t team_rows;         /* batch and server: target rows per block of a team, which sets
@@ -171,9 +173,10 @@ typedef struct {
                                 slices lies within 32767 columns of its row, 32-bit columns
                                 otherwise; 1 = 32-bit columns always.  The single-system
                                 kernels read the chosen format in both stages; the batched
-                                solve and the server read it in the single-precision SpMV
-                                that stages its pairs in shared memory (the batch's stage 1,
-                                the server's split mode) and 32-bit columns elsewhere.  Both
+                                solve and the server read it in the double-precision SpMV and
+                                in the single-precision SpMV that stages its pairs in shared
+                                memory (the batch's stage 1, the server's split mode), and
+                                32-bit columns in the server's other single-precision SpMV.  Both
                                 formats sum the same entries in the same order, so x and every
                                 count are bit-identical; 16-bit offsets move 6 instead of 8
                                 bytes a stored entry in single precision, 10 instead of 12 in
