@@ -192,29 +192,50 @@ int team_grid(const void* kernel, int requested, int smem) {
   return requested > 0 && requested < full ? requested : full;
 }
 
+// Queue 0 holds the systems of one launch block, queue 1 those of one plan
+// block (two launch blocks) and queue q > 1 those of 2^(q-1) plan blocks: 2^q
+// launch blocks each.  A system of one plan block gets one launch block while
+// the batch is bound by the sum of its work: two systems an SM hide each
+// other's latency.  It gets both when it is what the launch would wait for:
+// more than kHalfRows rows (below, the team barriers cost what the second
+// block gives) and more work than a launch block's share of the batch.  One
+// launch block each at every size, with few systems: 9.7 ms for 12 systems of
+// up to 8e4 rows (FP64, 16384 rows a block; now 6.8), 29.5 ms for 13 of up to
+// 4.7e4 (eps1 chosen; now 17.3).  12 systems of up to 6000 rows: 3.4 ms with
+// the line at 2048 rows, 3.8 at 4096, 4.0 at 8192; of up to 3000 rows 2.6 ms
+// with each.
+constexpr int kHalfRows = 2048;
+
 Plan make_plan(int nsys, const int* n, const double* work, int grid, int rows_per_block,
                bool whole_blocks, const int32_t* rows_sys) {
   if (rows_per_block <= 0) rows_per_block = kRowsPerBlock;
   Plan P;
+  const int blocks = grid * kBatchPerSm;
   std::vector<int> cls(nsys);
   std::vector<double> w(nsys);
-  double cw[kTeamClasses] = {0};
-  int cnt[kTeamClasses] = {0};
+  double cw[kTeamQueues] = {0};
+  int cnt[kTeamQueues] = {0};
+  double share = 0.0;
   for (int i = 0; i < nsys; ++i) {
     const int rpb = rows_sys && rows_sys[i] > 0 ? rows_sys[i] : rows_per_block;
-    cls[i] = size_class(n[i], rpb);
     w[i] = work[i];
+    share += w[i] / blocks;
+    cls[i] = size_class(n[i], rpb) + 1;
   }
+  for (int i = 0; i < nsys; ++i)
+    if (cls[i] == 1 && !whole_blocks && !(n[i] > kHalfRows && w[i] > share)) cls[i] = 0;
   // Demote the largest classes while one team of every non-empty class does
   // not fit in the grid.
+  const int least = whole_blocks ? 1 : 0;
   for (;;) {
     int need = 0, top = -1;
     for (int i = 0; i < nsys; ++i) top = std::max(top, cls[i]);
-    bool present[kTeamClasses] = {false};
+    bool present[kTeamQueues] = {false};
     for (int i = 0; i < nsys; ++i) present[cls[i]] = true;
-    for (int c = 0; c < kTeamClasses; ++c)
+    for (int c = 0; c < kTeamQueues; ++c)
       if (present[c]) need += 1 << c;
-    if (need <= grid || top <= 0) break;
+    if (need <= blocks || top <= least) break;
+    if (present[0] && present[1]) top = 1;  // one plan block's systems stay so
     for (int i = 0; i < nsys; ++i)
       if (cls[i] == top) cls[i] = top - 1;
   }
@@ -225,9 +246,9 @@ Plan make_plan(int nsys, const int* n, const double* work, int grid, int rows_pe
   // Teams per class: one each, then one more team at a time to the class
   // with the most work per block, while blocks remain and the class (with
   // the smaller ones it can take from) has systems for it.
-  int teams[kTeamClasses] = {0};
+  int teams[kTeamQueues] = {0};
   int used = 0;
-  for (int c = 0; c < kTeamClasses; ++c)
+  for (int c = 0; c < kTeamQueues; ++c)
     if (cnt[c]) {
       teams[c] = 1;
       used += 1 << c;
@@ -235,8 +256,8 @@ Plan make_plan(int nsys, const int* n, const double* work, int grid, int rows_pe
   for (;;) {
     int best = -1;
     double best_load = -1.0;
-    for (int c = 0; c < kTeamClasses; ++c) {
-      if (!cnt[c] || used + (1 << c) > grid) continue;
+    for (int c = 0; c < kTeamQueues; ++c) {
+      if (!cnt[c] || used + (1 << c) > blocks) continue;
       int avail = 0;
       for (int cc = 0; cc <= c; ++cc) avail += cnt[cc];
       if (teams[c] >= avail) continue;
@@ -250,27 +271,27 @@ Plan make_plan(int nsys, const int* n, const double* work, int grid, int rows_pe
     teams[best] += 1;
     used += 1 << best;
   }
-  // Block layout: largest teams first; the class-0 teams and the blocks left
-  // over are teams of one launch block.
-  P.team_of_block.assign(grid * kBatchPerSm, 0);
-  P.rank_of_block.assign(grid * kBatchPerSm, 0);
+  // Block layout: largest teams first; the blocks left over are teams of the
+  // smallest size.
+  P.team_of_block.assign(blocks, 0);
+  P.rank_of_block.assign(blocks, 0);
   int b = 0;
-  auto add = [&](int c, int size) {  // one team of `size` launch blocks
+  auto add = [&](int c) {
     const int tm = (int)P.team_size.size();
-    P.team_size.push_back(size);
+    P.team_size.push_back(1 << c);
     P.team_class.push_back(c);
-    for (int r = 0; r < size; ++r) {
+    for (int r = 0; r < 1 << c; ++r) {
       P.team_of_block[b] = tm;
       P.rank_of_block[b] = r;
       ++b;
     }
   };
-  for (int c = kTeamClasses - 1; c > 0; --c)
-    for (int k = 0; k < teams[c]; ++k) add(c, kBatchPerSm << c);
-  while (b < grid * kBatchPerSm) add(0, whole_blocks ? kBatchPerSm : 1);
+  for (int c = kTeamQueues - 1; c >= least; --c)
+    for (int k = 0; k < teams[c]; ++k) add(c);
+  while (b < blocks) add(least);
   // Queues: class by class, largest work first.
   int base = 0;
-  for (int c = 0; c < kTeamClasses; ++c) {
+  for (int c = 0; c < kTeamQueues; ++c) {
     std::vector<int> q;
     for (int i = 0; i < nsys; ++i)
       if (cls[i] == c) q.push_back(i);
@@ -348,8 +369,9 @@ extern "C" int32_t mpcg_batch_plan(int32_t nsys, const int32_t* n, const int32_t
   }
   const Plan P = make_plan(nsys, nv.data(), work.data(), grid, opts->team_rows, opts->acc32 != 0,
                            opts->team_rows_sys);
-  for (int c = 0; c < kTeamClasses; ++c)
-    for (int k = 0; k < P.qlen[c]; ++k) team_blocks_out[P.order[P.qbase[c] + k]] = 1 << c;
+  for (int c = 0; c < kTeamQueues; ++c)
+    for (int k = 0; k < P.qlen[c]; ++k)
+      team_blocks_out[P.order[P.qbase[c] + k]] = std::max(1, (1 << c) / kBatchPerSm);
   return MPCG_OK;
 }
 
@@ -408,7 +430,7 @@ extern "C" int32_t mpcg_solve_batch(int32_t nsys, const mpcg_csr_t* A, const dou
   const int* rob_d = put(P.rank_of_block, kMaxGrid);
   const int* tsz_d = put(P.team_size, kMaxGrid);
   const int* tcl_d = put(P.team_class, kMaxGrid);
-  for (int c = 0; c < kTeamClasses; ++c) {
+  for (int c = 0; c < kTeamQueues; ++c) {
     H->qbase[c] = P.qbase[c];
     H->qlen[c] = P.qlen[c];
   }
@@ -488,12 +510,12 @@ double simulate_launch(const Plan& P, const std::vector<SysTimes>& T, int stage)
   using Ev = std::pair<double, int>;
   std::priority_queue<Ev, std::vector<Ev>, std::greater<Ev>> q;
   for (int tm = 0; tm < (int)P.team_class.size(); ++tm) q.push({0.0, tm});
-  int head[kTeamClasses] = {0};
+  int head[kTeamQueues] = {0};
   double span = 0.0;
   while (!q.empty()) {
     const Ev e = q.top();
     q.pop();
-    const int c = P.team_class[e.second];
+    int c = P.team_class[e.second];
     int sys = -1;
     for (int cc = c; cc >= 0 && sys < 0; --cc)
       if (head[cc] < P.qlen[cc]) sys = P.order[P.qbase[cc] + head[cc]++];
@@ -502,6 +524,7 @@ double simulate_launch(const Plan& P, const std::vector<SysTimes>& T, int stage)
       continue;
     }
     const SysTimes& t = T[sys];
+    c = std::max(c - 1, 0);  // measured by plan blocks
     const double d = stage == 1 ? busy_at(t.s1, c)
                      : stage == 2 ? busy_at(t.s2, c)
                                   : busy_at(t.s1, c) + busy_at(t.s2, c);

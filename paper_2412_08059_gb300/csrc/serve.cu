@@ -387,7 +387,7 @@ extern "C" int32_t mpcg_batch_step(mpcg_server_t* s, int32_t max_iters, int32_t*
     char* m = s->mirror.data();
     BatchHdr* H = (BatchHdr*)m;
     memset(H, 0, sizeof(BatchHdr));
-    for (int c = 0; c < kTeamClasses; ++c) {
+    for (int c = 0; c < kTeamQueues; ++c) {
       H->qbase[c] = P.qbase[c];
       H->qlen[c] = P.qlen[c];
     }

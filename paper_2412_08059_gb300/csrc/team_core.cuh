@@ -28,7 +28,8 @@ namespace mpcg {
 constexpr int kBatchThreads = 256;
 constexpr int kBatchPerSm = 2;                 // launch blocks an SM (one plan block)
 constexpr int kBatchWarps = kBatchThreads / 32;
-constexpr int kTeamClasses = 8;                // team sizes 1, 2, 4, ..., 128 blocks
+constexpr int kTeamClasses = 8;                // team sizes 1, 2, 4, ..., 128 plan blocks
+constexpr int kTeamQueues = kTeamClasses + 1;  // and one launch block (half a plan block)
 constexpr int kRowsPerBlock = 16384;           // planner default: target rows per block of a team
 constexpr int kNoBudget = 0x7fffffff;          // iteration budget of a run-to-completion call
 constexpr int kTeamFastW = 8;                  // widest slice whose pairs the SpMV stages
@@ -61,8 +62,8 @@ struct BatchSys {
 struct BatchHdr {
   unsigned long long bar[kMaxGrid];  // per-team barrier counters
   int next[kMaxGrid];                // system index broadcast by each team leader
-  int head[kTeamClasses];            // queue heads (atomic)
-  int qbase[kTeamClasses], qlen[kTeamClasses];
+  int head[kTeamQueues];            // queue heads (atomic)
+  int qbase[kTeamQueues], qlen[kTeamQueues];
   int abort;                         // a team barrier timed out: every block leaves
   int pad;
 };
@@ -1378,10 +1379,10 @@ static __device__ bool team_pseudo_diameter(Team& t, const BatchSys& s, int smem
 // team_of_block, rank_of_block: by launch block; team_size: launch blocks.
 struct Plan {
   std::vector<int> team_of_block, rank_of_block, team_size, team_class, order;
-  int qbase[kTeamClasses], qlen[kTeamClasses];
+  int qbase[kTeamQueues], qlen[kTeamQueues];
 };
-// Teams for a grid of `grid` plan blocks (kBatchPerSm * grid launch blocks) and the class queues of nsys systems of
-// n rows with estimated work `work` (largest first within a class); a system
+// Teams for a grid of `grid` plan blocks (kBatchPerSm * grid launch blocks)
+// and the queues (teams of queue q: 2^q launch blocks) of nsys systems of n rows with estimated work `work` (largest first within a class); a system
 // goes to the smallest team with at most rows_per_block rows per block, or
 // rows_sys[i] when that array is given and its entry is positive.
 // whole_blocks (option acc32): teams of one plan block are two launch blocks
