@@ -506,7 +506,7 @@ __device__ __forceinline__ T row_tail(const CgArgs& a, int i, int w, T acc, Gath
 // One SpMV pass over the block's slices by the consumer warps.  For every
 // row i of the block's slices (padding rows included), Rw(i, acc) receives
 // sum_k v_k G(c_k) in stored order.  A warp takes two adjacent slices per
-// step (one when the block has no more slices than warps), so that the gathers
+// step (one when the block has no more slices than warps, or wide ones), so that the gathers
 // of both rows are in flight together; their entries are contiguous, at most 2 x 32 x 64 = kCH of them, so a step never
 // needs more than two chunks at once (the ring has at least four), which
 // keeps the producer/consumer ring free of deadlock.  The next step's widths
@@ -518,7 +518,11 @@ __device__ __forceinline__ bool ring_spmv(const CgArgs& a, Ring<T>& R, Cursor& C
                                           Gather G, Row Rw) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   bool ok = true;
-  const int per = S1 - S0 > NC ? 2 : 1;  // slices a step
+  // Slices a step: one where the rows are on average wider than the unrolled
+  // forms, whose two slices a warp would span more chunks than the ring holds
+  // (FP64, n = 2^20: half bandwidth 14, density 0.6, 4.55 ms with two slices
+  // and 3.82 with one; half bandwidth 7 12.6 and 11.3 ms).
+  const int per = S1 - S0 > NC && R.E1 - R.E0 <= 9 * kSlice * (S1 - S0) ? 2 : 1;
   int s0 = S0 + per * warp;
   uint32_t nf0 = 0u, nf1 = 0u;
   int np = 0;
