@@ -19,14 +19,14 @@ constexpr int kPdThreads = 1024;
 constexpr int kPdSmem = 200 * 1024;
 __global__ void __launch_bounds__(kPdThreads, 1) k_pdiam_block(BlockGraph g, BfsGraph q) {
   extern __shared__ __align__(16) unsigned char pd_smem[];
-  if (volatile_status(q.ctl) != 0) return;
+  if (block_status(q.ctl) != 0) return;
   g.c16 = q.ctl->col16;
   block_pdiam(g, q, pd_smem, kPdSmem);
 }
 
 __global__ void __launch_bounds__(kCgThreads, 1) k_pdiam(BfsGraph g, int32_t* d1, int32_t* d2,
                                                       int slot) {
-  if (volatile_status(g.ctl) != 0 || g.ctl->pd_done) return;
+  if (block_status(g.ctl) != 0 || g.ctl->pd_done) return;
   GridSync sync{g.ctl, slot, 0ull};
   const int tid = blockIdx.x * blockDim.x + threadIdx.x;
   pseudo_diameter_run(g, d1, d2, tid, gridDim.x * blockDim.x, sync);
@@ -34,7 +34,7 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_pdiam(BfsGraph g, int32_t* d1
 
 __global__ void __launch_bounds__(kCgThreads, 1) k_bfs1(BfsGraph g, int32_t* dist, int src,
                                                      int slot) {
-  if (volatile_status(g.ctl) != 0) return;
+  if (block_status(g.ctl) != 0) return;
   GridSync sync{g.ctl, slot, 0ull};
   const int tid = blockIdx.x * blockDim.x + threadIdx.x;
   bfs_run(g, dist, kSrcSingle, src, kRoleFirst, tid, gridDim.x * blockDim.x, sync);

@@ -438,7 +438,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
   Ctl* ctl = a.ctl;
   const bool trivial = *reinterpret_cast<volatile int*>(&ctl->trivial) != 0;
   if (a.mode == 1 && blockIdx.x < kClBlocks) {  // the 2BFS cluster
-    if (!trivial && volatile_status(ctl) == 0) cl_bfs(a, cl_smem);
+    if (!trivial && block_status(ctl) == 0) cl_bfs(a, cl_smem);
     return;
   }
   const int rank = (int)(blockIdx.x & (kClBlocks - 1));

@@ -176,6 +176,14 @@ __device__ __forceinline__ int volatile_status(const Ctl* c) {
   return *reinterpret_cast<const volatile int*>(&c->status);
 }
 
+// The status at a kernel's entry as thread 0 read it, in every thread of the
+// block.  Another block may set it at any moment (a cancel or a time limit met
+// in its first wait), so warps that each read it could part ways, and the
+// ones that stay would wait at a barrier for those that left.
+__device__ __forceinline__ int block_status(const Ctl* c) {
+  return __syncthreads_or(threadIdx.x == 0 ? volatile_status(c) : 0);
+}
+
 // Cancellation: the caller's cancel word, when set, ends the call's work with
 // MPCG_ERR_CANCELLED (first error wins).  Read in the periodic checks of the
 // bounded waits and, through cancel_word, at the head of every CG iteration.
