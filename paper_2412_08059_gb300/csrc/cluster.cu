@@ -26,10 +26,13 @@
 // stored order by fused multiply-adds, float-float inner products in single
 // precision, alpha and beta the double quotients rounded once to float.
 //
-// Algorithm II: a second cluster of the same launch runs the 2BFS meanwhile, and the iterations past k0 are speculative with
+// Algorithm II: the launch has two clusters.  The one that begins first runs
+// the 2BFS, the other CG, whose iterations past k0 are speculative with
 // snapshots at every candidate eps1, as in k_stage1.  The kNN vote is run by
-// whichever of the two clusters comes second with its part of the features,
-// so the 2BFS never waits for CG.
+// whichever comes second with its part of the features, so the 2BFS never
+// waits for CG, and CG, which may wait for the label, waits for a cluster that
+// has begun: the launch ends whatever the order in which its clusters are
+// placed, also one after the other on a device that other work has filled.
 #include <math.h>
 
 #include "feature_block.cuh"
@@ -417,14 +420,22 @@ __device__ __forceinline__ void cl_feature_ready(const KnnSpec& knn, Ctl* ctl) {
   if (__shfl_sync(0xffffffffu, second, 0) == 1) feature_vote(knn, ctl);
 }
 
-__device__ __noinline__ void cl_bfs(const ClusterArgs& a, unsigned char* smem) {
+__device__ __noinline__ void cl_bfs(const ClusterArgs& a, unsigned char* smem, int rank) {
   const BlockGraph g{a.rp, a.col, a.slice_ptr, a.slice_w, a.scol, a.n, a.ctl->col16};
-  const bool ok = feature_pdiam(g, a.g, a.d1, a.d2, smem, a.smem_bytes, a.bfs_slot, 0, kClBlocks);
+  const bool ok = feature_pdiam(g, a.g, a.d1, a.d2, smem, a.smem_bytes, a.bfs_slot,
+                                (int)blockIdx.x - rank, kClBlocks);
   __syncthreads();
-  if (blockIdx.x == 0 && threadIdx.x < 32) {
+  if (rank == 0 && threadIdx.x < 32) {
     if (ok) cl_feature_ready(a.knn, a.ctl);
     else if (threadIdx.x == 0) atomicExch(&a.ctl->eps1_ready, -1);
   }
+}
+
+// The part of a cluster of Algorithm II, by the order in which the two begin:
+// the first runs the 2BFS.
+enum ClPart { kClPartNone = 0, kClPartBfs = 1, kClPartCg = 2 };
+__device__ __forceinline__ double cl_part(Ctl* ctl) {
+  return atomicAdd(&ctl->cl_begun, 1) == 0 ? kClPartBfs : kClPartCg;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -437,10 +448,6 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
   __shared__ ClShared S;
   Ctl* ctl = a.ctl;
   const bool trivial = *reinterpret_cast<volatile int*>(&ctl->trivial) != 0;
-  if (a.mode == 1 && blockIdx.x < kClBlocks) {  // the 2BFS cluster
-    if (!trivial && block_status(ctl) == 0) cl_bfs(a, cl_smem);
-    return;
-  }
   const int rank = (int)(blockIdx.x & (kClBlocks - 1));
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n = a.n;
@@ -450,14 +457,18 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
     for (int i = S0 * kSlice + tid; i < min(n, (S0 + ns) * kSlice); i += kClThreads) a.x64[i] = 0.0;
     return;
   }
-  // The blocks of the cluster leave together: block 0's view of the status
-  // decides for all (the 2BFS cluster may set it at any time).  The first
-  // barrier makes sure that every block runs before its memory is written to.
+  // The blocks of the cluster leave, or take their part, together: block 0
+  // decides for all (the other cluster may set the status at any time).  The
+  // first barrier makes sure that every block runs before its memory is
+  // written to.
   cl_sync();
   int red = 1;
-  cl_exchange(S, rank, 0, 0.0, lead0 ? (double)volatile_status(ctl) : 0.0);
-  if (S.aux[0] != 0.0) {
-    cl_sync();
+  double part = kClPartCg;
+  if (lead0) part = volatile_status(ctl) != 0 ? kClPartNone : a.mode == 1 ? cl_part(ctl) : kClPartCg;
+  cl_exchange(S, rank, 0, 0.0, part);
+  part = S.aux[0];
+  if (part != kClPartCg) {
+    if (part == kClPartBfs) cl_bfs(a, cl_smem, rank);
     return;
   }
   ClMat M;

@@ -61,6 +61,7 @@ struct Ctl {
   int x32_src;     // stage-1 result: -1 = x32, s >= 0 = snapshot slot s
   int pd_done;     // the one-block 2BFS has succeeded
   int feat_sides;  // cluster kernel: sides of the features (l~, v) that are complete
+  int cl_begun;    // cluster kernel, Algorithm II: clusters that have begun
   // device clock marks (ns)
   unsigned long long t_start, t_prep, t_features, t_fp32, t_fp64, t_end;
   unsigned long long t_s2;  // team kernels: start of the double-precision stage (0: not marked)
