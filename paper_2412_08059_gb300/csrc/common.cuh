@@ -3,7 +3,9 @@
 // deterministic reductions and float-float accumulation.
 #pragma once
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
+#include <string.h>
 
 #include "../../include/mpcg.h"
 
@@ -124,23 +126,32 @@ __device__ __forceinline__ void red_release_add(unsigned long long* p, unsigned 
 __device__ __forceinline__ void set_status(Ctl* c, int s) { atomicCAS(&c->status, 0, s); }
 
 // Stop measure of the CG procedure: ||r|| / ||b|| (relative) or ||r||.
-__device__ __forceinline__ double stop_measure(double rr, double bnorm, int rel) {
+__host__ __device__ __forceinline__ double stop_measure(double rr, double bnorm, int rel) {
   return rel ? sqrt(rr) / bnorm : sqrt(rr);
 }
 
 // Comparisons of doubles by their bit patterns: an FP64 comparison takes its
 // turn of the FP64 pipe (about 80 clocks in a chain), an integer one does not.
 // Values that are not negative order like their bits; every NaN is above
-// infinity there.
-__device__ __forceinline__ long long dbits(double v) { return __double_as_longlong(v); }
-__device__ __forceinline__ bool bits_finite(double v) {
-  return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000;
+// infinity there.  (For the host too: the tests compare them with the
+// floating-point tests.)
+__host__ __device__ __forceinline__ long long dbits(double v) {
+#ifdef __CUDA_ARCH__
+  return __double_as_longlong(v);
+#else
+  long long b;
+  memcpy(&b, &v, sizeof(b));
+  return b;
+#endif
 }
-__device__ __forceinline__ bool bits_nan(double v) {
+__host__ __device__ __forceinline__ bool bits_finite(double v) {
+  return ((int)(dbits(v) >> 32) & 0x7ff00000) != 0x7ff00000;
+}
+__host__ __device__ __forceinline__ bool bits_nan(double v) {
   return (dbits(v) & 0x7fffffffffffffffll) > 0x7ff0000000000000ll;
 }
 // v > 0 (false for NaN)
-__device__ __forceinline__ bool bits_positive(double v) {
+__host__ __device__ __forceinline__ bool bits_positive(double v) {
   return dbits(v) > 0 && dbits(v) <= 0x7ff0000000000000ll;
 }
 
@@ -155,7 +166,7 @@ struct StopThr {
   double lo, hi, eps, bnorm;
   int rel;
 };
-__device__ __forceinline__ StopThr stop_thr(double eps, double bnorm, int rel) {
+__host__ __device__ __forceinline__ StopThr stop_thr(double eps, double bnorm, int rel) {
   const double s = rel ? eps * bnorm : eps;
   const double t = s * s;
   StopThr T{-1.0, INFINITY, eps, bnorm, rel};
@@ -165,11 +176,11 @@ __device__ __forceinline__ StopThr stop_thr(double eps, double bnorm, int rel) {
   }
   return T;
 }
-__device__ __forceinline__ bool stop_pass(const StopThr& T, double rr) {
-  // rr is a sum of squares (not negative) or NaN, for which the test fails; lo
-  // is -1 where it never passes by itself
+__host__ __device__ __forceinline__ bool stop_pass(const StopThr& T, double rr) {
+  // rr is a sum of squares, so not negative, or NaN.  Unsigned, every NaN is
+  // above hi, whatever its sign; lo is -1 where no rr passes by itself.
+  if ((unsigned long long)dbits(rr) > (unsigned long long)dbits(T.hi)) return false;
   if (dbits(rr) <= dbits(T.lo)) return true;
-  if (dbits(rr) > dbits(T.hi)) return false;
   return stop_measure(rr, T.bnorm, T.rel) <= T.eps;
 }
 
