@@ -184,16 +184,17 @@ int32_t mpcg_solve(const mpcg_csr_t* A, const double* b, double* x, const mpcg_s
   L.true_res = opts->stop_true_residual;
   cudaError_t e;
   if ((e = launch_init(L, *opts, fp64_only)) != cudaSuccess) return cuda_status(e);
-  if ((e = launch_prep(L, b)) != cudaSuccess) return cuda_status(e);
-  if (L.precond && (e = launch_jacobi(L)) != cudaSuccess) return cuda_status(e);
   // One cluster of blocks runs a small system whole; a grid asked for, and
   // the options that only the grid-wide kernels have, take those.
-  const bool small = opts->grid_blocks == 0 && !L.precond && !L.true_res && !opts->stage1_only &&
-                     !opts->acc32 && !(auto_eps1 && opts->bfs_starts > 1) && cluster_fits(L.d);
-  if (small) {
+  const bool plain = opts->grid_blocks == 0 && !L.precond && !L.true_res && !opts->stage1_only &&
+                     !opts->acc32 && !(auto_eps1 && opts->bfs_starts > 1);
+  const int line = plain ? cluster_line(L.d) : -1;
+  if ((e = launch_prep(L, b, line)) != cudaSuccess) return cuda_status(e);
+  if (L.precond && (e = launch_jacobi(L)) != cudaSuccess) return cuda_status(e);
+  if (line >= 0) {
     if ((e = launch_cluster(L, b, x, sample, *opts, fp64_only ? 2 : (auto_eps1 ? 1 : 0), kSlotPd)) != cudaSuccess)
       return cuda_status(e);
-    return cuda_status(launch_finalize(L, res, nullptr));
+    if (line == kClAlways) return cuda_status(launch_finalize(L, res, nullptr));
   }
   if (!fp64_only && auto_eps1 && (L.precond || L.true_res)) {
     // Algorithm II with Jacobi PCG or with the stop test on b - A x, its

@@ -750,7 +750,7 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_cg32(CgArgs a) {
   extern __shared__ __align__(128) char smem[];
   __shared__ CShared<NC> S;
   Ctl* ctl = a.ctl;
-  if (block_status(ctl) != 0 || ctl->trivial) return;
+  if (block_status(ctl) != 0 || ctl->trivial || ctl->small) return;
   if (a.mode == kCgContinue && ctl->broke32) {  // stage 1 already ended in the k0 phase
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       if (ctl->res32 > ctl->eps1) ctl->warn_eps1 = 1;
@@ -1125,7 +1125,7 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_cg64(CgArgs a) {
   extern __shared__ __align__(128) char smem[];
   __shared__ CShared<NC> S;
   Ctl* ctl = a.ctl;
-  if (block_status(ctl) != 0) return;
+  if (block_status(ctl) != 0 || ctl->small) return;
   Ring<double> R;
   int S0, S1;
   ring_setup<NC>(a, smem, R, S, (int)gridDim.x, S0, S1);
@@ -1461,7 +1461,7 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_stage1(Stage1Args sa) {
   __shared__ HelpLevel s_hl;   // the level the feature warp publishes to them
   const CgArgs& a = sa.a;
   Ctl* ctl = a.ctl;
-  if (block_status(ctl) != 0 || ctl->trivial) return;
+  if (block_status(ctl) != 0 || ctl->trivial || ctl->small) return;
   if (threadIdx.x == 0) {
     s_k0_ready = 0;
     s_cmask = 0u;

@@ -20,7 +20,7 @@
 // adds of the sums at 64 clocks each, one FP64 division a sum at 534 clocks,
 // three cluster barriers); from about 16,000 rows the FP64 pipes of the 16
 // SMs (one warp-wide FMA per 19 clocks and SM), which is why larger systems
-// take the grid-wide kernels (cluster_fits below has the line).
+// take the grid-wide kernels (cluster_line below).
 //
 // The arithmetic is that of the grid-wide kernels (cg.cu): rows summed in
 // stored order by fused multiply-adds, float-float inner products in single
@@ -42,7 +42,6 @@ namespace mpcg {
 
 constexpr int kClThreads = 512;
 constexpr int kClWarps = kClThreads / 32;
-constexpr int kClBlocks = 16;     // blocks of the cluster
 constexpr int kClSnaps = 6;       // snapshots of x~ in the workspace (as k_stage1)
 constexpr int kClMaxRpt = 6;      // rows per thread of the largest instance
 constexpr int kClSmem = 220 * 1024;  // dynamic shared memory a block may take
@@ -105,15 +104,6 @@ __device__ __forceinline__ void cl_st(uint32_t addr, float v) {
 }
 __device__ __forceinline__ void cl_st(uint32_t addr, double v) {
   asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(addr), "d"(v) : "memory");
-}
-
-// First slice of a block, and the block that owns a slice (the largest rank
-// whose first slice is not past it).
-__device__ __forceinline__ int cl_first(int nslices, int rank) {
-  return (int)((long long)nslices * rank / kClBlocks);
-}
-__device__ __forceinline__ int cl_owner(int nslices, int s) {
-  return (int)(((long long)kClBlocks * s + kClBlocks - 1) / nslices);
 }
 
 // Shared state of a block.  `slot` and `aux` are written by the other
@@ -420,7 +410,8 @@ __device__ __forceinline__ void cl_feature_ready(const KnnSpec& knn, Ctl* ctl) {
   if (__shfl_sync(0xffffffffu, second, 0) == 1) feature_vote(knn, ctl);
 }
 
-__device__ __noinline__ void cl_bfs(const ClusterArgs& a, unsigned char* smem, int rank) {
+__device__ __noinline__ void cl_bfs(const ClusterArgs& a, unsigned char* smem) {
+  const int rank = (int)cl_rank();
   const BlockGraph g{a.rp, a.col, a.slice_ptr, a.slice_w, a.scol, a.n, a.ctl->col16};
   const bool ok = feature_pdiam(g, a.g, a.d1, a.d2, smem, a.smem_bytes, a.bfs_slot,
                                 (int)blockIdx.x - rank, kClBlocks);
@@ -447,8 +438,9 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
   extern __shared__ __align__(128) unsigned char cl_smem[];
   __shared__ ClShared S;
   Ctl* ctl = a.ctl;
+  if (!ctl->small) return;
   const bool trivial = *reinterpret_cast<volatile int*>(&ctl->trivial) != 0;
-  const int rank = (int)(blockIdx.x & (kClBlocks - 1));
+  const int rank = (int)cl_rank();  // (read again where it is needed, which costs no register)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n = a.n;
   const int S0 = cl_first(a.nslices, rank), ns = cl_first(a.nslices, rank + 1) - S0;
@@ -468,7 +460,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
   cl_exchange(S, rank, 0, 0.0, part);
   part = S.aux[0];
   if (part != kClPartCg) {
-    if (part == kClPartBfs) cl_bfs(a, cl_smem, rank);
+    if (part == kClPartBfs) cl_bfs(a, cl_smem);
     return;
   }
   ClMat M;
@@ -1073,12 +1065,33 @@ bool cluster_device_ok() {
 // The line between the cluster and the grid-wide kernels: the block's part
 // fits in shared memory for every sparsity pattern with these counts, and
 // nnz + 5 n, the FP64 FMAs of an iteration, is at most kClMaxFma.
+//
+// Past kClRepN rows, where d is read from its owners, the gathers of a matrix
+// whose columns are scattered bound the iteration: 52 clocks for one whose
+// lanes reach most of the blocks.  The host does not know the pattern, so the
+// set-up counts the entries in other blocks' rows whose gather reaches four
+// blocks or more, and the cluster takes at most kClMaxFar of them.  Where the
+// two ways are even (FP64 solves): 8-regular graphs at 6,100 rows (46,000 such
+// entries; 0.43 ms), 4-regular at 12,500 (47,000; 0.60 ms), trees with n / 2
+// more edges at 16,000 (44,000; 11.6 ms), trees at 28,500 (52,000; 26 ms).
+// Past it (us, cluster and grid): 8-regular graph of 20,000 rows 861 and 458,
+// tree with n / 2 more edges of 36,000 rows 33,600 and 22,100.  Stencils and
+// bands have no such entries (a gather reaches two blocks, or three).
+//
+// The kernels not taken leave at once, 6 us each (3 % of the shortest solve, a
+// band of width 15 and 6,000 rows), so they are not launched where the
+// entries off the diagonal, of which a scattered matrix has fifteen of sixteen
+// in other blocks, keep the count below the line (kClMaxOff).
 constexpr long long kClMaxFma = 400000;
+constexpr int kClMaxFar = 45000;
+constexpr int kClMaxOff = 48000;
 
-bool cluster_fits(const Dims& d) {
+int cluster_line(const Dims& d) {
   int rows, ents;
-  return cluster_rpt(d.nslices) > 0 && (long long)d.nnz + 5ll * d.n <= kClMaxFma &&
-         cluster_smem(d, &rows, &ents) <= (size_t)kClSmem && cluster_device_ok();
+  const bool fits = cluster_rpt(d.nslices) > 0 && (long long)d.nnz + 5ll * d.n <= kClMaxFma &&
+                    cluster_smem(d, &rows, &ents) <= (size_t)kClSmem && cluster_device_ok();
+  if (!fits) return -1;
+  return d.n <= kClRepN || d.nnz - d.n <= kClMaxOff ? kClAlways : kClMaxFar;
 }
 
 cudaError_t launch_cluster(const Launch& L, const double* b, double* x, const mpcg_sample_t* S,

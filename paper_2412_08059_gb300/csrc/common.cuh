@@ -64,6 +64,8 @@ struct Ctl {
   int pd_done;     // the one-block 2BFS has succeeded
   int feat_sides;  // cluster kernel: sides of the features (l~, v) that are complete
   int cl_begun;    // cluster kernel, Algorithm II: clusters that have begun
+  int cl_far;      // stored entries whose gathers are spread over the cluster's blocks (k_fill)
+  int small;       // the cluster kernel runs the system, and the grid-wide kernels leave it alone
   // device clock marks (ns)
   unsigned long long t_start, t_prep, t_features, t_fp32, t_fp64, t_end;
   unsigned long long t_s2;  // team kernels: start of the double-precision stage (0: not marked)

@@ -46,7 +46,9 @@ bool sample_ok(const mpcg_sample_t* s);
 // prep.cu
 cudaError_t launch_init(const Launch& L, const mpcg_options_t& o, int fp64_only);
 cudaError_t launch_jacobi(const Launch& L);
-cudaError_t launch_prep(const Launch& L, const double* b);
+// cl_line: what cluster_line gave for a solve that may take the cluster
+// kernel (Ctl::small), -1 for every other call.
+cudaError_t launch_prep(const Launch& L, const double* b, int cl_line = -1);
 cudaError_t launch_finalize(const Launch& L, mpcg_result_t* res, mpcg_features_t* feat);
 
 // cg.cu
@@ -63,7 +65,20 @@ const void* cg64_kernel();
 int cg_grid(int requested);
 
 // cluster.cu: both stages of a small system in one cluster of blocks
-bool cluster_fits(const Dims& d);
+constexpr int kClBlocks = 16;  // blocks of the cluster
+// First slice of a block, and the block that owns a slice (the largest rank
+// whose first slice is not past it).
+__host__ __device__ __forceinline__ int cl_first(int nslices, int rank) {
+  return (int)((long long)nslices * rank / kClBlocks);
+}
+__host__ __device__ __forceinline__ int cl_owner(int nslices, int s) {
+  return (int)(((long long)kClBlocks * s + kClBlocks - 1) / nslices);
+}
+// Which kernels run a system of these sizes: the grid-wide ones (-1), the
+// cluster kernel (kClAlways), or the cluster kernel if the matrix has at most
+// the returned number of spread entries (Ctl::cl_far) and the others if not.
+constexpr int kClAlways = 0x7fffffff;
+int cluster_line(const Dims& d);
 cudaError_t launch_cluster(const Launch& L, const double* b, double* x, const mpcg_sample_t* S,
                            const mpcg_options_t& o, int mode, int bfs_slot);
 

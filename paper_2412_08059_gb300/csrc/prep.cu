@@ -238,10 +238,14 @@ __global__ void k_scan(const uint32_t* __restrict__ slice_w, int32_t* __restrict
 // the int32 form).  Columns are int16 offsets from the row (Ctl::col16) when
 // k_rows found that every one fits, int32 otherwise; the same entries are
 // summed in the same order either way.
+//
+// spread: also count into Ctl::cl_far the entries outside the rows of their
+// row's block, among gathers (entry k of a slice's 32 rows) that reach four
+// blocks or more; blocks as the cluster kernel divides the rows.
 __global__ void k_fill(Ctl* c, const int32_t* __restrict__ rp, const int32_t* __restrict__ col,
                        const double* __restrict__ val, const uint32_t* __restrict__ slice_w,
                        const int32_t* __restrict__ slice_ptr, int32_t* __restrict__ scol,
-                       float* __restrict__ sv32, double* __restrict__ sv64, int n, int nslices) {
+                       float* __restrict__ sv32, double* __restrict__ sv64, int n, int nslices, int spread) {
   if (volatile_status(c) != 0) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int s = i >> 5, lane = i & 31;
@@ -259,6 +263,7 @@ __global__ void k_fill(Ctl* c, const int32_t* __restrict__ rp, const int32_t* __
     a = rp[i];
     len = rp[i + 1] - a;
   }
+  int far = 0;
   for (int k = 0; k < w; ++k) {
     const int e = base + kSlice * k;
     double v = 0.0;
@@ -271,7 +276,14 @@ __global__ void k_fill(Ctl* c, const int32_t* __restrict__ rp, const int32_t* __
     else scol[e] = cc;
     sv64[e] = v;
     sv32[e] = (float)v;
+    if (spread) {
+      const int o = cl_owner(nslices, cc >> 5);
+      const unsigned blocks = __reduce_or_sync(0xffffffffu, 1u << o);
+      const unsigned out = __ballot_sync(0xffffffffu, o != cl_owner(nslices, s));
+      if (__popc(blocks) >= 4) far += __popc(out);
+    }
   }
+  if (far && lane == 0) atomicAdd(&c->cl_far, far);
 }
 
 // ||b||_2 in double: per-block partial sums, then a fixed-order final sum.
@@ -286,13 +298,14 @@ __global__ void k_bnorm_partial(const double* __restrict__ b, int n, double* __r
   if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
-__global__ void k_bnorm_final(Ctl* c, const double* __restrict__ part, int nb) {
+__global__ void k_bnorm_final(Ctl* c, const double* __restrict__ part, int nb, int cl_line) {
   __shared__ double sm[33];
   double s = block_sum_global(part, nb, sm);
   if (threadIdx.x == 0) {
     double bn = sqrt(s);
     c->t_prep = globaltimer();
     c->bnorm64 = bn;
+    c->small = c->cl_far <= cl_line ? 1 : 0;
     if (!isfinite(bn)) set_status(c, MPCG_ERR_NAN);
     else if (bn == 0.0) c->trivial = 1;
   }
@@ -307,7 +320,7 @@ cudaError_t launch_init(const Launch& L, const mpcg_options_t& o, int fp64_only)
   return cudaGetLastError();
 }
 
-cudaError_t launch_prep(const Launch& L, const double* b) {
+cudaError_t launch_prep(const Launch& L, const double* b, int cl_line) {
   const Dims& d = L.d;
   const int threads = 256;
   const int blocks = (int)(((long long)d.nslices * kSlice + threads - 1) / threads);
@@ -316,12 +329,12 @@ cudaError_t launch_prep(const Launch& L, const double* b) {
   k_scan<<<1, kScanThreads, 0, L.st>>>(L.ws.slice_w, L.ws.slice_ptr, d.nslices);
   k_fill<<<blocks, threads, 0, L.st>>>(L.ws.ctl, L.A->row_ptr, L.A->col, L.A->val, L.ws.slice_w,
                                        L.ws.slice_ptr, L.ws.scol, L.ws.sv32, L.ws.sv64, d.n,
-                                       d.nslices);
+                                       d.nslices, cl_line >= 0 && cl_line != kClAlways ? 1 : 0);
   if (b) {
     int nb = (d.n + 255) / 256;
     if (nb > kNormBlocks) nb = kNormBlocks;
     k_bnorm_partial<<<nb, 256, 0, L.st>>>(b, d.n, L.ws.partials);
-    k_bnorm_final<<<1, 1024, 0, L.st>>>(L.ws.ctl, L.ws.partials, nb);
+    k_bnorm_final<<<1, 1024, 0, L.st>>>(L.ws.ctl, L.ws.partials, nb, cl_line);
   }
   return cudaGetLastError();
 }

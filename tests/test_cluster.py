@@ -4,7 +4,7 @@ An explicit grid size keeps the grid-wide kernels, so the same call runs both
 ways.  Sizes at the edges: one row, a ragged last slice, fewer slices than
 blocks, one slice more than fills a block's 16 warps, every instance (rows
 per thread), the largest size, and one past it (both calls then take the
-grid).  The two ways sum the inner products in another order, so counts may
+grid), and matrices with scattered columns, which take it too.  The two ways sum the inner products in another order, so counts may
 differ by 2 % (at least 1), x within the parity bar of 1e-6; l~, the class
 and the status are equal."""
 import numpy as np
@@ -75,6 +75,42 @@ def test_cluster_against_grid(mp, name, mode):
     assert torch.linalg.vector_norm(xc - xg) <= 1e-6 * torch.linalg.vector_norm(xg)
     x2, r2 = mp.solve(dA, db, S, **MODES[mode])
     assert torch.equal(xc, x2)  # the sums have a fixed order
+
+
+ROUTES = {  # past 4,096 rows: whether the cluster kernel runs the system
+    "rreg_4097": (lambda: synth.random_regular_laplacian(4097, 8, 1e-3, seed=4), True),
+    "rreg_12000": (lambda: synth.random_regular_laplacian(12000, 8, 1e-3, seed=4), False),
+    "rreg_20000": (lambda: synth.random_regular_laplacian(20000, 8, 1e-3, seed=4), False),
+    "rtree_9000": (lambda: synth.random_tree_plus(9000, 0.5, 3.0, seed=8), True),
+    "rtree_36000": (lambda: synth.random_tree_plus(36000, 0.5, 3.0, seed=8), False),
+    "grid_2000x15": (lambda: synth.laplacian_2d(2000, 15, sigma=1e-2), True),  # neighbours two blocks away
+    "cube_30": (lambda: synth.laplacian_3d(30, sigma=1e-2), True),
+}
+
+
+@pytest.mark.parametrize("mode", ["eps1", "fp64", "auto"])
+@pytest.mark.parametrize("name", sorted(ROUTES))
+def test_scattered_columns_take_the_grid(mp, name, mode):
+    """A matrix whose gathers are scattered over the cluster's blocks runs in the
+    grid-wide kernels, which are then faster: x is theirs to the last bit (a call
+    that asks for a grid as large as the device takes), where the cluster's sums
+    have another order.  (Algorithm II has another grid then, so x is compared
+    with the bars of the two ways.)"""
+    make, cluster = ROUTES[name]
+    A = make()
+    _, b = synth.rhs(A, seed=5)
+    feat, cls = synth.random_sample(300, seed=2)
+    S = mp.DeviceSample(feat, cls) if mode == "auto" else None
+    dA, db = mp.DeviceCSR.from_host(A), torch.from_numpy(b).cuda()
+    x, r = mp.solve(dA, db, S, **MODES[mode])
+    xg, rg = mp.solve(dA, db, S, grid_blocks=4096, **MODES[mode])
+    assert r["status"] == rg["status"] and (r["cls"], r["pdiam"]) == (rg["cls"], rg["pdiam"])
+    assert torch.linalg.vector_norm(x - xg) <= 1e-6 * torch.linalg.vector_norm(xg)
+    if mode != "auto":
+        assert torch.equal(x, xg) != cluster
+    zero = torch.zeros_like(db)
+    x, r = mp.solve(dA, zero, S, **MODES[mode])
+    assert r["status"] == mp.OK and not x.any()
 
 
 def test_cluster_statuses(mp):
