@@ -309,15 +309,19 @@ static __device__ BlockBfsOut block_bfs2(const BlockBfs& b, int srcA, int srcB) 
 }
 
 // 2BFS of a connected graph in one block.  Returns false (in every thread)
-// if vertex 0 does not reach all n vertices, or the search was stopped; then
-// nothing is written.
-static __device__ bool block_pseudo_diameter(const BlockBfs& b, int* pdiam, int* t_out) {
+// if vertex 0 does not reach all n vertices (*apart is set) or the search was
+// stopped; then nothing else is written.
+static __device__ bool block_pseudo_diameter(const BlockBfs& b, int* pdiam, int* t_out, bool* apart) {
+  *apart = false;
   if (b.g.n <= 0) return false;
   const int guess = b.dual ? b.g.n - 1 : -1;
   int src = 0;
   for (int pass = 0; pass < 2; ++pass) {
     const BlockBfsOut o = block_bfs2(b, src, pass == 0 ? guess : -1);
-    if (o.reached != b.g.n) return false;
+    if (o.reached != b.g.n) {
+      *apart = o.reached >= 0;
+      return false;
+    }
     if (pass == 1) {
       *pdiam = o.la;
     } else {

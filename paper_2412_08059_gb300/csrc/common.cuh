@@ -62,6 +62,7 @@ struct Ctl {
   int eps1_ready;  // fused stage 1: 0 pending, t + 1 when the kNN chose t, -1 on failure
   int x32_src;     // stage-1 result: -1 = x32, s >= 0 = snapshot slot s
   int pd_done;     // the one-block 2BFS has succeeded
+  int pd_apart;    // it has found that vertex 0 does not reach every vertex
   int feat_sides;  // cluster kernel: sides of the features (l~, v) that are complete
   int cl_begun;    // cluster kernel, Algorithm II: clusters that have begun
   int cl_far;      // stored entries whose gathers are spread over the cluster's blocks (k_fill)

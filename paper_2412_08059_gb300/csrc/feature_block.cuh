@@ -40,8 +40,9 @@ constexpr int kPdMaxN = 300000;
 constexpr int kPdSmallN = 16384;
 
 // l~ by the calling block, into the control block (pd_done set).  False (in
-// every thread) if the graph has more than one component, its frontier grows
-// past the limits, or on an error or a cancel; then nothing is written.
+// every thread) if the graph has more than one component (pd_apart set: the
+// group goes on with the components, without another search from vertex 0),
+// its frontier grows past the limits, or on an error or a cancel.
 static __device__ bool block_pdiam(const BlockGraph& g, const BfsGraph& q, unsigned char* smem, int smem_bytes) {
   Ctl* ctl = q.ctl;
   int32_t* const gq[4] = {q.fq0, q.fq1, q.fq2, q.fq3};
@@ -49,8 +50,10 @@ static __device__ bool block_pdiam(const BlockGraph& g, const BfsGraph& q, unsig
   b.wide = g.n <= kPdSmallN ? 2048 : 1280;
   b.grow = g.n <= kPdSmallN ? 0 : 8;
   int pd = 0, tv = 0;
-  const bool ok = block_pseudo_diameter(b, &pd, &tv);
+  bool apart = false;
+  const bool ok = block_pseudo_diameter(b, &pd, &tv, &apart);
   __syncthreads();
+  if (apart && threadIdx.x == 0) ctl->pd_apart = 1;
   if (ok && threadIdx.x == 0) {
     ctl->pdiam = pd;
     ctl->far_t = tv;

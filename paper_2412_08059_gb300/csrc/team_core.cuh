@@ -1337,7 +1337,8 @@ static __device__ __noinline__ void block_bfs_system(const BatchSys* sp, int sme
                      c16 ? (const void*)s.w.scol16 : (const void*)s.w.scol, s.n, c16 ? 1 : 0};
   const BlockBfs b = block_bfs_layout(g, team_dyn, smem_bytes, reinterpret_cast<uint32_t*>(s.w.ckey), gq, nullptr);
   int pd = 0, tv = 0;
-  const bool ok = block_pseudo_diameter(b, &pd, &tv);
+  bool apart;
+  const bool ok = block_pseudo_diameter(b, &pd, &tv, &apart);
   if (threadIdx.x == 0) {
     if (ok) {
       ctl->pdiam = pd;

@@ -43,6 +43,11 @@ CASES = {
     "rreg_40000": lambda: synth.random_regular_laplacian(40000, 8, 1e-3, seed=5),
     "band_20000": lambda: synth.banded(20000, 15, 0.6, 1.1, seed=7),
     "two_parts": lambda: _two(synth.laplacian_2d(300, 20), synth.laplacian_2d(50, 50)),
+    "two_thin": lambda: _two(synth.laplacian_2d(20, 900), synth.laplacian_2d(20, 900)),
+    "lone_first": lambda: _two(synth.laplacian_2d(1, 1), synth.laplacian_2d(30, 700)),  # vertex 0 by itself
+    "lone_last": lambda: _two(synth.laplacian_2d(30, 700), synth.laplacian_2d(1, 1)),
+    "forest": lambda: synth.banded(30000, 3, 0.9, 1.1, seed=3),
+    "no_edges": lambda: synth.banded(20000, 3, 0.0, 1.1, seed=3),
 }
 
 
@@ -53,5 +58,10 @@ def test_block_pdiam(mp, name):
     want, t = oracle.pseudo_diameter(A, return_t=True)
     assert mp.pseudo_diameter(dA) == (want, t)
     _, b = synth.rhs(A, seed=3)
-    f = mp.features(dA, torch.from_numpy(b).cuda())
+    db = torch.from_numpy(b).cuda()
+    f = mp.features(dA, db)
     assert f["pdiam"] == want and f["status"] in (mp.OK, mp.WARN_EPS1_NOT_REACHED)
+    # beside the iterations of a solve: the same search by the feature blocks
+    feat, cls = synth.random_sample(60, seed=2)
+    x, r = mp.solve(dA, db, mp.DeviceSample(feat, cls), max_it_fp64=1, max_true_restarts=0)
+    assert r["pdiam"] == want
