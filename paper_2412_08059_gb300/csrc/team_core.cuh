@@ -45,6 +45,7 @@ constexpr int kScanSmem = kBScanTile * 4 + kBatchThreads * 8;  // the scan's til
 // shared-memory carve-out, so the L1 cache keeps 124 KB of the 256 KB.
 constexpr int kTeamSmem = kBatchWarps * kStageWarpBytes;
 static_assert(kTeamSmem >= kScanSmem, "scan buffer");
+constexpr int kTeamSearch = 4, kTeamWide = 8192;  // (team_pseudo_diameter)
 constexpr int kBlockBfsMaxN = 1 << 18;         // larger systems run the 2BFS over the whole team
 
 // One system of the batch (device copy written by the host).
@@ -1322,20 +1323,21 @@ static __device__ int batch_take(BatchHdr* h, const int* order, int c) {
 }
 
 // Block-local 2BFS of one system (every thread of the calling block):
-// ctl->pdiam, far_t, reached and connected = 1 if the graph is connected,
-// else only connected = 0.  Not inlined: its code then leaves the register
+// ctl->pdiam, far_t, reached and connected = 1 if the graph is connected and
+// no frontier has more than `wide` entries (0: no limit), else only connected = 0.  Not inlined: its code then leaves the register
 // allocation of the CG loops in the same kernel alone (measured: inlined, the
 // FP64 stage of a 512-system batch ran 12 % slower), and only the system's
 // pointer crosses the call, so the search itself keeps its state in
 // registers.
-static __device__ __noinline__ void block_bfs_system(const BatchSys* sp, int smem_bytes) {
+static __device__ __noinline__ void block_bfs_system(const BatchSys* sp, int smem_bytes, int wide) {
   const BatchSys& s = *sp;
   Ctl* ctl = s.w.ctl;
   int32_t* const gq[4] = {s.w.fq0, s.w.fq1, s.w.fq2, s.w.fq3};
   const bool c16 = ctl->col16 != 0;
   const BlockGraph g{s.A.row_ptr, s.A.col, s.w.slice_ptr, s.w.slice_w,
                      c16 ? (const void*)s.w.scol16 : (const void*)s.w.scol, s.n, c16 ? 1 : 0};
-  const BlockBfs b = block_bfs_layout(g, team_dyn, smem_bytes, reinterpret_cast<uint32_t*>(s.w.ckey), gq, nullptr);
+  BlockBfs b = block_bfs_layout(g, team_dyn, smem_bytes, reinterpret_cast<uint32_t*>(s.w.ckey), gq, nullptr);
+  b.wide = wide;
   int pd = 0, tv = 0;
   bool apart;
   const bool ok = block_pseudo_diameter(b, &pd, &tv, &apart);
@@ -1359,11 +1361,16 @@ static __device__ __noinline__ int team_vote(const KnnSpec* knn, const double* c
 // Connected systems of up to kBlockBfsMaxN rows: the team's first block runs
 // both searches alone in shared memory (bfs_block.cuh) while the others wait
 // at the barrier.  Larger or disconnected systems (and launches without the
-// shared buffer): the team version over all of the team's blocks.
+// shared buffer): the team version over all of the team's blocks.  So do, in
+// teams of at least kTeamSearch blocks, those whose frontiers grow past
+// kTeamWide entries of both searches (a cube of 2^18 vertices reaches 6,144):
+// the eight warps of one block bound a wide level.  8-regular graph of 149,382
+// vertices on 16 plan blocks: 6.7 ms by one block; 64 such graphs of 1e3 to
+// 1.5e5 vertices in a batch 10.1 ms, and 7.8 with the limit.
 static __device__ bool team_pseudo_diameter(Team& t, const BatchSys& s, int smem_bytes) {
   Ctl* ctl = s.w.ctl;
   if (s.n >= 1 && s.n <= kBlockBfsMaxN && smem_bytes > 0) {
-    if (t.rank == 0) block_bfs_system(&s, smem_bytes);
+    if (t.rank == 0) block_bfs_system(&s, smem_bytes, t.size >= kTeamSearch ? kTeamWide : 0);
     if (!team_sync(t)) return false;
     if (*reinterpret_cast<volatile int*>(&ctl->connected)) return true;
   }
