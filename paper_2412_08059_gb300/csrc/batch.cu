@@ -198,12 +198,17 @@ int team_grid(const void* kernel, int requested, int smem) {
 // the batch is bound by the sum of its work: two systems an SM hide each
 // other's latency.  It gets both when it is what the launch would wait for:
 // more than kHalfRows rows (below, the team barriers cost what the second
-// block gives) and more work than a launch block's share of the batch.  One
-// launch block each at every size, with few systems: 9.7 ms for 12 systems of
-// up to 8e4 rows (FP64, 16384 rows a block; now 6.8), 29.5 ms for 13 of up to
-// 4.7e4 (eps1 chosen; now 17.3).  12 systems of up to 6000 rows: 3.4 ms with
-// the line at 2048 rows, 3.8 at 4096, 4.0 at 8192; of up to 3000 rows 2.6 ms
-// with each.
+// block gives) and more work than a launch block's share of the batch, by the
+// whole solves (work_of) or by one iteration (nnz + 6 n): the iterations of a
+// well-conditioned matrix do not grow with n, and then the largest systems of
+// one plan block are what the launch waits for, although larger ones on many
+// blocks have more work by work_of.  With one launch block for every system of
+// one plan block against this rule: 12 systems of up to 8e4 rows (FP64, 16384
+// rows a block) 9.7 and 6.8 ms, 13 of up to 4.7e4 (eps1 chosen) 29.5 and 17.3.
+// By the whole solves alone against this rule, 64 systems of 1e3 to 1.5e5 rows
+// in FP64: 8-regular graphs 5.07 and 4.73 ms, bands of width 15 6.52 and 6.02.
+// The line in rows, 12 systems of up to 6000 rows: 3.4 ms at 2048, 3.8 at 4096,
+// 4.0 at 8192; of up to 3000 rows 2.6 ms with each.
 constexpr int kHalfRows = 2048;
 
 Plan make_plan(int nsys, const int* n, const double* work, int grid, int rows_per_block,
@@ -215,15 +220,18 @@ Plan make_plan(int nsys, const int* n, const double* work, int grid, int rows_pe
   std::vector<double> w(nsys);
   double cw[kTeamQueues] = {0};
   int cnt[kTeamQueues] = {0};
-  double share = 0.0;
+  double share = 0.0, turn = 0.0;
   for (int i = 0; i < nsys; ++i) {
     const int rpb = rows_sys && rows_sys[i] > 0 ? rows_sys[i] : rows_per_block;
     w[i] = work[i];
     share += w[i] / blocks;
+    turn += w[i] / sqrt((double)n[i]) / blocks;
     cls[i] = size_class(n[i], rpb) + 1;
   }
   for (int i = 0; i < nsys; ++i)
-    if (cls[i] == 1 && !whole_blocks && !(n[i] > kHalfRows && w[i] > share)) cls[i] = 0;
+    if (cls[i] == 1 && !whole_blocks &&
+        !(n[i] > kHalfRows && (w[i] > share || w[i] / sqrt((double)n[i]) > turn)))
+      cls[i] = 0;
   // Demote the largest classes while one team of every non-empty class does
   // not fit in the grid.
   const int least = whole_blocks ? 1 : 0;
