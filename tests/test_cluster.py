@@ -113,25 +113,58 @@ def test_scattered_columns_take_the_grid(mp, name, mode):
     assert r["status"] == mp.OK and not x.any()
 
 
-def test_cluster_statuses(mp):
-    """b = 0, NaN in b, an indefinite matrix, a cap, a cancel word set, a broken CSR."""
+@pytest.mark.parametrize("mode", sorted(MODES))
+def test_cluster_statuses(mp, mode):
+    """b = 0, NaN in b, an indefinite matrix, a cap, a cancel word set, a broken CSR;
+    in Algorithm II (the 2BFS cluster beside CG) also a label that is no class.
+    Both ways end alike, and a call after them is right."""
     A = _grid(3000)
     _, b = synth.rhs(A, seed=5)
+    feat, cls = synth.random_sample(300, seed=2)
+    S = mp.DeviceSample(feat, cls) if mode == "auto" else None
+    kw = dict(MODES[mode])
     dA, db = mp.DeviceCSR.from_host(A), torch.from_numpy(b).cuda()
-    x, r = mp.solve(dA, torch.zeros_like(db), eps1=1e-4)
+    want, _ = mp.solve(dA, db, S, **kw)
+
+    def both(A_, b_, S_=S, **more):
+        r = mp.solve(A_, b_, S_, **kw, **more)[1]
+        g = mp.solve(A_, b_, S_, grid_blocks=4096, **kw, **more)[1]
+        assert r["status"] == g["status"], (r, g)
+        return r, g
+
+    x, r = mp.solve(dA, torch.zeros_like(db), S, **kw)
     assert r["status"] == mp.OK and not x.any()
     bad = db.clone()
     bad[1234] = float("nan")
-    for kw in (dict(eps1=1e-4), dict(fp64_only=1)):
-        assert mp.solve(dA, bad, **kw)[1]["status"] == mp.ERR_NAN
-        neg = mp.DeviceCSR(dA.row_ptr, dA.col, -dA.val)
-        assert mp.solve(neg, db, **kw)[1]["status"] == mp.ERR_BREAKDOWN
-        r = mp.solve(dA, db, max_it_fp64=3, max_it_fp32=2, **kw)[1]
-        g = mp.solve(dA, db, max_it_fp64=3, max_it_fp32=2, grid_blocks=4096, **kw)[1]
-        assert r["status"] == g["status"] == mp.ERR_NOT_CONVERGED and r["n2"] == g["n2"] == 3
-        assert abs(r["true_rel_resid"] - g["true_rel_resid"]) <= 1e-6 * g["true_rel_resid"]
-        word = torch.ones(1, dtype=torch.int32, pin_memory=True)
-        assert mp.solve(dA, db, cancel=word.data_ptr(), **kw)[1]["status"] == mp.ERR_CANCELLED
+    assert both(dA, bad)[0]["status"] == mp.ERR_NAN
+    # d^T A d < 0 at the first iteration: in Algorithm II a breakdown in the k0 phase
+    assert both(mp.DeviceCSR(dA.row_ptr, dA.col, -dA.val), db)[0]["status"] == mp.ERR_BREAKDOWN
+    r, g = both(dA, db, max_it_fp64=3, max_it_fp32=2)
+    assert r["status"] == mp.ERR_NOT_CONVERGED and r["n2"] == g["n2"] == 3 and r["n1"] == g["n1"]
+    assert abs(r["true_rel_resid"] - g["true_rel_resid"]) <= 1e-6 * g["true_rel_resid"]
+    word = torch.ones(1, dtype=torch.int32, pin_memory=True)
+    assert both(dA, db, cancel=word.data_ptr())[0]["status"] == mp.ERR_CANCELLED
     col = dA.col.clone()
     col[0] = A.n
-    assert mp.solve(mp.DeviceCSR(dA.row_ptr, col, dA.val), db, eps1=1e-4)[1]["status"] == mp.ERR_INVALID_ARG
+    assert both(mp.DeviceCSR(dA.row_ptr, col, dA.val), db)[0]["status"] == mp.ERR_INVALID_ARG
+    if mode == "auto":
+        for label in (-1, 16, 77):
+            assert both(dA, db, mp.DeviceSample(feat, np.full_like(cls, label)))[0]["status"] == mp.ERR_INVALID_ARG
+        mixed = cls.copy()
+        mixed[::2] = 16  # valid classes are met before the vote finds the label
+        assert both(dA, db, mp.DeviceSample(feat, mixed), knn_k=64)[0]["status"] == mp.ERR_INVALID_ARG
+    assert torch.equal(mp.solve(dA, db, S, **kw)[0], want)
+
+
+def test_label_wait_that_runs_out(mp):
+    """Every class of the sample is met long before the 2BFS of a long path ends: CG
+    waits for the label until its time limit, and the call ends with the status."""
+    A = synth.path(30000)
+    _, b = synth.rhs(A, seed=5)
+    feat, _ = synth.random_sample(60, seed=2)
+    S = mp.DeviceSample(feat, np.full(60, 1, np.int8))
+    dA, db = mp.DeviceCSR.from_host(A), torch.from_numpy(b).cuda()
+    for kw in (dict(), dict(grid_blocks=4096)):
+        assert mp.solve(dA, db, S, timeout_ms=2, **kw)[1]["status"] == mp.ERR_TIMEOUT
+    x, r = mp.solve(dA, db, S)
+    assert r["status"] >= 0 and r["pdiam"] == A.n - 1

@@ -125,7 +125,10 @@ def mp():
 @pytest.mark.gpu
 @pytest.mark.parametrize("count,k,weighted,mask", [(1, 5, 1, 0xF), (7, 5, 1, 0xF), (300, 1, 1, 0xE),
                                                     (300, 20, 0, 0xE), (2000, 15, 1, 0xF),
-                                                    (150, 64, 1, 0x7)])
+                                                    (150, 64, 1, 0x7),
+                                                    # one tile of the scaled sample, and several
+                                                    (4095, 5, 1, 0xF), (4096, 64, 1, 0xF), (4097, 5, 1, 0xF),
+                                                    (9001, 33, 0, 0xE)])
 def test_knn_batch_matches_oracle(mp, count, k, weighted, mask):
     feat, cls = synth.random_sample(count, seed=count + k)
     rng = np.random.default_rng(count)
@@ -142,6 +145,30 @@ def test_knn_batch_matches_oracle(mp, count, k, weighted, mask):
         if t >= 0:
             kk = min(k, count)
             assert list(nbr[i, :kk]) == list(nb) and np.all(nbr[i, kk:] == -1)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("count", [60, 4200])
+def test_knn_batch_beyond_the_filter(mp, count):
+    """Scaled values past 1e15, or not finite: no distance is left to single precision.  A
+    NaN in the sample makes every query invalid."""
+    feat, cls = synth.random_sample(count, seed=count)
+    rng = np.random.default_rng(count)
+    lo, hi = feat.min(axis=0), feat.max(axis=0)
+    q = feat[rng.integers(0, count, 37)] * rng.uniform(0.7, 1.3, (37, 4))
+    q[:9] *= 1e16                               # the query alone
+    far, inf, nan = feat.copy(), feat.copy(), feat.copy()
+    far[::5] = lo + (hi - lo) * 1e17 * rng.uniform(-1, 1, (far[::5].shape[0], 4))
+    far[::7] *= 1e170                           # squares past the type's range
+    inf[3, 1], inf[-1, 3] = np.inf, -np.inf
+    nan[count // 2, 0] = np.nan
+    for f in (feat, far, inf):
+        S, Sh = mp.DeviceSample(f, cls, lo, hi), oracle.sample(f, cls, lo, hi)
+        got, nbr = mp.knn_batch(q, S, neighbours=True, knn_k=7)
+        for i, qi in enumerate(q):
+            t, nb, _ = oracle.knn(qi, Sh, k=7, details=True)
+            assert got[i].item() == t and list(nbr[i].cpu().numpy()) == list(nb), i
+    assert (mp.knn_batch(q, mp.DeviceSample(nan, cls, lo, hi)) == -1).all()
 
 
 @pytest.mark.gpu

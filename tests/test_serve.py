@@ -238,3 +238,28 @@ def test_serve_step_does_not_wait_for_earlier_stream_work(mp):
         assert close_count(res["n1"], ro["n1"]) and close_count(res["n2"], ro["n2"])
         assert np.linalg.norm(x - xo) <= 1e-6 * np.linalg.norm(xo)
     srv.close()
+
+
+@pytest.mark.parametrize("mode", ["fp64", "auto"])
+def test_serve_steps_do_not_change_the_result(mp, mode):
+    """A system suspended after every few iterations ends with the same x, to the last
+    bit, as in one long step.  With this many rows a block keeps part of r in shared
+    memory and part in the workspace (8,192 rows a launch block fit)."""
+    mats = [synth.laplacian_2d(200, 201, sigma=1e-2), synth.laplacian_3d(33, sigma=1e-2), synth.path(901)]
+    feat, cls = sample_over(mats)
+    kw = dict(fp64_only=1) if mode == "fp64" else {}
+    S = mp.DeviceSample(feat, cls) if mode == "auto" else None
+    got = []
+    for iters in (100000, 40, 7, 1):
+        srv = mp.Server(4, sum(mp.workspace_bytes(A.n, A.nnz) + 256 for A in mats),
+                        mp.options(team_rows=1 << 16, **kw), S)
+        reqs = [Request(mp, A, synth.rhs(A, seed=40 + i)[1]) for i, A in enumerate(mats)]
+        for q in reqs:  # one at a time: the planner then gives it the same blocks every step
+            serve(mp, srv, [q], [[q]], iters)
+        got.append([q.result(mp) for q in reqs])
+        srv.close()
+    for other in got[1:]:
+        for (x0, r0), (x, r) in zip(got[0], other):
+            assert r["status"] == r0["status"] == 0 and (r["n1"], r["n2"]) == (r0["n1"], r0["n2"])
+            assert r["team_blocks"] == r0["team_blocks"] == 1
+            assert np.array_equal(x, x0)
