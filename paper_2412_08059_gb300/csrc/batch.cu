@@ -1,11 +1,12 @@
 // batch.cu -- many independent systems in one persistent launch (a batching
 // pattern; the paper solves one system at a time).
 //
-// The grid (one block per SM, cooperative) is split into teams of 1, 2, 4,
-// ..., 128 blocks.  A host-side planner puts every system in the queue of a
-// team-size class (larger systems, larger teams; largest first) and gives
-// each class a number of teams in proportion to its estimated work.  The
-// leader of a team takes the next system from its class queue, or, when
+// The plan has one block per SM, split into teams of 1, 2, 4, ..., 128 blocks;
+// the launch (cooperative) has two blocks per SM for each of them, and a
+// system of one plan block runs on one or on both (make_plan).  A host-side
+// planner puts every system in the queue of a team-size class (larger
+// systems, larger teams; largest first) and gives each class a number of
+// teams in proportion to its estimated work.  The leader of a team takes the next system from its class queue, or, when
 // that queue is empty, from a queue of a smaller class; the team then runs
 // the whole method on it and writes its result record:
 //   set-up (CSR check, b~ = float32(b), sliced layout, ||b||),

@@ -506,13 +506,14 @@ __device__ __forceinline__ T row_tail(const CgArgs& a, int i, int w, T acc, Gath
 // One SpMV pass over the block's slices by the consumer warps.  For every
 // row i of the block's slices (padding rows included), Rw(i, acc) receives
 // sum_k v_k G(c_k) in stored order.  A warp takes two adjacent slices per
-// step (one when the block has no more slices than warps, or wide ones), so that the gathers
-// of both rows are in flight together; their entries are contiguous, at most 2 x 32 x 64 = kCH of them, so a step never
-// needs more than two chunks at once (the ring has at least four), which
-// keeps the producer/consumer ring free of deadlock.  The next step's widths
-// and offsets are loaded a step ahead: they come from L2 (the gathers evict
-// them from L1), and a step would otherwise start with that round trip.
-// Returns false if a wait failed.
+// step (one when the block has no more slices than warps, or wide ones), so
+// that the gathers of both rows are in flight together; their entries are
+// contiguous, at most 2 x 32 x 64 = kCH of them, so a step never needs more
+// than two chunks at once (the ring has at least four), which keeps the
+// producer/consumer ring free of deadlock.  The next step's widths and offsets
+// are loaded a step ahead: they come from L2 (the gathers evict them from L1),
+// and a step would otherwise start with that round trip.  Returns false if a
+// wait failed.
 template <int NC, typename T, class Gather, class Row>
 __device__ __forceinline__ bool ring_spmv(const CgArgs& a, Ring<T>& R, Cursor& C, int S0, int S1,
                                           Gather G, Row Rw) {
@@ -1367,10 +1368,12 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_cg64(CgArgs a) {
 // Fused single-precision stage of Algorithm II.
 //
 // The 2BFS of Sec. 6 is a chain of grid-wide levels (latency-bound); CG is
-// bandwidth-bound.  This kernel runs them side by side: in every block one
-// feature warp runs the 2BFS (with the component rule) on its own bounded
-// barrier, and in block 0 it then runs the kNN vote once v (Eq. 13) is
-// known; fourteen consumer warps run CG from x~0 = 0 meanwhile.
+// bandwidth-bound.  This kernel runs them side by side.  With feature blocks
+// (kFeat, the usual form) the last sixteen blocks of the grid run the 2BFS and
+// then, once v (Eq. 13) is known, the kNN vote, and fifteen consumer warps in
+// each of the others run CG from x~0 = 0 meanwhile.  Without, one feature warp
+// in every block runs the 2BFS on a bounded barrier of its own, that of block 0
+// then the vote, and fourteen consumer warps a block run CG.
 //
 // Past the k0 iterations the consumers keep iterating before the label is
 // known.  For every class t present in the sample they record the first
@@ -1385,7 +1388,8 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_cg64(CgArgs a) {
 // buffer (one extra slot written by block 0), so all blocks take the same
 // decisions.
 // ---------------------------------------------------------------------------------------
-constexpr int kNC1 = 14;      // consumer warps; warp 14 = feature warp, warp 15 = producer
+// Without feature blocks: consumer warps (warp 14: feature warp, 15: producer).
+constexpr int kNC1 = 14;
 constexpr int kSnapSlots = 6; // snapshots of x~ kept in the workspace
 
 struct Stage1Args {
@@ -1417,8 +1421,12 @@ __device__ __noinline__ bool stage1_pdiam(const BfsGraph g, int32_t* d1, int32_t
 // blocks are too few for wide levels (random 8-regular graph of 2^20 vertices,
 // 2BFS alone: 4.8 ms, 2.4 by sixteen), thirty-two cost CG a fifth of the chip.
 constexpr int kFeatBlocks = 16;
-// The feature blocks: the 2BFS; then, in the first, v (bounded wait for block 0's consumers) and the vote.  Every block
-// of the launch is resident (cooperative launch), so the wait ends.
+// (Past the vote these blocks have nothing to do, a tenth of the chip: 128^3
+// anisotropic systems take 37 us an iteration here and 34.1 in k_cg32.)
+//
+// The feature blocks: the 2BFS; then, in the first, v (bounded wait for block
+// 0's consumers) and the vote.  Every block of the launch is resident
+// (cooperative launch), so the wait ends.
 __device__ __noinline__ void stage1_feature_block(const Stage1Args& sa, unsigned char* smem, int first) {
   const CgArgs& a = sa.a;
   Ctl* ctl = a.ctl;

@@ -223,8 +223,8 @@ __device__ __forceinline__ double cl_total_ff(ClShared& S, int rank, int ns, int
 // targets), and a row's gathers bound the iteration (n = 3,001 random tree:
 // 4,900 of 15,500 clocks).  (8-regular graph of 2,000 rows: 6.6 us a
 // double-precision iteration that way, 5.7 with whole copies; tree of 4,000
-// rows 7.9 and 7.2, in single precision 7.6 and 6.1.)  Up to kClRepN rows every block then keeps the whole
-// vector: the owner writes each value to all sixteen, the entries' owner is
+// rows 7.9 and 7.2, in single precision 7.6 and 6.1.)  Up to kClRepN rows
+// every block then keeps the whole vector: the owner writes each value to all sixteen, the entries' owner is
 // the block itself, and a gather stays in its own shared memory.
 constexpr int kClRepN = 4096;
 struct ClMat {

@@ -63,7 +63,7 @@ struct Ctl {
   int x32_src;     // stage-1 result: -1 = x32, s >= 0 = snapshot slot s
   int pd_done;     // the one-block 2BFS has succeeded
   int pd_apart;    // it has found that vertex 0 does not reach every vertex
-  int feat_sides;  // cluster kernel: sides of the features (l~, v) that are complete
+  int feat_sides;  // sides of the features (l~, v) that are complete (k_stage1: 1 once v is)
   int cl_begun;    // cluster kernel, Algorithm II: clusters that have begun
   int cl_far;      // stored entries whose gathers are spread over the cluster's blocks (k_fill)
   int small;       // the cluster kernel runs the system, and the grid-wide kernels leave it alone
@@ -314,9 +314,9 @@ __device__ __forceinline__ bool mbar_try_wait(unsigned long long* bar, uint32_t 
 // Returns false on timeout (status set) or when *stop becomes non-zero.  A
 // try_wait that finds the phase open suspends the thread for microseconds
 // before it gives up, so *stop is read after every one: read after every
-// 64th, the producer left its kernel 0.25 ms after the consumers (measured
-// at every size: 0.25 ms between the end of the iterations and the end of
-// the call; 64 x 64 grid, fixed eps1: 2.96 ms a solve before, 2.45 ms after).
+// 64th, the producer left its kernel 0.25 ms after the consumers, at every
+// size (64 x 64 grid by the grid-wide kernels, eps1 given: 2.96 ms a solve
+// that way, 2.45 this way).
 __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, uint32_t parity, Ctl* ctl,
                                           const volatile int* stop) {
   if (mbar_try_wait(bar, parity)) return true;

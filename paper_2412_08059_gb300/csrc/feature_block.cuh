@@ -1,5 +1,6 @@
-// feature_block.cuh -- the features of Algorithm II by one block beside the
-// blocks that run CG (the cluster kernel and the fused single-precision stage).
+// feature_block.cuh -- the features of Algorithm II by one block, or by a
+// group of blocks beside those that run CG (the cluster kernel and the fused
+// single-precision stage).
 #pragma once
 #include "bfs_block.cuh"
 #include "bfs_core.cuh"
@@ -35,7 +36,9 @@ static __device__ __noinline__ void feature_vote(const KnnSpec& knn, Ctl* ctl) {
 // 1,280: a 2-D grid (2 level) of up to kPdMaxN vertices stays within that (512 x
 // 512: 5.5 against 5.9 ms), a cube leaves it at level 16 (level^2), some 50 us
 // into a search of a millisecond.  A larger square grid would leave it late
-// (700 x 700: 12.8 ms against 8.8), so larger graphs are not tried.
+// (700 x 700: 12.8 ms against 8.8), so larger graphs are not tried; that the
+// line is drawn by n keeps long thin grids past it, which would stay within
+// the limits, with the search of all blocks (5 to 6 us a level).
 constexpr int kPdMaxN = 300000;
 constexpr int kPdSmallN = 16384;
 

@@ -67,8 +67,8 @@ KnnSpec knn_spec(const mpcg_sample_t& S, const mpcg_options_t& o) {
 // single-precision distance is above the k-th distance by more than that is
 // not among the k nearest.  Past M = 1e15, or where a value is not finite,
 // every point is computed in double.
-// 4,800 queries, 1,260 points, k = 5, with neighbours: 7.37 ms when every
-// query computed every distance k + 1 times, divisions included.
+// 4,800 queries, 1,260 points, k = 5, with neighbours: 0.118 ms, against 7.37
+// by a pass of all distances, divisions included, for every neighbour.
 constexpr int kKnnWarps = 16;
 constexpr int kKnnTile = 4096;  // points of a tile: 32 + 16 bytes each
 __global__ void __launch_bounds__(kKnnWarps * 32) k_knn_batch(KnnSpec s, const double* chi4, int count,

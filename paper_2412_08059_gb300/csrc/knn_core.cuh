@@ -6,9 +6,8 @@
 // The squared Euclidean distance (Sec. 11.5) is summed over the selected
 // components in index order.  The k nearest are the k smallest pairs
 // (d2, index): one pass over the sample, 32 points at a time, keeps them as a
-// sorted list spread over the warp's lanes (a distance is computed once; the
-// form that selected one neighbour a pass computed each k + 1 times, its four
-// FP64 divisions included).  Vote: weight 1/sqrt(d2) (Eq. 23) or 1 (Eq. 22), summed in
+// sorted list spread over the warp's lanes, so that a distance, with its four
+// FP64 divisions, is computed once.  Vote: weight 1/sqrt(d2) (Eq. 23) or 1 (Eq. 22), summed in
 // selection order; when a selected neighbour is at distance 0 only the
 // zero-distance neighbours vote, by count; ties go to the smallest class t.
 // Every operation is an explicit IEEE-rounded intrinsic, so the result does

@@ -60,7 +60,7 @@ size_t carve(const Dims& d, char* base, Ws* ws) {
   w.ckey = (unsigned long long*)take(sizeof(unsigned long long) * n);
   w.snap = (float*)take(sizeof(float) * 6 * n);
   // team kernels (batched solve, server): a 16-bit copy of the columns for
-  // the staged single-precision SpMV
+  // the double-precision and the staged single-precision SpMV
   w.scol16 = (int16_t*)take(sizeof(int16_t) * P);
   w.bytes = off;
   if (ws) *ws = w;

@@ -435,13 +435,6 @@ static __device__ void sys_fill(const Team& t, const BatchSys& s, bool narrow) {
 // lane l owns row 32 s + l of slice s in every phase, so the vector updates
 // of a row are done by the thread that produced its SpMV result.
 // ---------------------------------------------------------------------------------------
-template <typename T>
-__device__ __forceinline__ const T* bvals(const BatchSys& s);
-template <>
-__device__ __forceinline__ const float* bvals<float>(const BatchSys& s) { return s.w.sv32; }
-template <>
-__device__ __forceinline__ const double* bvals<double>(const BatchSys& s) { return s.w.sv64; }
-
 // Overflow tail of row i (entries past the slice width, from the CSR).
 template <typename T, class Gather>
 __device__ __forceinline__ T btail(const BatchSys& s, int i, int w, T acc, Gather G) {
@@ -501,17 +494,17 @@ __device__ __forceinline__ int col_at(typename std::conditional<C16, int16_t, in
 // Slices wider than kTeamFastW, or with an overflow tail, read their pairs
 // from global memory instead.  The metadata of 32 of the warp's slices is
 // loaded at once (one slice per lane).
-template <typename T, bool C16, class Gather, class Pre, class Row>
+template <bool C16, class Gather, class Pre, class Row>
 __device__ __forceinline__ void team_spmv_staged(const Team& t, const BatchSys& s, Gather G, Pre P,
                                                  Row Rw) {
-  static_assert(sizeof(T) == 4, "the stages hold 4-byte values");
+  using T = float;
   using CT = typename std::conditional<C16, int16_t, int32_t>::type;
   constexpr int kS = kSpmvStep;
   constexpr int kE = kSlice * kTeamFastW;      // elements of a staged slice
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int gw = team_warp(t), W = team_warps(t);
-  const T* sv = bvals<T>(s);
+  const float* sv = s.w.sv32;
   const CT* sc;
   if constexpr (C16) sc = s.w.scol16;
   else sc = s.w.scol;
@@ -591,21 +584,23 @@ __device__ __forceinline__ void team_spmv_staged(const Team& t, const BatchSys& 
   }
 }
 
-// SpMV over the team's slices, operands from global memory (the double-
-// precision stage): warp gw owns slices gw, gw + W, ...; lane l
-// owns row 32 s + l.  Rw(i, acc, own) receives row i's sum in stored order
-// (fused multiply-adds from zero, padding rows included) and the row's own
-// values that P(i) loaded before the gathers (P gets i >= n for absent rows).  The metadata of 32 of
-// the warp's slices is loaded at once (one slice per lane) and kU slices are
-// summed together so that their loads and gathers overlap.
-template <typename T, class Gather, class Pre, class Row>
+// The single-precision SpMV with operands from global memory (the server's
+// step, which runs both stages in one kernel): warp gw owns slices gw, gw + W,
+// ...; lane l owns row 32 s + l.  Rw(i, acc, own) receives row i's sum in
+// stored order (fused multiply-adds from zero, padding rows included) and the
+// row's own values that P(i) loaded before the gathers (P gets i >= n for
+// absent rows).  32-bit columns.  The metadata of 32 of the warp's slices is
+// loaded at once (one slice per lane) and kU slices are summed together so
+// that their loads and gathers overlap.
+template <class Gather, class Pre, class Row>
 __device__ __forceinline__ void team_spmv_regs(const Team& t, const BatchSys& s, Gather G, Pre P,
                                                Row Rw) {
+  using T = float;
   constexpr int kU = 4;
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int gw = team_warp(t), W = team_warps(t);
-  const T* sv = bvals<T>(s);
+  const float* sv = s.w.sv32;
   const int32_t* sc = s.w.scol;
   for (int base = gw; base < s.nslices; base += 32 * W) {
     const int mine = base + lane * W;
@@ -653,25 +648,20 @@ __device__ __forceinline__ void team_spmv_regs(const Team& t, const BatchSys& s,
   }
 }
 
-// The SpMV of the team kernels.  The single-precision stage stages its
-// pairs in shared memory; the double-precision stage loads them from global
-// memory: staged double pairs would need 12 bytes an element, and the shared
-// memory they take comes out of the L1 cache that the stage's gathers use
-// (measured on the 512-system batch: the FP64 stage lost more to the
-// smaller L1 than it gained from the staging).
-//
-// The staged SpMV reads the 16-bit copy of the columns when the set-up built
-// one (Ctl::col16; each format has its own copy of the loop); the SpMV from
-// global memory reads the 32-bit columns, so the double-precision loops keep
-// the one form whose schedule was measured.
-template <typename T, bool kStage, class Gather, class Pre, class Row>
+// The single-precision SpMV of the team kernels: staged in shared memory, with
+// the 16-bit copy of the columns when the set-up built one (Ctl::col16; each
+// format has its own copy of the loop), or from global memory.  (The
+// double-precision one, team_spmv64, loads its pairs from global memory: staged
+// they would need 10 or 12 bytes an element, and the shared memory they take
+// comes out of the L1 cache that the gathers use.)
+template <bool kStage, class Gather, class Pre, class Row>
 __device__ __forceinline__ void team_spmv(const Team& t, const BatchSys& s, Gather G, Pre P,
                                           Row Rw) {
-  if constexpr (kStage && sizeof(T) == 4) {
-    if (s.w.ctl->col16) team_spmv_staged<T, true>(t, s, G, P, Rw);
-    else team_spmv_staged<T, false>(t, s, G, P, Rw);
+  if constexpr (kStage) {
+    if (s.w.ctl->col16) team_spmv_staged<true>(t, s, G, P, Rw);
+    else team_spmv_staged<false>(t, s, G, P, Rw);
   } else {
-    team_spmv_regs<T>(t, s, G, P, Rw);
+    team_spmv_regs(t, s, G, P, Rw);
   }
 }
 
@@ -751,9 +741,12 @@ __device__ __forceinline__ void team_step64(const BatchSys& s, const int (&p)[U]
 // slices have it: all entries and gathers of both rows in flight.  Up to K =
 // 5 the next step's columns are loaded while this step's sums run, so that a
 // step costs one round trip, its gathers; wider rows have no registers left
-// for that and take two.  (A pair of entries at a time took two round trips
-// each.)  j: the first slice's place among the warp's 32 whose metadata is at
-// hand (mwf, mp by lane), of cnt.
+// for that and take two.  (team_step64, which has the other widths, takes two
+// round trips for every pair of entries.  Forms of one slice for widths 8 and
+// 9 made batches of 15-wide bands 10 % and of trees 8 % faster, but of grids,
+// which do not use them, 5 % slower: the kernel's other loops were scheduled
+// differently.  Two slices of these widths spill.)  j: the first slice's place
+// among the warp's 32 whose metadata is at hand (mwf, mp by lane), of cnt.
 template <bool C16, int K, class Gather, class Pre, class Row>
 __device__ __forceinline__ void team_run64(const BatchSys& s, uint32_t mwf, int mp, int base, int W, int cnt,
                                            int& j, Gather G, Pre P, Row Rw) {
@@ -1021,7 +1014,7 @@ static __device__ bool sys_cg32(Team& t, const BatchSys& s, int mode, int& red, 
     float* dnew = parity ? s.w.d32a : s.w.d32b;
     const float bt = first ? 0.0f : beta;
     FF pdq{0.f, 0.f};
-    team_spmv<float, kStage>(
+    team_spmv<kStage>(
         t, s, [&](int c) -> float { return __fmaf_rn(bt, dold[c], r[c]); },
         [&](int i) -> float2 { return i < n ? make_float2(dold[i], r[i]) : make_float2(0.f, 0.f); },
         [&](int i, float acc, float2 own) {
@@ -1324,7 +1317,8 @@ static __device__ int batch_take(BatchHdr* h, const int* order, int c) {
 
 // Block-local 2BFS of one system (every thread of the calling block):
 // ctl->pdiam, far_t, reached and connected = 1 if the graph is connected and
-// no frontier has more than `wide` entries (0: no limit), else only connected = 0.  Not inlined: its code then leaves the register
+// no frontier has more than `wide` entries (0: no limit), else only
+// connected = 0.  Not inlined: its code then leaves the register
 // allocation of the CG loops in the same kernel alone (measured: inlined, the
 // FP64 stage of a 512-system batch ran 12 % slower), and only the system's
 // pointer crosses the call, so the search itself keeps its state in
@@ -1390,7 +1384,8 @@ struct Plan {
   int qbase[kTeamQueues], qlen[kTeamQueues];
 };
 // Teams for a grid of `grid` plan blocks (kBatchPerSm * grid launch blocks)
-// and the queues (teams of queue q: 2^q launch blocks) of nsys systems of n rows with estimated work `work` (largest first within a class); a system
+// and the queues (teams of queue q: 2^q launch blocks) of nsys systems of n
+// rows with estimated work `work` (largest first within a class); a system
 // goes to the smallest team with at most rows_per_block rows per block, or
 // rows_sys[i] when that array is given and its entry is positive.
 // whole_blocks (option acc32): teams of one plan block are two launch blocks
