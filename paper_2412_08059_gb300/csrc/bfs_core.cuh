@@ -56,12 +56,10 @@ struct GridSync {
   int slot;
   unsigned long long round;
   __device__ bool operator()() { return grid_barrier(ctl, slot, round); }
-  __device__ int first() const { return 0; }               // the group's first block
-  __device__ int* scratch() const { return nullptr; }      // no memory of its own for narrow levels
 };
 
-// Whole blocks `first_block` .. `first_block` + `blocks` - 1 of the grid; the
-// narrow levels' memory is the caller's (kNarrowScratch ints).
+// `blocks` whole blocks of the grid, those that call it; the narrow levels'
+// memory is the caller's (kNarrowScratch ints).
 struct BlockGroupSync {
   static constexpr bool kWholeBlock = true;
   static constexpr bool kNarrow = true;
@@ -69,11 +67,9 @@ struct BlockGroupSync {
   Ctl* ctl;
   int slot;
   unsigned long long round;
-  int first_block, blocks;
+  int blocks;
   int* mem;
   __device__ bool operator()() { return grid_barrier(ctl, slot, round, blocks); }
-  __device__ int first() const { return first_block; }
-  __device__ int* scratch() const { return mem; }
 };
 
 // One warp per block: lane 0 arrives on the counter and polls (bounded).
@@ -84,8 +80,6 @@ struct WarpGroupSync {
   Ctl* ctl;
   int slot;
   unsigned long long round;
-  __device__ int first() const { return 0; }
-  __device__ int* scratch() const { return nullptr; }
   __device__ bool operator()() {
     __syncwarp();
     round += 1;
@@ -449,13 +443,17 @@ __device__ bool bfs_run(const BfsGraph& g, int32_t* dist, int sources, int src, 
 // level).  As nothing else writes the distance arrays meanwhile, a claim is
 // a read of the candidate's distance, a shared-memory set that settles
 // candidates reached twice in the level, and a plain store (levels with a
-// row wider than kNarrowHashDeg claim by compare-and-swap instead).  The warp also writes every claimed vertex to the group's queue of
-// the next level, so that when a frontier grows past kNarrowItems it hands the
-// search back at that level with nothing to copy.  The rest of the group waits
-// on the control block's mode word: one lane of one warp a block polls it with
-// pauses (the one-warp levels are latency-bound and must not share the memory
-// system with a crowd of pollers), and in a whole-block group passes it on
-// through shared memory.
+// row wider than kNarrowHashDeg claim by compare-and-swap instead).  The warp
+// also writes every claimed vertex to the group's queue of the next level, so
+// that when a frontier grows past kNarrowItems it hands the search back at that
+// level with nothing to copy.  The rest of the group waits on the control
+// block's mode word: one lane of one warp a block polls it with pauses (the
+// one-warp levels are latency-bound and must not share the memory system with
+// a crowd of pollers).  In a whole-block group the block's other warps, also
+// those of the searching block, wait at its barrier.  Polling a copy of the
+// word in shared memory every 500 ns, they slowed the searching warp beside
+// them: Algorithm II on a 20000 x 16 grid (20,014 levels) 64.4 ms, 60.8 this
+// way.
 constexpr int kNarrowItems = 64;
 constexpr int kNarrowHash = 2048;  // shared-memory set of the level's claims (load <= 1/2)
 constexpr int kNarrowHashDeg = 16; // levels with a wider row claim by compare-and-swap
@@ -471,42 +469,28 @@ __device__ __forceinline__ bool nm_ends(int m, int L) {
   return m == -1 || (m & 3) == kNmDone || ((m & 3) == kNmResume && (m >> 2) > L);
 }
 
-template <bool kBlk>
-__device__ int nm_wait(Ctl* ctl, int L, volatile int* s_mode, int first) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const bool poller = !kBlk || warp == ((int)blockIdx.x == first ? 1 : 0);
+static __device__ int nm_wait(Ctl* ctl, int L) {  // by a whole warp
   int m = 0;
-  if (lane == 0) {
+  if ((threadIdx.x & 31) == 0) {
     const unsigned long long t0 = globaltimer();
     unsigned spins = 0;
     for (;;) {
-      if (poller) {
-        m = *reinterpret_cast<volatile int*>(&ctl->nmode);
-        if (nm_ends(m, L)) break;
-        __nanosleep(1000);
-        if ((++spins & 15u) == 0) {
-          if (volatile_status(ctl) != 0 || poll_cancel(ctl)) {
-            m = -1;
-            break;
-          }
-          if (globaltimer() - t0 > (unsigned long long)ctl->timeout_ns) {
-            set_status(ctl, MPCG_ERR_TIMEOUT);
-            m = -1;
-            break;
-          }
+      m = *reinterpret_cast<volatile int*>(&ctl->nmode);
+      if (nm_ends(m, L)) break;
+      __nanosleep(1000);
+      if ((++spins & 15u) == 0) {
+        if (volatile_status(ctl) != 0 || poll_cancel(ctl)) {
+          m = -1;
+          break;
         }
-      } else {  // the block's poller relays the word (and a failure) in shared memory
-        m = *s_mode;
-        if (nm_ends(m, L)) break;
-        __nanosleep(500);
-        if (globaltimer() - t0 > (unsigned long long)ctl->timeout_ns + 100000000ull) {
-          m = -1;  // the poller's own limit passed long ago (it records the status)
+        if (globaltimer() - t0 > (unsigned long long)ctl->timeout_ns) {
+          set_status(ctl, MPCG_ERR_TIMEOUT);
+          m = -1;
           break;
         }
       }
     }
     __threadfence();
-    if (kBlk && poller) *s_mode = m;
   }
   m = __shfl_sync(0xffffffffu, m, 0);
   __syncwarp();
@@ -726,37 +710,44 @@ __device__ bool bfs_dual(const BfsGraph& g, int32_t* dA, int32_t* dB, int srcA, 
       // ---- narrow frontiers: one warp runs the next levels alone ----
       int* nmem;
       if constexpr (std::is_same<Sync, BlockGroupSync>::value) {
-        nmem = sync.scratch();
+        nmem = sync.mem;
       } else {
         __shared__ int s_narrow[kNarrowScratch];
         nmem = s_narrow;
       }
       int (*const nbuf)[kNarrowItems] = reinterpret_cast<int (*)[kNarrowItems]>(nmem);
       int* const nhash = nmem + 4 * kNarrowItems;
-      volatile int* const nmode = nmem + 4 * kNarrowItems + kNarrowHash;  // whole-block groups
-      if constexpr (Sync::kWholeBlock) {
-        if (threadIdx.x == 0) *nmode = 0;
-        __syncthreads();  // every thread of the block is here (same level, same decision)
-      }
-      int resume;
+      int* const nmode = nmem + 4 * kNarrowItems + kNarrowHash;  // whole-block groups
+      // (whole-block groups: every thread of the block is here, with the same
+      // level and decision, and has read the word of an earlier turn)
+      if constexpr (Sync::kWholeBlock) __syncthreads();
+      int m = 0;
       if (tid < 32) {
-        resume = narrow_levels(g, dA, dB, level, sa, sb, la, lb, reached, nbuf, nbuf + 2, nhash);
+        const int resume = narrow_levels(g, dA, dB, level, sa, sb, la, lb, reached, nbuf, nbuf + 2, nhash);
+        m = resume < 0 ? kNmDone : ((resume << 2) | kNmResume);
         if (lane == 0) {
           ctl->nla = la;
           ctl->nlb = lb;
           ctl->nreached = reached;
           __threadfence();
-          atomicExch(&ctl->nmode, resume < 0 ? kNmDone : ((resume << 2) | kNmResume));
+          atomicExch(&ctl->nmode, m);
         }
         __syncwarp();
-      } else {
-        const int m = nm_wait<Sync::kWholeBlock>(ctl, level, nmode, sync.first());
-        if (m == -1) return false;
+      } else if (!Sync::kWholeBlock || threadIdx.x < 32) {
+        m = nm_wait(ctl, level);
+      }
+      if constexpr (Sync::kWholeBlock) {
+        if (threadIdx.x == 0) *nmode = m;
+        __syncthreads();
+        m = *nmode;
+      }
+      if (m == -1) return false;
+      if (tid >= 32) {
         la = *reinterpret_cast<volatile int*>(&ctl->nla);
         lb = *reinterpret_cast<volatile int*>(&ctl->nlb);
         reached = *reinterpret_cast<volatile long long*>(&ctl->nreached);
-        resume = (m & 3) == kNmDone ? -1 : (m >> 2);
       }
+      const int resume = (m & 3) == kNmDone ? -1 : (m >> 2);
       if (resume < 0) break;
       // resume: the loop's head reads the level's sizes from the counters
       // and adds them to the state (the published state stops before it);

@@ -75,7 +75,7 @@ static __device__ bool feature_pdiam(const BlockGraph& g, const BfsGraph& q, int
                                      unsigned char* smem, int smem_bytes, int slot, int first, int blocks) {
   const int rank = (int)blockIdx.x - first;
   if (rank == 0 && g.n <= kPdMaxN) block_pdiam(g, q, smem, smem_bytes);
-  BlockGroupSync sync{q.ctl, slot, 0ull, first, blocks, reinterpret_cast<int*>(smem)};
+  BlockGroupSync sync{q.ctl, slot, 0ull, blocks, reinterpret_cast<int*>(smem)};
   if (!sync()) return false;
   if (*reinterpret_cast<volatile int*>(&q.ctl->pd_done)) return true;
   return pseudo_diameter_run<BlockGroupSync, false>(q, d1, d2, rank * (int)blockDim.x + (int)threadIdx.x,

@@ -29,6 +29,17 @@ def _two(A, B):
                      np.concatenate([A.val, B.val]))
 
 
+def _lollipop(path, nx, ny):
+    """A path into the corner of a grid and another path out of the opposite one."""
+    a = np.arange(path - 1)
+    g = np.arange(nx * ny).reshape(ny, nx) + path
+    n = 2 * path + nx * ny
+    i = np.concatenate([a, [path - 1], g[:, :-1].ravel(), g[:-1].ravel(), [g[-1, -1]], a + path + nx * ny])
+    j = np.concatenate([a + 1, [g[0, 0]], g[:, 1:].ravel(), g[1:].ravel(), [path + nx * ny], a + path + nx * ny + 1])
+    deg = np.bincount(i, minlength=n) + np.bincount(j, minlength=n)
+    return synth.from_edges(n, i, j, -np.ones(i.size), deg + 0.1)
+
+
 CASES = {
     "one": lambda: synth.laplacian_2d(1, 1),
     "path_3000": lambda: synth.path(3000),
@@ -47,6 +58,10 @@ CASES = {
     "lone_first": lambda: _two(synth.laplacian_2d(1, 1), synth.laplacian_2d(30, 700)),  # vertex 0 by itself
     "lone_last": lambda: _two(synth.laplacian_2d(30, 700), synth.laplacian_2d(1, 1)),
     "forest": lambda: synth.banded(30000, 3, 0.9, 1.1, seed=3),
+    # past the largest size, where the blocks search together: levels of one warp, also handed
+    # back to the blocks for a wide middle part, and again to the warp
+    "thin_20100x15": lambda: synth.laplacian_2d(20100, 15),
+    "lollipop": lambda: _lollipop(2000, 600, 500),
     "no_edges": lambda: synth.banded(20000, 3, 0.0, 1.1, seed=3),
 }
 
