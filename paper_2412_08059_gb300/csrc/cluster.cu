@@ -253,11 +253,54 @@ __device__ __forceinline__ uint16_t cl_pack(int nslices, int c) {
   return (uint16_t)((o << 12) | (c - kSlice * cl_first(nslices, o)));
 }
 
+// acc + the sum over the entries [f, f1) of one row in the caller's CSR, in
+// stored order, by the whole warp (acc alike in every lane): each lane loads
+// and gathers one of 32 entries, the next 32 on their way, and the chain of
+// fused multiply-adds runs in every lane, so that an entry costs about its
+// dependent FMA.  Stars, FP64, an iteration: 12,000 rows 0.69 ms, 2.57 by one
+// lane an entry at a time and 1.08 by the grid-wide kernels; 4,000 rows 0.22,
+// 0.42 and 0.37.  (Many long rows in one slice stay with their lanes: sixteen
+// hubs of 20,000 rows 0.37 ms, 0.27 by the grid.)
+template <typename T>
+__device__ __noinline__ T cl_warp_tail(const ClusterArgs& a, bool rep, uint32_t gb, int f, int f1, T acc) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const uint32_t self = cl_rank() << 12;
+  int c = 0;  // (a lane without an entry gathers a row that exists and is not used)
+  T v = (T)0;
+  if (f + lane < f1) {
+    c = a.col[f + lane];
+    v = (T)a.val[f + lane];
+  }
+  for (; f < f1; f += 32) {  // warp-uniform
+    const uint32_t p = rep ? self | (uint32_t)c : (uint32_t)cl_pack(a.nslices, c);
+    const T w = v;
+    T x;
+    cl_ld(cl_map(gb, p >> 12) + (p & 4095u) * (uint32_t)sizeof(T), x);
+    if (f + 32 + lane < f1) {
+      c = a.col[f + 32 + lane];
+      v = (T)a.val[f + 32 + lane];
+    }
+    const int m = min(32, f1 - f);
+    if (m == 32) {
+#pragma unroll
+      for (int k = 0; k < 32; ++k) acc = fma(__shfl_sync(full, w, k), __shfl_sync(full, x, k), acc);
+    } else {
+      for (int k = 0; k < m; ++k) acc = fma(__shfl_sync(full, w, k), __shfl_sync(full, x, k), acc);
+    }
+  }
+  return acc;
+}
+
 // Columns once (`cols`), values at the start of each stage.  The entries of a
 // row past the layout's width cap go behind the slices' where there is room
 // (tail[j]: first entry | number << 16; 0: none, or read from the CSR).  Read
 // from the caller's CSR at every pass, with a division for the owner of each,
 // they made a random tree's SpMV three times as long as its other rows need.
+// Where one or two rows of a slice have many (the hub of a star), the warp sums
+// each together (kClTailWarp, whose number reads as 0).
+constexpr uint32_t kClTailWarp = 0x80000000u;
+constexpr int kClLongTail = 64;
 template <typename T, int RPT>
 __device__ __forceinline__ void cl_load(const ClusterArgs& a, ClShared& S, const ClMat& M, int S0,
                                         int rank, int ns, const T* sv, bool cols, uint32_t (&tail)[RPT]) {
@@ -286,13 +329,22 @@ __device__ __forceinline__ void cl_load(const ClusterArgs& a, ClShared& S, const
         M.c[e - E0] = M.rep ? (uint16_t)((rank << 12) | c) : cl_pack(a.nslices, c);
       }
     }
-    if ((wf & kOverflowBit) && i < a.n) {
-      const int e0 = a.rp[i] + w, cnt = a.rp[i + 1] - e0;
-      if (cols && cnt > 0 && cnt < (1 << 15)) {
+    if (wf & kOverflowBit) {  // warp-uniform
+      int e0 = 0, cnt = 0;
+      if (i < a.n) {
+        e0 = a.rp[i] + w;
+        cnt = a.rp[i + 1] - e0;
+      }
+      if (cols) {
+        // (rows in turn against all lanes at once: even at two rows or more)
+        const unsigned lng = __ballot_sync(0xffffffffu, cnt > kClLongTail);
+        if (cnt > kClLongTail && __popc(lng) <= 2) tail[j] = kClTailWarp;
+      }
+      if (cols && tail[j] == 0u && cnt > 0 && cnt < (1 << 15)) {
         const int at = E + atomicAdd(&S.tail, cnt);
         if (at + cnt <= a.ent_cap && at < (1 << 16)) tail[j] = (uint32_t)at | ((uint32_t)cnt << 16);
       }
-      const int at = (int)(tail[j] & 0xffffu), m = (int)(tail[j] >> 16);
+      const int at = (int)(tail[j] & 0xffffu), m = (int)(tail[j] >> 16) & 0x7fff;
       for (int k = 0; k < m; ++k) {
         vd[at + k] = (T)a.val[e0 + k];
         if (cols) {
@@ -303,6 +355,14 @@ __device__ __forceinline__ void cl_load(const ClusterArgs& a, ClShared& S, const
     }
   }
   __syncthreads();
+}
+
+template <int RPT>
+__device__ __forceinline__ bool cl_longs(const uint32_t (&tail)[RPT]) {
+  uint32_t t = 0u;
+#pragma unroll
+  for (int j = 0; j < RPT; ++j) t |= tail[j];
+  return __any_sync(0xffffffffu, (t & kClTailWarp) != 0u);
 }
 
 // acc + the sum over K entries of a row, from shared memory: all columns, then
@@ -323,9 +383,10 @@ __device__ __forceinline__ T cl_entries(uint32_t gb, const uint16_t* cp, const T
 
 // Row sums of the block's slices: q[j] = sum_k v_k g(c_k) of row
 // 32 (warp + 16 j) + lane, in stored order (0 where the thread has no row).
+// longs (warp-uniform): some tail[j] is kClTailWarp.
 template <typename T, int RPT>
 __device__ __forceinline__ void cl_spmv(const ClusterArgs& a, const ClShared& S, const ClMat& M, int S0,
-                                        int ns, const uint32_t (&tail)[RPT], T (&q)[RPT]) {
+                                        int ns, const uint32_t (&tail)[RPT], bool longs, T (&q)[RPT]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t gb = smem_addr(M.g);
 #pragma unroll
@@ -359,7 +420,7 @@ __device__ __forceinline__ void cl_spmv(const ClusterArgs& a, const ClShared& S,
       }
       const int i = (S0 + s) * kSlice + lane;
       if (wf & kOverflowBit) {
-        const int m = (int)(tail[j] >> 16);
+        const int m = (int)(tail[j] >> 16) & 0x7fff;
         const uint16_t* tc = M.c + (tail[j] & 0xffffu);
         const T* tv = reinterpret_cast<const T*>(M.v) + (tail[j] & 0xffffu);
         int e = 0;
@@ -379,7 +440,7 @@ __device__ __forceinline__ void cl_spmv(const ClusterArgs& a, const ClShared& S,
           cl_ld(cl_map(gb, c >> 12) + (c & 4095u) * (uint32_t)sizeof(T), x);
           acc = fma(tv[e], x, acc);
         }
-        if (m == 0 && i < a.n) {  // no room: from the caller's CSR
+        if (tail[j] == 0u && i < a.n) {  // no room: from the caller's CSR
           const int e1 = a.rp[i + 1];
           for (int f = a.rp[i] + w; f < e1; ++f) {
             const uint32_t c = M.rep ? (uint32_t)a.col[f] : cl_pack(a.nslices, a.col[f]);
@@ -392,6 +453,20 @@ __device__ __forceinline__ void cl_spmv(const ClusterArgs& a, const ClShared& S,
       if (i >= a.n) acc = (T)0;
     }
     q[j] = acc;
+  }
+  // (in a pass of their own, which keeps the calls out of the loop above)
+  if (longs) {
+#pragma unroll
+    for (int j = 0; j < RPT; ++j) {
+      unsigned rows = __ballot_sync(0xffffffffu, tail[j] == kClTailWarp);
+      while (rows) {  // warp-uniform
+        const int s = warp + kClWarps * j, src = __ffs(rows) - 1, r = (S0 + s) * kSlice + src;
+        rows &= rows - 1;
+        const int w = (int)((uint32_t)S.tab[s].y & ~kOverflowBit);
+        const T t = cl_warp_tail<T>(a, M.rep, gb, a.rp[r] + w, a.rp[r + 1], __shfl_sync(0xffffffffu, q[j], src));
+        if (lane == src) q[j] = t;
+      }
+    }
   }
 }
 
@@ -510,6 +585,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
   // =================== single-precision stage ===================
   if (a.mode != 2) {
     cl_load<float, RPT>(a, S, M, S0, rank, ns, a.sv32, true, tail);
+    const bool longs = cl_longs<RPT>(tail);
     const float* g = reinterpret_cast<const float*>(M.g) + M.base;
     const bool autom = a.mode == 1;
     const int max1 = ctl->max1, k0 = ctl->k0;
@@ -667,7 +743,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
         cw = cancel_word(ctl);
         if (autom && cls < 0) label_now = *reinterpret_cast<volatile int*>(&ctl->eps1_ready);
       }
-      cl_spmv<float, RPT>(a, S, M, S0, ns, tail, q);
+      cl_spmv<float, RPT>(a, S, M, S0, ns, tail, longs, q);
       FF pdq{0.f, 0.f};
       float d[RPT];
 #pragma unroll
@@ -816,6 +892,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
 
   // =================== double-precision stage ===================
   cl_load<double, RPT>(a, S, M, S0, rank, ns, a.sv64, a.mode == 2, tail);
+  const bool longs = cl_longs<RPT>(tail);
   const double* g = reinterpret_cast<const double*>(M.g) + M.base;
   const double bnorm = ctl->bnorm64, eps2 = ctl->eps2;
   const int max2 = ctl->max2, max_restarts = ctl->max_restarts;
@@ -831,7 +908,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
     for (int j = 0; j < RPT; ++j)
       if (warp + kClWarps * j < ns) cl_put(M, (warp + kClWarps * j) * kSlice + lane, xd[j]);
     cl_sync();
-    cl_spmv<double, RPT>(a, S, M, S0, ns, tail, q);
+    cl_spmv<double, RPT>(a, S, M, S0, ns, tail, longs, q);
     double p = 0.0;
 #pragma unroll
     for (int j = 0; j < RPT; ++j) {
@@ -893,7 +970,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_cluster(ClusterArgs a) {
     while (dec == kClGo) {
       if (lead0) cw = cancel_word(ctl);  // used with the r^T r sum
       // ---- q = A d, d^T q ----
-      cl_spmv<double, RPT>(a, S, M, S0, ns, tail, q);
+      cl_spmv<double, RPT>(a, S, M, S0, ns, tail, longs, q);
       // (A predicated-off FP64 instruction takes its turn of the FP64 pipe:
       // warps without a slice branch around these.  The __syncwarp keeps the
       // compiler from predicating the short bodies.)

@@ -40,10 +40,34 @@ def _two(n):
                      np.concatenate([A.val, B.val]))
 
 
+def _hubs(n, hubs, far=0):
+    """Every vertex joined to one of the first `hubs` vertices, which form a chain; vertices past
+    the hubs also to `far` others."""
+    i = np.arange(hubs, n)
+    c = np.arange(hubs - 1)
+    a = [np.stack([i % hubs, i]), np.stack([c, c + 1])]
+    for k in range(far):
+        j = i + 37 * (k + 1)
+        a.append(np.stack([i[j < n], j[j < n]]))
+    e = np.unique(np.concatenate(a, 1), axis=1)
+    deg = np.bincount(e[0], minlength=n) + np.bincount(e[1], minlength=n)
+    off = -0.5 - np.random.default_rng(n).random(e.shape[1])
+    return synth.from_edges(n, e[0], e[1], off, 2.0 * deg + 1.0)
+
+
 CASES = {f"grid{n}": (lambda n=n: _grid(n)) for n in
          (1, 31, 33, 480, 512, 513, 8192, 8224, 16384, 16400, 32768, 39990, 40200)}
 CASES.update({
     "star_1001": lambda: synth.star(1001, 1.1),          # one row past the width cap
+    # long rows: one or two of a slice (summed by the warp), more (by their lanes, behind the
+    # slices' entries or, without room there, from the CSR), and more entries than a count holds
+    "star_12000": lambda: synth.star(12000, 3.0),
+    "star_40000": lambda: synth.star(40000, 3.0),
+    "hubs_2_4000": lambda: _hubs(4000, 2),
+    "hubs_5_4000": lambda: _hubs(4000, 5, 1),
+    "hubs_16_9000": lambda: _hubs(9000, 16),
+    "hubs_70_9000": lambda: _hubs(9000, 70, 2),
+    "hubs_400_30000": lambda: _hubs(30000, 400),
     "rtree_5000": lambda: synth.random_tree_plus(5000, 0.5, 1.1, seed=3),
     # whole copies of the gathered vector up to 4,096 rows, where columns are far away
     "rreg_300": lambda: synth.random_regular_laplacian(300, 6, 1e-2, seed=4),
